@@ -28,7 +28,7 @@ struct auv_env {
   Status* status;
   float* w_policy_f32;      // fp32 mode: row-major weights as given
   float* w_value_f32;
-  void* w_policy_packed;    // bf16 mode: packed operand images
+  void* w_policy_packed;    // packed images (bf16 and tf32 operands, fp32 slices)
   void* w_value_packed;
   float* staging;           // fp32 copy of the caller's weights (bf16 mode)
   size_t policy_count, value_count;
@@ -403,6 +403,12 @@ int env_create(const auv_config* cfg, const auv_buffers* buf, auv_env** out) {
   } else if (cfg->mlp_mode == AUV_MLP_TF32) {
     pol_pk_off = off;
     off += ((auv::tf32_policy_image_bytes() + 1023) / 1024) * 1024;
+  } else {
+    const size_t b = auv::fp32_image_bytes(obs_dim(cfg), cfg->hidden);
+    pol_pk_off = off;
+    off += ((b + 1023) / 1024) * 1024;
+    val_pk_off = off;
+    if (cfg->has_value) off += ((b + 1023) / 1024) * 1024;
   }
   cudaError_t e = cudaMalloc(&env->workspace, off);
   if (e != cudaSuccess) {
@@ -417,6 +423,9 @@ int env_create(const auv_config* cfg, const auv_buffers* buf, auv_env** out) {
     env->w_value_packed = env->workspace + val_pk_off;
   } else if (cfg->mlp_mode == AUV_MLP_TF32) {
     env->w_policy_packed = env->workspace + pol_pk_off;
+  } else {
+    env->w_policy_packed = env->workspace + pol_pk_off;
+    env->w_value_packed = cfg->has_value ? env->workspace + val_pk_off : nullptr;
   }
   Status s0 = {0, 0, INT_MAX, 0};
   e = cudaMemcpy(env->status, &s0, sizeof(s0), cudaMemcpyHostToDevice);
@@ -468,6 +477,11 @@ int env_set_weights(auv_env* env, const float* policy, const float* value, void*
   } else if (env->cfg.mlp_mode == AUV_MLP_TF32) {
     e = auv::launch_pack_tf32(env->model, env->w_policy_f32, env->w_policy_packed, s);
     if (e != cudaSuccess) return cuda_fail(env, e, "pack tf32 weights");
+  } else {
+    e = auv::launch_pack_fp32(env->model, env->w_policy_f32, env->w_policy_packed, s);
+    if (e == cudaSuccess && value)
+      e = auv::launch_pack_fp32(env->model, env->w_value_f32, env->w_value_packed, s);
+    if (e != cudaSuccess) return cuda_fail(env, e, "pack fp32 weights");
   }
   // host sources are read before return
   void* d = nullptr;
@@ -492,16 +506,16 @@ int env_reset(auv_env* env, const uint8_t* mask, void* stream) {
 
 namespace {
 
+auv::Fp32Nets fp32_nets(const auv_env* env) {
+  return {env->w_policy_f32, env->w_value_f32, env->w_policy_packed, env->w_value_packed};
+}
+
 // The kernels of T control steps from global step t_g0 (bf16 mode: the fused
 // rollout, then the value network over the observations just written).
 cudaError_t launch_rollout_any(auv_env* env, const Traj& tr, int T, uint64_t t_g0,
                                cudaStream_t s) {
   if (env->cfg.mlp_mode == AUV_MLP_FP32)
-    return is_paper(&env->cfg)
-               ? auv::launch_paper_rollout_fp32(env->model, env->buf, env->w_policy_f32,
-                                                env->w_value_f32, tr, T, t_g0, env->status, s)
-               : auv::launch_rollout_fp32(env->model, env->buf, env->w_policy_f32,
-                                          env->w_value_f32, tr, T, t_g0, env->status, s);
+    return auv::launch_rollout_fp32(env->model, env->buf, fp32_nets(env), tr, T, t_g0, env->status, s);
   if (env->cfg.mlp_mode == AUV_MLP_TF32)
     return auv::launch_rollout_tf32(env->model, env->buf, env->w_policy_packed, tr, T, t_g0,
                                     env->status, s);
@@ -661,8 +675,8 @@ int env_value(auv_env* env, const float* obs, int T, float* value, void* stream)
   if (env->cfg.mlp_mode == AUV_MLP_TF32)
     return fail(env, AUV_ERR_UNSUPPORTED, "tf32 mode has no value network");
   if (env->cfg.mlp_mode == AUV_MLP_FP32)
-    e = auv::launch_value_fp32(env->model, env->w_value_f32, static_cast<const float*>(o), rows,
-                               env->model.n, static_cast<float*>(v), s);
+    e = auv::launch_rows_fp32(env->model, fp32_nets(env), static_cast<const float*>(o), rows,
+                              env->model.n, nullptr, static_cast<float*>(v), env->status, s);
   else
     e = auv::launch_value_bf16(env->model, env->w_value_packed, env->w_value_f32,
                                static_cast<const float*>(o), rows, env->model.n,
@@ -877,8 +891,8 @@ int env_policy_forward(auv_env* env, const float* obs, int n, float* head, float
   if (env->cfg.mlp_mode == AUV_MLP_TF32)
     return fail(env, AUV_ERR_UNSUPPORTED, "tf32 mode evaluates the policy inside env_rollout only");
   if (env->cfg.mlp_mode == AUV_MLP_FP32)
-    e = auv::launch_forward_fp32(env->model, env->w_policy_f32, env->w_value_f32, obs, n, head,
-                                 value, s);
+    e = auv::launch_rows_fp32(env->model, fp32_nets(env), obs, (size_t)n, 1, head, value, env->status,
+                              s);
   else
     e = auv::launch_forward_bf16(env->model, env->w_policy_packed, env->w_value_packed,
                                  env->w_value_f32, obs, n, head, value, env->status, s);

@@ -34,15 +34,21 @@ cudaError_t launch_replay(const Model& M, const Buffers& B, const float* act, in
 cudaError_t launch_observe(const Model& M, const Buffers& B, float* obs, cudaStream_t s);
 cudaError_t launch_draw_words(const Model& M, uint32_t stream_id, uint64_t index, int n_blocks,
                               uint32_t* out, cudaStream_t s);
-cudaError_t launch_rollout_fp32(const Model& M, const Buffers& B, const float* wp,
-                                const float* wv, const Traj& tr, int T, uint64_t t_g0, Status* st,
-                                cudaStream_t s);
-// Value network over stored observations obs[t][obs_dim][n] (row r = t*n + i).
-cudaError_t launch_value_fp32(const Model& M, const float* wv, const float* obs, size_t rows,
-                              int n, float* value, cudaStream_t s);
-cudaError_t launch_forward_fp32(const Model& M, const float* wp, const float* wv,
-                                const float* obs, int n, float* head, float* value,
-                                cudaStream_t s);
+// The exact-fp32 networks of both models (k_fp32.cu): the networks' flat
+// weights and their packed images (launch_pack_fp32; 16-byte aligned).
+struct Fp32Nets {
+  const float *policy, *value;
+  const void *policy_img, *value_img;
+};
+size_t fp32_image_bytes(int in_dim, int hidden);
+cudaError_t launch_pack_fp32(const Model& M, const float* w, void* img, cudaStream_t s);
+cudaError_t launch_rollout_fp32(const Model& M, const Buffers& B, const Fp32Nets& w, const Traj& tr,
+                                int T, uint64_t t_g0, Status* st, cudaStream_t s);
+// Networks over rows: input k of row r at obs[((r / ns) * obs_dim + k) * ns +
+// r % ns] (ns = 1: row-major; ns = n: a trajectory's observations), head
+// [rows][policy_out] and value [rows] as given (either may be NULL).
+cudaError_t launch_rows_fp32(const Model& M, const Fp32Nets& w, const float* obs, size_t rows, int ns,
+                             float* head, float* value, Status* st, cudaStream_t s);
 
 // The paper model's CUDA-core kernels (k_paper.cu)
 cudaError_t launch_paper_reset(const Model& M, const Buffers& B, const uint8_t* mask,
@@ -51,9 +57,6 @@ cudaError_t launch_paper_replay(const Model& M, const Buffers& B, const float* a
                                 float* rew, uint8_t* done, float* trace, Status* st,
                                 cudaStream_t s);
 cudaError_t launch_paper_observe(const Model& M, const Buffers& B, float* obs, cudaStream_t s);
-cudaError_t launch_paper_rollout_fp32(const Model& M, const Buffers& B, const float* wp,
-                                      const float* wv, const Traj& tr, int T, uint64_t t_g0,
-                                      Status* st, cudaStream_t s);
 
 // Reverse-mode adjoint of the Fossen control step over an action window
 // (k_adjoint.cu).  scratch: adjoint_scratch_floats(n, T) floats.  T <= 64,
