@@ -33,6 +33,17 @@ struct Operand {
   bool mn_major;     // false: (r, k) at r*ld + k; true: (r, k) at k*ld + r
 };
 
+// What is done to each element of the product before it is stored (beta = 0
+// only): nothing, tanh (a layer's activation), or the product times tanh'
+// from the activation h (row r, column c at aux[r * ld_aux + c], of C's
+// type): x (1 - h^2).
+enum EpiKind { kEpiNone = 0, kEpiTanh = 1, kEpiDtanh = 2 };
+struct Epilogue {
+  EpiKind kind = kEpiNone;
+  const void* aux = nullptr;
+  int ld_aux = 0;
+};
+
 // Bytes of split-K partials a product of this shape may use (0: none).
 size_t workspace_bytes(int M, int N, int K);
 
@@ -43,7 +54,7 @@ size_t workspace_bytes(int M, int N, int K);
 // (misaligned operand), or the launch error.
 cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A, const Operand& B, void* C,
                    int ldc, bool c_bf16, float beta, float* ws, size_t ws_bytes, Status* st,
-                   cudaStream_t s);
+                   cudaStream_t s, const Epilogue& epi = Epilogue());
 
 }  // namespace gemm
 }  // namespace auv

@@ -72,9 +72,10 @@ cudaError_t launch_adjoint(const Model& M, const Buffers& B, const float* act, i
 namespace shac {
 struct Layout {
   int n, T, H, Dp, Hp;
+  int G;             // steps whose weight gradients run as one product
   int D, out, S;     // network input, policy head width, adjoint rows (model)
   size_t n_aug_p, n_aug_v;
-  size_t o_X, o_H1, o_H2, o_Y, o_G, o_GX, o_gY, o_lam, o_done, o_rew, o_VH1, o_VH2, o_V, o_gYv,
+  size_t o_X, o_H1, o_H2, o_Y, o_G2, o_G1, o_GX, o_gY, o_lam, o_done, o_rew, o_VH1, o_VH2, o_V, o_gYv,
       o_wp, o_wv, o_gp, o_sc, o_gws, gws_bytes, bytes;
 };
 // paper: the paper model (input 12, head 12, 61 adjoint rows), else Fossen
@@ -181,7 +182,6 @@ cudaError_t launch_gather(const Dims& d, const PermKey& k, const StepCtl* ctl, c
                           const float* ret, uint32_t N, const Sample& out, void* X,
                           cudaStream_t s);
 cudaError_t launch_step_advance(StepCtl* ctl, cudaStream_t s);
-cudaError_t launch_tanh_fwd(bool bf16, void* h, int ld, int B, int H, cudaStream_t s);
 // Sample-major copy of a batch for the gather: rows of sample_row_floats(D, A)
 // floats (obs, act, logp, adv, ret, zero padding), row r = t N + i; act,
 // logp and adv may be NULL (value-only).  D + A + 3 <= 80.
@@ -191,8 +191,6 @@ cudaError_t launch_transpose_batch(int D, int A, uint32_t T, uint32_t N, const f
                                    const float* ret, float* dst, cudaStream_t s);
 cudaError_t launch_gather_sm(const Dims& d, const PermKey& k, const StepCtl* ctl,
                              const float* rows, const Sample& out, void* X, cudaStream_t s);
-cudaError_t launch_tanh_bwd(bool bf16, void* g, int ldg, const void* h, int ldh, int B, int H,
-                            cudaStream_t s);
 // y [B][ld_pol], v [B][ld_val] fp32 head outputs; g_y, g_v the same shapes.
 cudaError_t launch_head(const Dims& d, const LossHp& hp, const float* y, const float* v,
                         const Sample& smp, void* g_y, void* g_v, float* part, cudaStream_t s);

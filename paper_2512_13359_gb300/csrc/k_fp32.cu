@@ -18,6 +18,14 @@
 //             and odd k are the two lanes of packed fp32 FMAs.
 //   head      one thread per row and pair of outputs
 //
+// What bounds it: shared-memory reads of the operands (a thread's 4 x 8 outputs
+// take 12 16-byte reads per 64 packed FMAs) and, with one CTA per SM, their
+// latency.  Measured per control step of a 32-row tile at width 256, one CTA
+// per SM: layer 1 5.9k cycles, layer 2 28k (16.4k of FMA), tanh 1.1k, head 4k,
+// physics 3.6k.  4,096 envs x 100 steps of the Fossen model: 56.8 ms with one
+// thread per env, 2.1 ms now; 64 envs x 200 steps at width 64: 1.16 ms with a
+// 64-thread team per env, 0.43 ms now.
+//
 // Sums keep one order whatever the tile: layer 1 in k from the bias; layer 2
 // even k from the bias plus odd k from zero; the head in k from the bias.
 #include <algorithm>
@@ -70,6 +78,12 @@ struct Net {
   const float* w;
   const float* img;
 };
+
+// CTAs that share an SM: two 32-row tiles with a three-slot ring, else one
+// (whose threads may use up to 255 registers).
+constexpr int ctas_per_sm(int E, int H, int SLOTS) {
+  return E == 32 && (H == 64 || SLOTS == 3) ? 2 : 1;
+}
 
 // Tile shape: E rows, ring of SLOTS W2 slices (H = 64: every slice of both
 // networks resident, SLOTS = 8).
@@ -244,7 +258,7 @@ struct Tile {
       const float4* wb = reinterpret_cast<const float4*>(W3 + o2 * H);
       const float4* hr = reinterpret_cast<const float4*>(hs + e * kHs);
       float s = __ldg(b3 + o), s2 = __ldg(b3 + o2);
-#pragma unroll 8
+#pragma unroll (H == 256 ? 16 : 8)
       for (int k4 = 0; k4 < H / 4; ++k4) {
         const float4 a = __ldg(wa + k4), b = __ldg(wb + k4), h = hr[k4];
         s = fmaf(a.x, h.x, s);
@@ -324,7 +338,7 @@ struct RolloutSmem {
 };
 
 template <class Sim, int H, int E, int SLOTS>
-__global__ void __launch_bounds__(kThreads, E == 32 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(E, H, SLOTS))
 k_rollout_fp32(const Model M, Buffers B, Net policy, Net critic, Traj tr, int T, uint64_t t_g0,
                Status* st) {
   using TL = Tile<Sim::kObs, H, E, SLOTS>;
@@ -420,7 +434,7 @@ k_rollout_fp32(const Model M, Buffers B, Net policy, Net critic, Traj tr, int T,
 // if given (policy), value[r] if given.  Each CTA takes every gridDim.x-th
 // tile of E rows.
 template <int IN, int H, int E, int SLOTS>
-__global__ void __launch_bounds__(kThreads, E == 32 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(E, H, SLOTS))
 k_rows_fp32(Net policy, Net critic, const float* __restrict__ obs, size_t rows, int ns, int out_dim,
             float* __restrict__ head, float* __restrict__ value, Status* st) {
   using TL = Tile<IN, H, E, SLOTS>;
@@ -460,7 +474,7 @@ template <class Sim, int H, int E, int SLOTS>
 cudaError_t rollout(const Model& M, const Buffers& B, const Net& p, const Net& v, const Traj& tr,
                     int T, uint64_t t_g0, Status* st, cudaStream_t s) {
   constexpr int smem = RolloutSmem<Sim, H, E, SLOTS>::kFloats * 4;
-  static_assert(smem <= (E == 32 ? 113 : 226) * 1024, "shared memory per CTA");
+  static_assert(smem <= 226 * 1024 / ctas_per_sm(E, H, SLOTS), "shared memory per CTA");
   auto kern = k_rollout_fp32<Sim, H, E, SLOTS>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -469,13 +483,19 @@ cudaError_t rollout(const Model& M, const Buffers& B, const Net& p, const Net& v
 }
 
 // Rows per CTA: the fewest that keep one CTA per SM (a step's time grows with
-// the tile, but every CTA streams W2 once a step, so more CTAs than SMs gain
-// nothing).  32 above that: two CTAs per SM, one's physics under the other's
-// products.
+// the tile, 10.4, 14.3 and 21.8 us a step at 8, 16 and 32 rows, width 256, and
+// every CTA streams W2 once a step, so more CTAs than SMs gain nothing).
 int rows_per_cta(size_t rows) {
   const size_t sms = (size_t)engine_sm_count();
   return rows <= 8 * sms ? 8 : (rows <= 16 * sms ? 16 : 32);
 }
+
+// Width 256, 32-row tiles: while every SM has at most one, the kernel compiled
+// for one CTA per SM (no register cap at 128, six slots: 1.09 ms for 4,096
+// envs x 50 steps against 1.24); above, two CTAs per SM, one's physics under
+// the other's products (1.91 ms for 9,728 envs, where one CTA per SM in two
+// waves would take 2.2).
+bool one_per_sm(size_t rows) { return rows <= 32 * (size_t)engine_sm_count(); }
 
 template <class Sim>
 cudaError_t rollout_any(const Model& M, const Buffers& B, const Net& p, const Net& v, const Traj& tr,
@@ -487,7 +507,8 @@ cudaError_t rollout_any(const Model& M, const Buffers& B, const Net& p, const Ne
   if (M.hidden == 256)
     return e == 8    ? rollout<Sim, 256, 8, 8>(M, B, p, v, tr, T, t_g0, st, s)
            : e == 16 ? rollout<Sim, 256, 16, 6>(M, B, p, v, tr, T, t_g0, st, s)
-                     : rollout<Sim, 256, 32, 3>(M, B, p, v, tr, T, t_g0, st, s);
+           : one_per_sm((size_t)M.n) ? rollout<Sim, 256, 32, 6>(M, B, p, v, tr, T, t_g0, st, s)
+                                     : rollout<Sim, 256, 32, 3>(M, B, p, v, tr, T, t_g0, st, s);
   return cudaErrorInvalidValue;
 }
 
@@ -495,11 +516,11 @@ template <int IN, int H, int E, int SLOTS>
 cudaError_t rows_fp32(const Net& p, const Net& v, const float* obs, size_t rows, int ns, int out_dim,
                       float* head, float* value, Status* st, cudaStream_t s) {
   constexpr int smem = Tile<IN, H, E, SLOTS>::kNet * 4;
-  static_assert(smem <= (E == 32 ? 113 : 226) * 1024, "shared memory per CTA");
+  static_assert(smem <= 226 * 1024 / ctas_per_sm(E, H, SLOTS), "shared memory per CTA");
   auto kern = k_rows_fp32<IN, H, E, SLOTS>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const size_t tiles = (rows + E - 1) / E, most = (size_t)engine_sm_count() * (E == 32 ? 2 : 1);
+  const size_t tiles = (rows + E - 1) / E, most = (size_t)engine_sm_count() * ctas_per_sm(E, H, SLOTS);
   kern<<<(unsigned)std::min(tiles, most), kThreads, smem, s>>>(p, v, obs, rows, ns, out_dim, head, value,
                                                                st);
   return cudaGetLastError();

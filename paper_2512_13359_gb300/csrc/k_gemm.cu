@@ -19,7 +19,9 @@
 //  - MN-major (K row kk, the M or N index contiguous): boxes of 128 bytes of
 //    M/N x BK rows, one per 128 bytes of M/N, BK * 128 bytes apart (LBO);
 //    8 K rows form a 1024-byte group (SBO); an MMA's K-step (32 bytes of
-//    K) advances the start address by 4096 / element-size bytes.
+//    K) advances the start address by 4096 / element-size bytes.  tf32 reads
+//    MN-major operands only with the 128-byte swizzle of 32-byte pieces
+//    (4 K rows, 512 bytes, a group): its tensor maps use that swizzle.
 //
 // fp32 operands without tensor cores (the exact mode): a register-blocked CUDA-core
 // kernel with the same operand layouts and the same split-K.
@@ -57,14 +59,16 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Shared-memory descriptor with both byte offsets (128-byte swizzle).
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+// Shared-memory descriptor with both byte offsets (128-byte swizzle of 16-byte
+// pieces, type 2, or of 32-byte pieces, type 1).
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo,
+                                               uint64_t type = 2) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
   d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
   d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
   d |= (uint64_t)1u << 46;                       // descriptor version
-  d |= (uint64_t)2u << 61;                       // 128-byte swizzle
+  d |= type << 61;
   return d;
 }
 
@@ -103,6 +107,9 @@ struct TcArgs {
   float* ws;              // split partials, or null (write C directly)
   int n_pad, m_pad;
   Status* st;
+  int epi;                // EpiKind, on elements written to C with beta = 0
+  const void* aux;
+  int ld_aux, aux_vec;    // aux_vec: rows of aux start on 32-byte boundaries
   int vec;                // C base and ldc allow 16-byte (1) or 32-byte (2) row segments
   int ws_wide;            // ws 32-byte aligned: partial rows as whole 32-byte sectors
 };
@@ -114,6 +121,130 @@ __device__ __forceinline__ void st_f32x8(float* p, const uint32_t* v) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
                "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                : "memory");
+}
+
+__device__ __forceinline__ void ld_f32x8(const float* p, float* v) {
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+
+// One element's epilogue; h: tanh' activation.
+__device__ __forceinline__ float epilogue(int epi, float x, float h) {
+  return epi == kEpiTanh ? tanhf(x) : (epi == kEpiDtanh ? x * (1.0f - h * h) : x);
+}
+// aux element (row, col) of C's type.
+__device__ __forceinline__ float aux_at(const void* aux, int ld, int c_bf16, size_t row, int col) {
+  return c_bf16 ? __uint_as_float((uint32_t)static_cast<const uint16_t*>(aux)[row * ld + col] << 16)
+                : static_cast<const float*>(aux)[row * ld + col];
+}
+
+// 32 columns of C from column nb of one row: beta C + acc, columns below N.
+__device__ __forceinline__ void store32(const TcArgs& a, const uint32_t (&acc)[32], size_t row, int nb) {
+  if (a.beta == 0.0f && nb + 32 <= a.N && a.vec) {
+    // whole 32-column segment, 16-byte aligned rows: vector stores (32-byte
+    // aligned rows: whole sectors)
+    if (a.c_bf16) {
+      uint16_t* crow = static_cast<uint16_t*>(a.C) + row * a.ldc + nb;
+      uint32_t w[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        w[e] = tc::pack_bf16x2(__uint_as_float(acc[2 * e]), __uint_as_float(acc[2 * e + 1]));
+      if (a.vec == 2) {
+        st_f32x8(reinterpret_cast<float*>(crow), w);
+        st_f32x8(reinterpret_cast<float*>(crow + 16), w + 8);
+      } else {
+        uint4* dst = reinterpret_cast<uint4*>(crow);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+      }
+    } else if (a.vec == 2) {
+      float* crow = static_cast<float*>(a.C) + row * a.ldc + nb;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st_f32x8(crow + 8 * q, acc + 8 * q);
+    } else {
+      uint4* dst = reinterpret_cast<uint4*>(static_cast<float*>(a.C) + row * a.ldc + nb);
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        dst[q] = make_uint4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    }
+  } else if (a.c_bf16) {
+    uint16_t* crow = static_cast<uint16_t*>(a.C) + row * a.ldc;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      const int n = nb + q;
+      if (n < a.N) {
+        float v = __uint_as_float(acc[q]);
+        if (a.beta != 0.0f) v = fmaf(a.beta, __uint_as_float((uint32_t)crow[n] << 16), v);
+        crow[n] = (uint16_t)(tc::pack_bf16x2(v, 0.0f) & 0xFFFFu);
+      }
+    }
+  } else {
+    float* crow = static_cast<float*>(a.C) + row * a.ldc;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int n = nb + 8 * g;
+      if (a.vec == 2 && a.beta == 0.0f && n + 8 <= a.N) {   // narrow heads: whole sectors
+        st_f32x8(crow + n, acc + 8 * g);
+        continue;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (n + q < a.N) {
+          float v = __uint_as_float(acc[8 * g + q]);
+          if (a.beta != 0.0f) v = fmaf(a.beta, crow[n + q], v);
+          crow[n + q] = v;
+        }
+      }
+    }
+  }
+}
+
+// The tanh' activations of one row's 32 columns from nb (0 beyond N), all in
+// flight at once.
+__device__ __forceinline__ void load_aux32(const TcArgs& a, size_t row, int nb, float (&h)[32]) {
+  if (a.aux_vec && nb + 32 <= a.N) {
+    if (a.c_bf16) {
+      const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.aux) +
+                                                      row * a.ld_aux + nb);
+      uint4 u[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) u[g] = __ldg(p + g);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const uint32_t w[4] = {u[g].x, u[g].y, u[g].z, u[g].w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          h[8 * g + j] = __uint_as_float(j & 1 ? w[j >> 1] & 0xFFFF0000u : w[j >> 1] << 16);
+      }
+    } else {
+      const float* p = static_cast<const float*>(a.aux) + row * a.ld_aux + nb;
+#pragma unroll
+      for (int g = 0; g < 4; ++g) ld_f32x8(p + 8 * g, h + 8 * g);
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    h[j] = nb + j < a.N ? aux_at(a.aux, a.ld_aux, a.c_bf16, row, nb + j) : 0.0f;
+}
+
+// 32 accumulator columns of one row.  A bf16 result is rounded before its
+// tanh or tanh' too, as when they were passes over the stored product.
+__device__ __forceinline__ void epilogue32(const TcArgs& a, uint32_t (&acc)[32], const float (&h)[32]) {
+  if (a.c_bf16) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      acc[q] = tc::pack_bf16x2(__uint_as_float(acc[q]), 0.0f) << 16;
+  }
+  if (a.epi == kEpiTanh) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] = __float_as_uint(tanhf(__uint_as_float(acc[q])));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      acc[q] = __float_as_uint(__uint_as_float(acc[q]) * (1.0f - h[q] * h[q]));
+  }
 }
 
 // BN = 320 (for N in (256, 320]: the weight gradients' 264 augmented
@@ -148,6 +279,7 @@ __global__ void __launch_bounds__(192, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
           TcArgs args) {
   using TL = Tile<TF32, A_MN, B_MN, BN>;
+  constexpr int kProducer = 4, kIssuer = 5;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~(uintptr_t)1023u);
@@ -170,7 +302,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     bar->abort = 0;
     tc::mbar_fence_init();
   }
-  if (warp == 5) {
+  if (warp == kIssuer) {
     tc::tmem_alloc(&bar->tmem_base, TL::kTmemCols);
     tc::tmem_relinquish();
   }
@@ -180,9 +312,15 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
   const uint32_t tmem = bar->tmem_base;
   const uint32_t s_base = tc::smem_u32(smem);
 
-  if (warp == 4) {
+  if (warp == kProducer) {
     // ---- producer: TMA tiles of A and B into the ring ----
     if ((tid & 31) == 0) {
+      // MN-major blocks of 128 bytes that hold rows or columns of the product
+      // (the others' accumulator rows and columns are never read back)
+      const int na = min(kBM / TL::kElemsPer128, (args.M - m0 + TL::kElemsPer128 - 1) / TL::kElemsPer128);
+      const int nb = min(BN / TL::kElemsPer128, (args.N - n0 + TL::kElemsPer128 - 1) / TL::kElemsPer128);
+      const uint32_t bytes = (A_MN ? na * (TL::kBK * 128) : TL::kABytes) +
+                             (B_MN ? nb * (TL::kBK * 128) : TL::kBBytes);
       for (int c = 0; c < n_chunks; ++c) {
         const int s = c % kStages;
         if (c >= kStages &&
@@ -190,18 +328,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
           break;
         uint8_t* a_dst = smem + s * TL::kStage;
         uint8_t* b_dst = a_dst + TL::kABytes;
-        tc::mbar_arrive_expect_tx(&bar->full[s], TL::kStage);
+        tc::mbar_arrive_expect_tx(&bar->full[s], bytes);
         const int k = (c0 + c) * TL::kBK;
         if (A_MN) {
-#pragma unroll
-          for (int j = 0; j < kBM / TL::kElemsPer128; ++j)
+          for (int j = 0; j < na; ++j)
             tma_load_2d(a_dst + j * (TL::kBK * 128), &map_a, m0 + j * TL::kElemsPer128, k, &bar->full[s]);
         } else {
           tma_load_2d(a_dst, &map_a, k, m0, &bar->full[s]);
         }
         if (B_MN) {
-#pragma unroll
-          for (int j = 0; j < BN / TL::kElemsPer128; ++j)
+          for (int j = 0; j < nb; ++j)
             tma_load_2d(b_dst + j * (TL::kBK * 128), &map_b, n0 + j * TL::kElemsPer128, k, &bar->full[s]);
         } else {
 #pragma unroll
@@ -212,7 +348,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
       }
     }
     __syncwarp();
-  } else if (warp == 5) {
+  } else if (warp == kIssuer) {
     // ---- MMA issue ----
     if ((tid & 31) == 0) {
       constexpr uint32_t kId = idesc(TF32, A_MN, B_MN, kBM, BN > 256 ? 256 : BN);
@@ -222,6 +358,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
       constexpr uint32_t kB2 = B_MN ? (256 / TL::kElemsPer128) * (TL::kBK * 128) : 256 * 128;
       constexpr uint32_t kLbo = TL::kBK * 128;          // MN-major: between 128-byte M/N blocks
       constexpr uint32_t kKStepMn = 4096 / TL::kEs;     // MN-major: bytes per 32 bytes of K
+      constexpr uint32_t kSboMn = TF32 ? 512 : 1024;    // and between its K-row groups
+      constexpr uint64_t kTypeMn = TF32 ? 1 : 2;
       bool ok = true;
       for (int c = 0; c < n_chunks && ok; ++c) {
         const int s = c % kStages;
@@ -231,13 +369,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         const uint32_t a0 = s_base + s * TL::kStage, b0 = a0 + TL::kABytes;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t da = A_MN ? desc_sw128(a0 + kk * kKStepMn, kLbo, 1024)
+          const uint64_t da = A_MN ? desc_sw128(a0 + kk * kKStepMn, kLbo, kSboMn, kTypeMn)
                                    : desc_sw128(a0 + kk * 32, 16, 1024);
-          const uint64_t db = B_MN ? desc_sw128(b0 + kk * kKStepMn, kLbo, 1024)
+          const uint64_t db = B_MN ? desc_sw128(b0 + kk * kKStepMn, kLbo, kSboMn, kTypeMn)
                                    : desc_sw128(b0 + kk * 32, 16, 1024);
           mma<TF32>(tmem, da, db, kId, (c > 0 || kk > 0) ? 1u : 0u);
           if constexpr (BN > 256) {
-            const uint64_t db2 = B_MN ? desc_sw128(b0 + kB2 + kk * kKStepMn, kLbo, 1024)
+            const uint64_t db2 = B_MN ? desc_sw128(b0 + kB2 + kk * kKStepMn, kLbo, kSboMn, kTypeMn)
                                       : desc_sw128(b0 + kB2 + kk * 32, 16, 1024);
             mma<TF32>(tmem + 256, da, db2, kId2, (c > 0 || kk > 0) ? 1u : 0u);
           }
@@ -248,10 +386,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     }
     __syncwarp();
   } else {
-    // ---- epilogue: row m0 + tid of the tile, BN columns in chunks of 32 ----
+    // ---- epilogue: one row per thread, BN columns in chunks of 32 ----
+    const int row = m0 + tid;
+    const bool epi = args.epi != kEpiNone && !args.ws && row < args.M;
+    const bool dtanh = epi && args.epi == kEpiDtanh;
+    // tanh': a chunk's activations are loaded while the accumulator is still
+    // being computed, the next chunk's while this one is stored
+    float h[32];
+    if (dtanh) load_aux32(args, (size_t)row, n0, h);
     const bool ok = n_chunks > 0 && tc::mbar_wait(&bar->acc_full, 0, abort, kWaitLimitNs);
     tc::tc_fence_after();
-    const int row = m0 + tid;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
     for (int j = 0; j < BN / 32; ++j) {
@@ -263,6 +407,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         for (int q = 0; q < 32; ++q) acc[q] = 0u;   // no K in range (or a timed-out wait)
       }
       const int nb = n0 + j * 32;
+      if (epi) epilogue32(args, acc, h);
+      if (dtanh && j + 1 < BN / 32) load_aux32(args, (size_t)row, nb + 32, h);
       if (args.ws) {
         // partials of the rows and 32-column groups the reduction reads
         if (row < args.M && nb < args.N) {
@@ -278,60 +424,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
                                   __uint_as_float(acc[4 * q + 2]), __uint_as_float(acc[4 * q + 3]));
           }
         }
-      } else if (row < args.M && args.beta == 0.0f && nb + 32 <= args.N && args.vec) {
-        // whole 32-column segment, 16-byte aligned rows: vector stores
-        // (32-byte aligned rows: whole sectors)
-        if (args.c_bf16) {
-          uint16_t* crow = static_cast<uint16_t*>(args.C) + (size_t)row * args.ldc + nb;
-          uint32_t w[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            w[e] = tc::pack_bf16x2(__uint_as_float(acc[2 * e]), __uint_as_float(acc[2 * e + 1]));
-          if (args.vec == 2) {
-            st_f32x8(reinterpret_cast<float*>(crow), w);
-            st_f32x8(reinterpret_cast<float*>(crow + 16), w + 8);
-          } else {
-            uint4* dst = reinterpret_cast<uint4*>(crow);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-          }
-        } else if (args.vec == 2) {
-          float* crow = static_cast<float*>(args.C) + (size_t)row * args.ldc + nb;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) st_f32x8(crow + 8 * q, acc + 8 * q);
-        } else {
-          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(args.C) +
-                                                  (size_t)row * args.ldc + nb);
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            dst[q] = make_float4(__uint_as_float(acc[4 * q]), __uint_as_float(acc[4 * q + 1]),
-                                 __uint_as_float(acc[4 * q + 2]), __uint_as_float(acc[4 * q + 3]));
-        }
       } else if (row < args.M) {
-        if (args.c_bf16) {
-          uint16_t* crow = static_cast<uint16_t*>(args.C) + (size_t)row * args.ldc;
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const int n = nb + q;
-            if (n < args.N) {
-              float v = __uint_as_float(acc[q]);
-              if (args.beta != 0.0f)
-                v = fmaf(args.beta, __uint_as_float((uint32_t)crow[n] << 16), v);
-              crow[n] = (uint16_t)(tc::pack_bf16x2(v, 0.0f) & 0xFFFFu);
-            }
-          }
-        } else {
-          float* crow = static_cast<float*>(args.C) + (size_t)row * args.ldc;
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const int n = nb + q;
-            if (n < args.N) {
-              float v = __uint_as_float(acc[q]);
-              if (args.beta != 0.0f) v = fmaf(args.beta, crow[n], v);
-              crow[n] = v;
-            }
-          }
-        }
+        store32(args, acc, (size_t)row, nb);
       }
     }
   }
@@ -341,9 +435,304 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     atomicAdd(&args.st->timeouts, 1);
     atomicCAS(&args.st->code, 0, -4);
   }
-  if (warp == 5) {
+  if (warp == kIssuer) {
     tc::tc_fence_after();
     tc::tmem_dealloc(tmem, TL::kTmemCols);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Products over many rows with a short contraction (a layer's forward product
+// or input gradient over a batch: A K-major, at most 9 K-chunks).  They move
+// their rows once and reuse one small B, so a CTA keeps its BN columns of B
+// resident (147 KB at K = 264 tf32, BN = 128) and walks over row tiles: A
+// streams through a ring, two accumulators in tensor memory let a tile's MMAs
+// run under the previous tile's epilogue, and 256-column layers are two
+// column halves on neighbouring CTAs, which read the same rows at the same
+// time (from L2 the second time).  fp32 results with BN = 128 leave as TMA
+// boxes of 32 rows x 32 columns (rows of 128 bytes, 16-byte pieces swizzled so
+// that a thread per row meets no bank conflicts), and the tanh' operand comes
+// in the same way into the same buffer, one per epilogue warp: stores and
+// loads of each thread's own row, 32 bytes at a time, took 49 us for a
+// 65,536 x 256 input gradient with tanh' (32 us here).
+//
+// Where the general kernel would have split K in two over CTAs (fewer than
+// half as many of its tiles as SMs), chunks from `half` on go to a second
+// accumulator and the two are added once: the same sums, bit for bit, without
+// the partials' round trip (a closed loop amplifies a changed rounding).
+//
+// Warps 0-7 (BN = 128) or 0-3: epilogue, warp w on rows 32 (w mod 4) .. + 31
+// and column groups w / 4, w / 4 + 2; then the producer and the MMA issuer.
+// ---------------------------------------------------------------------------
+template <bool TF32, bool B_MN, int BN>
+struct RowTile {
+  static constexpr int kEs = TF32 ? 4 : 2;
+  static constexpr int kBK = 128 / kEs;
+  static constexpr int kElemsPer128 = 128 / kEs;
+  static constexpr int kMaxChunks = 9, kMaxStages = 8;
+  static constexpr uint32_t kStage = kBM * 128;           // A: 128 rows x 128 bytes
+  static constexpr uint32_t kBChunk = BN * 128;
+  static constexpr bool kBoxes = BN == 128;               // TMA epilogue
+  static constexpr int kEpiWarps = kBoxes ? 8 : 4;
+  static constexpr int kThreads = 32 * kEpiWarps + 64;
+  static constexpr int kCtas = kBoxes ? 1 : 2;            // per SM
+  static constexpr uint32_t kBoxBytes = kBoxes ? kEpiWarps * 4096 : 0;
+  static constexpr uint32_t kFixed = kBoxBytes + 512 + 1024;   // boxes, barriers, alignment
+  static constexpr uint32_t kBudget = (kCtas == 1 ? 227 : 113) * 1024;
+  // A stages beside `chunks` resident chunks of B
+  static int stages(int chunks) {
+    const int n = (int)((kBudget - kFixed - chunks * kBChunk) / kStage);
+    return n < kMaxStages ? n : kMaxStages;
+  }
+  static_assert(kBudget >= kFixed + kMaxChunks * kBChunk + 2 * kStage, "at least two stages");
+};
+
+struct RowBars {
+  uint64_t full[8], empty[8];      // A stages
+  uint64_t b_full;
+  uint64_t acc_full[2], acc_empty[2];
+  uint64_t aux[8];                 // per epilogue warp: its tanh' box
+  uint32_t tmem_base;
+  int abort;
+};
+
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(tc::smem_u32(src)), "r"(x), "r"(y)
+               : "memory");
+}
+
+// Wait with the limit whatever the abort flag says (copies still in flight).
+__device__ __forceinline__ void wait_landed(uint64_t* b, uint32_t phase) {
+  const uint64_t t0 = tc::global_timer_ns();
+  while (!tc::mbar_test(b, phase) && tc::global_timer_ns() - t0 < kWaitLimitNs) {
+  }
+}
+
+template <bool TF32, bool B_MN, int BN>
+__global__ void __launch_bounds__((RowTile<TF32, B_MN, BN>::kThreads), (RowTile<TF32, B_MN, BN>::kCtas))
+k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+            const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_aux,
+            TcArgs args, int tiles_m, int tiles_n, int stages, int half, int boxes) {
+  using TL = RowTile<TF32, B_MN, BN>;
+  constexpr int kProducer = TL::kEpiWarps, kIssuer = kProducer + 1;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~(uintptr_t)1023u);
+  const int n_chunks = (args.K + TL::kBK - 1) / TL::kBK;
+  uint8_t* ring = smem + n_chunks * TL::kBChunk;
+  uint8_t* box_mem = ring + stages * TL::kStage;
+  RowBars* bar = reinterpret_cast<RowBars*>(box_mem + TL::kBoxBytes);
+  volatile int* abort = &bar->abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // this CTA's columns, and its row tiles m_first, m_first + m_step, ...
+  const int n0 = (int)(blockIdx.x % tiles_n) * BN;
+  const int m_first = blockIdx.x / tiles_n, m_step = gridDim.x / tiles_n;
+
+  if (tid == 0) {
+    for (int s = 0; s < stages; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    tc::mbar_init(&bar->b_full, 1);
+    for (int k = 0; k < 2; ++k) {
+      tc::mbar_init(&bar->acc_full[k], 1);
+      tc::mbar_init(&bar->acc_empty[k], TL::kEpiWarps);
+    }
+    for (int w = 0; w < TL::kEpiWarps; ++w) tc::mbar_init(&bar->aux[w], 1);
+    bar->abort = 0;
+    tc::mbar_fence_init();
+  }
+  if (warp == kIssuer) {
+    tc::tmem_alloc(&bar->tmem_base, 4 * BN);   // two tiles x (sum, second half's sum)
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+
+  if (warp == kProducer) {
+    if (lane == 0) {
+      tc::mbar_arrive_expect_tx(&bar->b_full, n_chunks * TL::kBChunk);
+      for (int c = 0; c < n_chunks; ++c) {
+        uint8_t* dst = smem + c * TL::kBChunk;
+        const int k = c * TL::kBK;
+        if (B_MN) {
+#pragma unroll
+          for (int j = 0; j < BN / TL::kElemsPer128; ++j)
+            tma_load_2d(dst + j * (TL::kBK * 128), &map_b, n0 + j * TL::kElemsPer128, k, &bar->b_full);
+        } else {
+          tma_load_2d(dst, &map_b, k, n0, &bar->b_full);
+        }
+      }
+      int s = 0, fill = 0;   // next stage, and how often the ring has gone round
+      bool ok = true;
+      for (int m = m_first; m < tiles_m && ok; m += m_step) {
+        for (int c = 0; c < n_chunks; ++c) {
+          ok = fill == 0 || tc::mbar_wait(&bar->empty[s], (uint32_t)(fill - 1) & 1u, abort, kWaitLimitNs);
+          if (!ok) break;
+          tc::mbar_arrive_expect_tx(&bar->full[s], TL::kStage);
+          tma_load_2d(ring + s * TL::kStage, &map_a, c * TL::kBK, m * kBM, &bar->full[s]);
+          if (++s == stages) {
+            s = 0;
+            ++fill;
+          }
+        }
+      }
+      if (*abort) {
+        wait_landed(&bar->b_full, 0);
+        for (int q = 0; q < stages; ++q) {
+          const int fills = fill + (q < s ? 1 : 0);
+          if (fills > 0) wait_landed(&bar->full[q], (uint32_t)(fills - 1) & 1u);
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == kIssuer) {
+    if (lane == 0) {
+      constexpr uint32_t kId = idesc(TF32, false, B_MN, kBM, BN);
+      constexpr uint32_t kLbo = TL::kBK * 128;
+      constexpr uint32_t kKStepMn = 4096 / TL::kEs;
+      constexpr uint32_t kSboMn = TF32 ? 512 : 1024;
+      constexpr uint64_t kTypeMn = TF32 ? 1 : 2;
+      const uint32_t b_base = tc::smem_u32(smem), r_base = tc::smem_u32(ring);
+      bool ok = tc::mbar_wait(&bar->b_full, 0, abort, kWaitLimitNs);
+      int s = 0, item = 0;
+      uint32_t phase = 0;
+      for (int m = m_first; m < tiles_m && ok; m += m_step, ++item) {
+        const uint32_t d0 = tmem + (item & 1) * 2 * BN;
+        ok = item < 2 || tc::mbar_wait(&bar->acc_empty[item & 1], (uint32_t)(item / 2 - 1) & 1u, abort,
+                                       kWaitLimitNs);
+        for (int c = 0; c < n_chunks && ok; ++c) {
+          ok = tc::mbar_wait(&bar->full[s], phase, abort, kWaitLimitNs);
+          if (!ok) break;
+          tc::tc_fence_after();
+          const uint32_t a0 = r_base + s * TL::kStage, b0 = b_base + c * TL::kBChunk;
+          const uint32_t d = d0 + (half && c >= half ? BN : 0);
+          const bool first = c == 0 || c == half;
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint64_t da = desc_sw128(a0 + kk * 32, 16, 1024);
+            const uint64_t db = B_MN ? desc_sw128(b0 + kk * kKStepMn, kLbo, kSboMn, kTypeMn)
+                                     : desc_sw128(b0 + kk * 32, 16, 1024);
+            mma<TF32>(d, da, db, kId, first && kk == 0 ? 0u : 1u);
+          }
+          tc::mma_commit(&bar->empty[s]);
+          if (++s == stages) {
+            s = 0;
+            phase ^= 1u;
+          }
+        }
+        if (ok) tc::mma_commit(&bar->acc_full[item & 1]);
+      }
+      // every MMA has completed before tensor memory is freed (b_full's second phase)
+      tc::mma_commit(&bar->b_full);
+      wait_landed(&bar->b_full, 1);
+    }
+    __syncwarp();
+  } else {
+    const bool box = TL::kBoxes && boxes, box_aux = box && args.epi == kEpiDtanh;
+    uint8_t* mine = box_mem + warp * 4096;   // this warp's box: 32 rows of 128 bytes
+    const int rw = (warp & 3) * 32;          // its rows of the tile
+    const uint32_t lane_addr = tmem + ((uint32_t)rw << 16);
+    constexpr int kGroups = BN / 32, kStep = TL::kEpiWarps / 4;
+    uint32_t aux_phase = 0;
+    bool aux_sent = false, ok = true;
+    // lane 0: the tanh' box of row tile m, column group j
+    auto fetch_aux = [&](int m, int j) {
+      if (lane != 0 || n0 + 32 * j >= args.N) return;
+      tc::mbar_arrive_expect_tx(&bar->aux[warp], 4096);
+      tma_load_2d(mine, &map_aux, n0 + 32 * j, m * kBM + rw, &bar->aux[warp]);
+      aux_sent = true;
+    };
+    if (box_aux && m_first < tiles_m) fetch_aux(m_first, warp >> 2);
+    int item = 0;
+    for (int m = m_first; m < tiles_m; m += m_step, ++item) {
+      const int row = m * kBM + rw + lane;
+      const bool live = row < args.M;
+      const bool direct_aux = args.epi == kEpiDtanh && !box_aux && live;
+      float h[32];
+      if (direct_aux) load_aux32(args, (size_t)row, n0 + (warp >> 2) * 32, h);
+      ok = tc::mbar_wait(&bar->acc_full[item & 1], (uint32_t)(item / 2) & 1u, abort, kWaitLimitNs);
+      if (!ok) break;
+      tc::tc_fence_after();
+#pragma unroll 1
+      for (int j = warp >> 2; j < kGroups; j += kStep) {
+        const int nb = n0 + j * 32;
+        if (nb >= args.N) break;
+        uint32_t acc[32];
+        tc::tmem_ld32(lane_addr + (item & 1) * 2 * BN + j * 32, acc);
+        tc::tmem_ld_wait(acc);
+        if (half) {
+          uint32_t b[32];
+          tc::tmem_ld32(lane_addr + (item & 1) * 2 * BN + BN + j * 32, b);
+          tc::tmem_ld_wait(b);
+#pragma unroll
+          for (int q = 0; q < 32; ++q)
+            acc[q] = __float_as_uint(__uint_as_float(acc[q]) + __uint_as_float(b[q]));
+        }
+        if (box_aux) {
+          ok = tc::mbar_wait(&bar->aux[warp], aux_phase, abort, kWaitLimitNs);
+          if (!ok) break;
+          aux_phase ^= 1u;
+          aux_sent = false;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(mine + lane * 128 + ((q ^ (lane & 7)) << 4));
+            h[4 * q] = v.x;
+            h[4 * q + 1] = v.y;
+            h[4 * q + 2] = v.z;
+            h[4 * q + 3] = v.w;
+          }
+        }
+        if (args.epi != kEpiNone && live) epilogue32(args, acc, h);
+        if (direct_aux && j + kStep < kGroups) load_aux32(args, (size_t)row, nb + 32 * kStep, h);
+        if (box) {
+          if (!box_aux) {   // the warp's previous box has left (tanh': waited for below)
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            __syncwarp();
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<uint4*>(mine + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                make_uint4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+          tc::fence_async_smem();
+          __syncwarp();
+          if (lane == 0 && m * kBM + rw < args.M) {
+            tma_store_2d(&map_c, mine, nb, m * kBM + rw);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
+          if (box_aux) {   // the next tanh' box, once this one has been read out
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            const bool more = j + kStep < kGroups && nb + 32 * kStep < args.N;
+            if (more) fetch_aux(m, j + kStep);
+            else if (m + m_step < tiles_m) fetch_aux(m + m_step, warp >> 2);
+          }
+        } else if (live) {
+          store32(args, acc, (size_t)row, nb);
+        }
+      }
+      if (!ok) break;
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bar->acc_empty[item & 1]);
+    }
+    if (box && lane == 0) {
+      if (aux_sent) wait_landed(&bar->aux[warp], aux_phase);   // (only after a wait gave up)
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && bar->abort) {
+    atomicAdd(&args.st->timeouts, 1);
+    atomicCAS(&args.st->code, 0, -4);
+  }
+  if (warp == kIssuer) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 4 * BN);
   }
 }
 
@@ -360,7 +749,7 @@ template <int BM, bool A_MN, bool B_MN>
 __global__ void __launch_bounds__(256, 2)
 k_gemm_fp32(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B,
             int ldb, int chunks_per_split, void* C, int ldc, float beta, float* ws, int m_pad,
-            int n_pad) {
+            int n_pad, int epi, const float* __restrict__ aux, int ld_aux) {
   constexpr int RM = BM / 16, QA = BM / 32;
   __shared__ __align__(16) float As[2][8][BM + 4];
   __shared__ __align__(16) float Bs[2][8][132];
@@ -445,7 +834,8 @@ k_gemm_fp32(int M, int N, int K, const float* __restrict__ A, int lda, const flo
         if (m < M && n < N) ws[((size_t)blockIdx.z * m_pad + m) * n_pad + n] = acc[i][j];
       } else if (m < M && n < N) {
         float* c = static_cast<float*>(C) + (size_t)m * ldc + n;
-        *c = beta != 0.0f ? fmaf(beta, *c, acc[i][j]) : acc[i][j];
+        const float h = epi == kEpiDtanh ? aux[(size_t)m * ld_aux + n] : 0.0f;
+        *c = beta != 0.0f ? fmaf(beta, *c, acc[i][j]) : epilogue(epi, acc[i][j], h);
       }
     }
   }
@@ -463,7 +853,7 @@ constexpr int kRedGroups = 8;
 constexpr int kRedQuads = 32;
 __global__ void __launch_bounds__(kRedGroups * kRedQuads)
 k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int n_pad, void* C,
-         int ldc, int c_bf16, float beta) {
+         int ldc, int c_bf16, float beta, int epi, const void* __restrict__ aux, int ld_aux) {
   __shared__ float4 part[kRedGroups][kRedQuads];
   const int lane = threadIdx.x % kRedQuads, grp = threadIdx.x / kRedQuads;
   const int qpr = (N + 3) / 4;   // groups of four per row (n_pad is a multiple of 128)
@@ -515,7 +905,9 @@ k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int 
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (n + j >= N) break;
-    float x = r[j];
+    const float h = epi == kEpiDtanh ? aux_at(aux, ld_aux, c_bf16, (size_t)m, n + j) : 0.0f;
+    const float v = c_bf16 && epi ? __uint_as_float(tc::pack_bf16x2(r[j], 0.0f) << 16) : r[j];
+    float x = epilogue(epi, v, h);
     if (c_bf16) {
       uint16_t* c = static_cast<uint16_t*>(C) + (size_t)m * ldc + n + j;
       if (beta != 0.0f) x = fmaf(beta, __uint_as_float((uint32_t)*c << 16), x);
@@ -528,8 +920,8 @@ k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int 
 }
 
 // An MN-major fp32 operand (element (r, k) at k * ld + r) copied K-major:
-// out[r * ldo + k], 32 x 32 tiles through shared memory, both sides coalesced.
-// (The tf32 tensor-core path reads its operands K-major.)
+// out[r * ldo + k], 32 x 32 tiles through shared memory, both sides coalesced
+// (tf32 operands that TMA cannot read in place: base or rows off 16 bytes).
 __global__ void k_transpose(int R, int K, const float* __restrict__ in, int ld, float* out,
                             int ldo) {
   __shared__ float tile[32][33];
@@ -571,8 +963,8 @@ EncodeFn encode_fn() {
 
 // 2-D map of a stored operand: inner dimension (contiguous) and outer
 // dimension, rows ld elements apart; a box of 128 bytes x box_outer rows.
-bool make_map(CUtensorMap* map, bool tf32, const void* ptr, uint64_t inner, uint64_t outer, int ld,
-              uint32_t box_outer) {
+bool make_map(CUtensorMap* map, bool tf32, bool mn, const void* ptr, uint64_t inner, uint64_t outer,
+              int ld, uint32_t box_outer) {
   EncodeFn fn = encode_fn();
   if (!fn) return false;
   const int es = tf32 ? 4 : 2;
@@ -584,8 +976,24 @@ bool make_map(CUtensorMap* map, bool tf32, const void* ptr, uint64_t inner, uint
   // GEMM rounds its operands, instead of the MMA dropping the low bits
   return fn(map, tf32 ? CU_TENSOR_MAP_DATA_TYPE_TFLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
             const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            tf32 && mn ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 2-D fp32 map of a row-major array's boxes of 32 columns (128 bytes, 16-byte
+// pieces swizzled) x box_rows rows.
+bool make_box_map(CUtensorMap* map, const void* ptr, uint64_t cols, uint64_t rows, int ld,
+                  uint32_t box_rows) {
+  EncodeFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[2] = {cols, rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
+  const cuuint32_t box[2] = {32, box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int sm_count_dev() {
@@ -603,23 +1011,35 @@ struct Plan {
   int tiles_m, tiles_n;
   int chunks, per_split, splits;
   int m_pad, n_pad;
+  bool rows;             // many rows, few K-chunks: k_gemm_rows
+  int half;              // its first chunk of the second accumulator, or 0
 };
 
-Plan plan(Prec prec, int M, int N, int K) {
+constexpr int kRowsMaxChunks = RowTile<true, false, 128>::kMaxChunks;
+
+// The narrow tile of k_gemm_rows: one 128-byte block of an MN-major B.
+int narrow_bn(Prec prec) { return prec == kTf32 ? 32 : 64; }
+
+Plan plan(Prec prec, int M, int N, int K, bool a_kmajor) {
   Plan p;
+  p.rows = false;
+  p.half = 0;
   if (prec == kFp32) {
     p.bm = M <= 32 ? 32 : 128;
     p.bn = 128;
     p.bk = 8;
   } else {
     p.bm = kBM;
+    p.bk = prec == kTf32 ? 32 : 64;
     // 320-wide tiles (one CTA over the weight gradients' 264 augmented
     // columns: the other operand read once instead of three times) pay when
-    // there are at least two M-tiles; with one, three 128-wide tiles keep more
-    // CTAs per K-range (measured 28.1 against 37.9 us for 256 x 264 x 65,536,
-    // 25.4 against 21.4 us for 16 x 264 x 65,536)
-    p.bn = (N > 128 && N <= 256) ? 256 : ((N > 256 && N <= 320 && M > kBM) ? 320 : 128);
-    p.bk = prec == kTf32 ? 32 : 64;
+    // there are at least two M-tiles (28.1 against 37.9 us for 256 x 264 x
+    // 65,536, bf16) or a long contraction: 16 x 264 x K in tf32 takes 21 / 35
+    // / 95 us against 27 / 45 / 199 at K = 65,536 / 131,072 / 524,288, but 18
+    // against 16 at 16,384.
+    p.bn = (N > 128 && N <= 256) ? 256
+                                 : ((N > 256 && N <= 320 && (M > kBM || K >= 1024 * p.bk)) ? 320 : 128);
+    p.rows = a_kmajor && p.bn <= 256 && M >= 8 * kBM && K <= kRowsMaxChunks * p.bk;
   }
   p.tiles_m = (M + p.bm - 1) / p.bm;
   p.tiles_n = (N + p.bn - 1) / p.bn;
@@ -633,6 +1053,12 @@ Plan plan(Prec prec, int M, int N, int K) {
   want = std::max(1, std::min(want, p.chunks / 4));
   p.per_split = (p.chunks + want - 1) / want;
   p.splits = (p.chunks + p.per_split - 1) / p.per_split;
+  if (p.rows) {   // nine chunks or fewer: at most two splits
+    p.half = p.splits > 1 ? p.per_split : 0;
+    p.splits = 1;
+    p.bn = N <= narrow_bn(prec) ? narrow_bn(prec) : 128;
+    p.tiles_n = (N + p.bn - 1) / p.bn;
+  }
   p.m_pad = p.tiles_m * p.bm;
   p.n_pad = p.tiles_n * p.bn;
   return p;
@@ -658,56 +1084,94 @@ cudaError_t dispatch_major(bool a_mn, bool b_mn, const Plan& P, const CUtensorMa
   return launch_tc<TF32, false, false, BN>(P, ma, mb, a, s);
 }
 
+template <bool TF32, bool B_MN, int BN>
+cudaError_t launch_rows(const Plan& P, const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a,
+                        cudaStream_t s) {
+  using TL = RowTile<TF32, B_MN, BN>;
+  auto kern = k_gemm_rows<TF32, B_MN, BN>;
+  const int chunks = P.chunks, stages = TL::stages(chunks);
+  const uint32_t smem = TL::kFixed + chunks * TL::kBChunk + stages * TL::kStage;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)TL::kBudget);
+  if (e != cudaSuccess) return e;
+  // result and tanh' boxes by TMA where the arrays allow it: fp32, 16-byte
+  // rows, and whole 16-byte pieces up to column N (a store clips no finer)
+  auto box_ok = [](const void* p, int ld) {
+    return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && ld % 4 == 0;
+  };
+  CUtensorMap mc = ma, mx = ma;
+  bool boxes = TL::kBoxes && !a.c_bf16 && a.beta == 0.0f && a.N % 4 == 0 && box_ok(a.C, a.ldc) &&
+               (a.epi != kEpiDtanh || box_ok(a.aux, a.ld_aux));
+  if (boxes) {
+    boxes = make_box_map(&mc, a.C, a.N, a.M, a.ldc, 32) &&
+            (a.epi != kEpiDtanh || make_box_map(&mx, a.aux, a.N, a.M, a.ld_aux, 32));
+  }
+  // every column tile on the same number of CTAs, at most kCtas per SM in all
+  const int groups = std::max(1, std::min(P.tiles_m, sm_count_dev() * TL::kCtas / P.tiles_n));
+  kern<<<groups * P.tiles_n, TL::kThreads, smem, s>>>(ma, mb, mc, mx, a, P.tiles_m, P.tiles_n, stages,
+                                                      P.half, boxes ? 1 : 0);
+  return cudaGetLastError();
+}
+
+template <bool TF32>
+cudaError_t dispatch_rows(bool b_mn, const Plan& P, const CUtensorMap& ma, const CUtensorMap& mb,
+                          const TcArgs& a, cudaStream_t s) {
+  constexpr int kNarrow = TF32 ? 32 : 64;
+  if (P.bn == 128)
+    return b_mn ? launch_rows<TF32, true, 128>(P, ma, mb, a, s) : launch_rows<TF32, false, 128>(P, ma, mb, a, s);
+  return b_mn ? launch_rows<TF32, true, kNarrow>(P, ma, mb, a, s)
+              : launch_rows<TF32, false, kNarrow>(P, ma, mb, a, s);
+}
+
 bool tma_ok(const Operand& o, int es) {
   return (reinterpret_cast<uintptr_t>(o.ptr) & 15u) == 0 && ((size_t)o.ld * es) % 16 == 0;
 }
 
 }  // namespace
 
-// tf32 with MN-major operands: K-major copies of A and B ahead of the partials.
+// Room for a K-major copy of an MN-major operand, in 256-byte multiples.
 size_t transposed_floats(int rows, int K) {
-  return ((size_t)rows * ((K + 3) & ~3) + 63) & ~(size_t)63;   // 256-byte multiples
+  return ((size_t)rows * ((K + 3) & ~3) + 63) & ~(size_t)63;
 }
 
 size_t workspace_bytes(int M, int N, int K) {
   size_t best = 0;
   for (Prec p : {kFp32, kTf32, kBf16}) {
-    const Plan P = plan(p, M, N, K);
-    size_t b = P.splits > 1 ? (size_t)P.splits * P.m_pad * P.n_pad * sizeof(float) : 0;
-    if (p == kTf32) b += (transposed_floats(M, K) + transposed_floats(N, K)) * sizeof(float);
-    best = std::max(best, b);
+    const Plan P = plan(p, M, N, K, false);   // (K-major A may need fewer splits, never more)
+    best = std::max(best, P.splits > 1 ? (size_t)P.splits * P.m_pad * P.n_pad * sizeof(float) : 0);
   }
   return best;
 }
 
 cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Operand& B_in,
                    void* C, int ldc, bool c_bf16, float beta, float* ws, size_t ws_bytes,
-                   Status* st, cudaStream_t s) {
+                   Status* st, cudaStream_t s, const Epilogue& epi) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  if (epi.kind != kEpiNone && beta != 0.0f) return cudaErrorInvalidValue;
   Operand A = A_in, B = B_in;
-  if (prec == kTf32 && (A.mn_major || B.mn_major)) {
-    // kind::tf32 reads K-major operands: transpose the MN-major ones into
-    // the front of the workspace, 256-byte aligned
+  if (prec == kTf32 && ((A.mn_major && !tma_ok(A, 4)) || (B.mn_major && !tma_ok(B, 4)))) {
+    // transpose the operands that TMA cannot read into the front of the
+    // workspace, 256-byte aligned
     const size_t need = (transposed_floats(M, K) + transposed_floats(N, K)) * sizeof(float);
     if (!ws || ws_bytes < need) return cudaErrorInvalidValue;
     float* dst = ws;
     for (Operand* o : {&A, &B}) {
       const int rows = o == &A ? M : N;
-      if (o->mn_major) {
+      if (o->mn_major && !tma_ok(*o, 4)) {
         const int ldo = (K + 3) & ~3;
         k_transpose<<<dim3((rows + 31) / 32, (ldo + 31) / 32), dim3(32, 8), 0, s>>>(
             rows, K, static_cast<const float*>(o->ptr), o->ld, dst, ldo);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         *o = {dst, ldo, false};
+        dst += transposed_floats(rows, K);
       }
-      dst += transposed_floats(rows, K);
     }
     const size_t used = (size_t)(dst - ws) * sizeof(float);
     ws = dst;
     ws_bytes -= used;
   }
-  Plan P = plan(prec, M, N, K);
+  Plan P = plan(prec, M, N, K, !A.mn_major);
   const size_t need = (size_t)P.splits * P.m_pad * P.n_pad * sizeof(float);
   if (P.splits > 1 && (!ws || ws_bytes < need)) {
     // no room for partials: one CTA per tile over the whole K
@@ -722,7 +1186,8 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
     const float* b = static_cast<const float*>(B.ptr);
 #define AUV_FP32_GEMM(TM, AM, BM)                                                           \
   k_gemm_fp32<TM, AM, BM><<<grid, 256, 0, s>>>(M, N, K, a, A.ld, b, B.ld, P.per_split, C, ldc, \
-                                               beta, part, P.m_pad, P.n_pad)
+                                               beta, part, P.m_pad, P.n_pad, (int)epi.kind, \
+                                               static_cast<const float*>(epi.aux), epi.ld_aux)
 #define AUV_FP32_MAJOR(TM)                                         \
   if (A.mn_major && B.mn_major) AUV_FP32_GEMM(TM, true, true);     \
   else if (A.mn_major) AUV_FP32_GEMM(TM, true, false);             \
@@ -741,19 +1206,25 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
     CUtensorMap ma, mb;
     // K-major: inner = K, outer = rows (box: 128 B of K x tile rows);
     // MN-major: inner = rows, outer = K (box: 128 B of rows x BK).
-    const bool ok_a = A.mn_major ? make_map(&ma, tf32, A.ptr, M, K, A.ld, bk)
-                                 : make_map(&ma, tf32, A.ptr, K, M, A.ld, kBM);
-    const bool ok_b = B.mn_major ? make_map(&mb, tf32, B.ptr, N, K, B.ld, bk)
-                                 : make_map(&mb, tf32, B.ptr, K, N, B.ld, P.bn > 256 ? 64 : P.bn);
+    const bool ok_a = A.mn_major ? make_map(&ma, tf32, true, A.ptr, M, K, A.ld, bk)
+                                 : make_map(&ma, tf32, false, A.ptr, K, M, A.ld, kBM);
+    const bool ok_b = B.mn_major ? make_map(&mb, tf32, true, B.ptr, N, K, B.ld, bk)
+                                 : make_map(&mb, tf32, false, B.ptr, K, N, B.ld, P.bn > 256 ? 64 : P.bn);
     if (!ok_a || !ok_b) return cudaErrorInvalidValue;
     const int ces = c_bf16 ? 2 : 4;
     const int vec = (reinterpret_cast<uintptr_t>(C) % 32 == 0 && ((size_t)ldc * ces) % 32 == 0)
                         ? 2
                         : ((reinterpret_cast<uintptr_t>(C) % 16 == 0 && ((size_t)ldc * ces) % 16 == 0) ? 1 : 0);
     const int ws_wide = reinterpret_cast<uintptr_t>(part) % 32 == 0 ? 1 : 0;
-    TcArgs a = {M,     N,      K,       P.per_split, C,  ldc,    c_bf16 ? 1 : 0,
-                beta,  part,   P.n_pad, P.m_pad,     st, vec,    ws_wide};
-    if (tf32)
+    const int aux_vec = epi.kind == kEpiDtanh && reinterpret_cast<uintptr_t>(epi.aux) % 32 == 0 &&
+                        ((size_t)epi.ld_aux * ces) % 32 == 0;
+    TcArgs a = {M,    N,    K,       P.per_split, C,  ldc,           c_bf16 ? 1 : 0,
+                beta, part, P.n_pad, P.m_pad,     st, (int)epi.kind, epi.aux,
+                epi.ld_aux, aux_vec, vec, ws_wide};
+    if (P.rows)
+      e = tf32 ? dispatch_rows<true>(B.mn_major, P, ma, mb, a, s)
+               : dispatch_rows<false>(B.mn_major, P, ma, mb, a, s);
+    else if (tf32)
       e = P.bn == 320   ? dispatch_major<true, 320>(A.mn_major, B.mn_major, P, ma, mb, a, s)
           : P.bn == 256 ? dispatch_major<true, 256>(A.mn_major, B.mn_major, P, ma, mb, a, s)
                         : dispatch_major<true, 128>(A.mn_major, B.mn_major, P, ma, mb, a, s);
@@ -765,7 +1236,8 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
   if (e != cudaSuccess || !part) return e;
   const size_t quads = (size_t)M * ((N + 3) / 4);
   k_reduce<<<(unsigned)((quads + kRedQuads - 1) / kRedQuads), kRedGroups * kRedQuads, 0, s>>>(
-      M, N, P.splits, part, P.m_pad, P.n_pad, C, ldc, c_bf16 ? 1 : 0, beta);
+      M, N, P.splits, part, P.m_pad, P.n_pad, C, ldc, c_bf16 ? 1 : 0, beta, (int)epi.kind, epi.aux,
+      epi.ld_aux);
   return cudaGetLastError();
 }
 
@@ -775,8 +1247,16 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
 // ---------------------------------------------------------------------------
 // C ABI (include/auvenv.h): the learners' dense product on its own
 // ---------------------------------------------------------------------------
+namespace {
+// The part of the workspace that holds K-major copies of MN-major tf32
+// operands (used for those that TMA cannot read in place).
+size_t copies_bytes(int M, int N, int K) {
+  return (auv::gemm::transposed_floats(M, K) + auv::gemm::transposed_floats(N, K)) * sizeof(float);
+}
+}  // namespace
+
 extern "C" size_t auv_gemm_workspace_bytes(int M, int N, int K) {
-  return (M > 0 && N > 0 && K > 0) ? auv::gemm::workspace_bytes(M, N, K) : 0;
+  return (M > 0 && N > 0 && K > 0) ? auv::gemm::workspace_bytes(M, N, K) + copies_bytes(M, N, K) : 0;
 }
 
 extern "C" int auv_gemm(uint32_t precision, int M, int N, int K, const void* A, int lda, int a_mn,
@@ -788,6 +1268,9 @@ extern "C" int auv_gemm(uint32_t precision, int M, int N, int K, const void* A, 
       lda < (a_mn ? M : K) || ldb < (b_mn ? N : K))
     return AUV_ERR_INVALID;
   static_assert(sizeof(auv::Status) == sizeof(auv_status), "status block layout");
+  // an MN-major tf32 operand needs the copies' room whatever its alignment
+  if (precision == AUV_PPO_TF32 && (a_mn || b_mn) && (!workspace || workspace_bytes < copies_bytes(M, N, K)))
+    return AUV_ERR_SIZE;
   const auv::gemm::Operand a = {A, lda, a_mn != 0}, b = {B, ldb, b_mn != 0};
   const cudaError_t e = auv::gemm::launch(static_cast<auv::gemm::Prec>(precision), M, N, K, a, b, C,
                                           ldc, c_bf16 != 0, beta, static_cast<float*>(workspace),

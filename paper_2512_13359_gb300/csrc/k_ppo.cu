@@ -156,7 +156,7 @@ cudaError_t launch_gae(int n, int T, const float* rew, const uint8_t* done, cons
 // ---------------------------------------------------------------------------
 // PPO minibatch update (Schulman et al. 2017).  The GEMMs of the two MLPs run
 // in k_gemm.cu and the tcgen05 engine; these kernels do everything around them: the
-// epoch permutation and minibatch gather, tanh forward and backward, the
+// epoch permutation and minibatch gather, the
 // per-sample loss and its gradient at the heads, the minibatch statistics,
 // the global gradient norm and Adam, and the weight-layout conversion.
 // ---------------------------------------------------------------------------
@@ -452,70 +452,6 @@ __global__ void __launch_bounds__(kT) k_gather_sm(Dims d, PermKey key, const Ste
   if (threadIdx.x == 0) {
     out.adv_part[2 * blockIdx.x] = s[0];
     out.adv_part[2 * blockIdx.x + 1] = s[1];
-  }
-}
-
-__global__ void __launch_bounds__(kT) k_tanh_fwd(float* __restrict__ h, int ld, int B, int H4) {
-  const size_t n = (size_t)B * H4;
-  for (size_t e = blockIdx.x * (size_t)kT + threadIdx.x; e < n; e += (size_t)gridDim.x * kT) {
-    const size_t row = e / H4, c = e - row * H4;
-    float4* p = reinterpret_cast<float4*>(h + row * ld) + c;
-    float4 z = *p;
-    z.x = tanhf(z.x); z.y = tanhf(z.y); z.z = tanhf(z.z); z.w = tanhf(z.w);
-    *p = z;
-  }
-}
-
-__global__ void __launch_bounds__(kT) k_tanh_fwd_bf16(__nv_bfloat16* __restrict__ h, int ld,
-                                                      int B, int H8) {
-  const size_t n = (size_t)B * H8;
-  for (size_t e = blockIdx.x * (size_t)kT + threadIdx.x; e < n; e += (size_t)gridDim.x * kT) {
-    const size_t row = e / H8, c = e - row * H8;
-    uint4* p = reinterpret_cast<uint4*>(h + row * ld) + c;
-    uint4 u = *p;
-    __nv_bfloat162* v = reinterpret_cast<__nv_bfloat162*>(&u);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 z = __bfloat1622float2(v[k]);
-      v[k] = __floats2bfloat162_rn(tanhf(z.x), tanhf(z.y));
-    }
-    *p = u;
-  }
-}
-
-__global__ void __launch_bounds__(kT) k_tanh_bwd_bf16(__nv_bfloat16* __restrict__ g, int ldg,
-                                                      const __nv_bfloat16* __restrict__ h,
-                                                      int ldh, int B, int H8) {
-  const size_t n = (size_t)B * H8;
-  for (size_t e = blockIdx.x * (size_t)kT + threadIdx.x; e < n; e += (size_t)gridDim.x * kT) {
-    const size_t row = e / H8, c = e - row * H8;
-    uint4* pg = reinterpret_cast<uint4*>(g + row * ldg) + c;
-    uint4 hv = __ldg(reinterpret_cast<const uint4*>(h + row * ldh) + c);
-    uint4 gv = *pg;
-    __nv_bfloat162* gg = reinterpret_cast<__nv_bfloat162*>(&gv);
-    const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&hv);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 y = __bfloat1622float2(hh[k]);
-      const float2 x = __bfloat1622float2(gg[k]);
-      gg[k] = __floats2bfloat162_rn(x.x * (1.0f - y.x * y.x), x.y * (1.0f - y.y * y.y));
-    }
-    *pg = gv;
-  }
-}
-
-__global__ void __launch_bounds__(kT) k_tanh_bwd(float* __restrict__ g, int ldg,
-                                                 const float* __restrict__ h, int ldh, int B,
-                                                 int H4) {
-  const size_t n = (size_t)B * H4;
-  for (size_t e = blockIdx.x * (size_t)kT + threadIdx.x; e < n; e += (size_t)gridDim.x * kT) {
-    const size_t row = e / H4, c = e - row * H4;
-    float4* pg = reinterpret_cast<float4*>(g + row * ldg) + c;
-    const float4 y = __ldg(reinterpret_cast<const float4*>(h + row * ldh) + c);
-    float4 v = *pg;
-    v.x *= 1.0f - y.x * y.x; v.y *= 1.0f - y.y * y.y;
-    v.z *= 1.0f - y.z * y.z; v.w *= 1.0f - y.w * y.w;
-    *pg = v;
   }
 }
 
@@ -839,27 +775,6 @@ cudaError_t launch_gather_sm(const Dims& d, const PermKey& k, const StepCtl* ctl
 
 cudaError_t launch_step_advance(StepCtl* ctl, cudaStream_t s) {
   k_step_advance<<<1, 1, 0, s>>>(ctl);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tanh_fwd(bool bf16, void* h, int ld, int B, int H, cudaStream_t s) {
-  if (bf16)
-    k_tanh_fwd_bf16<<<grid_for((size_t)B * H / 8), kT, 0, s>>>(static_cast<__nv_bfloat16*>(h), ld,
-                                                               B, H / 8);
-  else
-    k_tanh_fwd<<<grid_for((size_t)B * H / 4), kT, 0, s>>>(static_cast<float*>(h), ld, B, H / 4);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tanh_bwd(bool bf16, void* g, int ldg, const void* h, int ldh, int B, int H,
-                            cudaStream_t s) {
-  if (bf16)
-    k_tanh_bwd_bf16<<<grid_for((size_t)B * H / 8), kT, 0, s>>>(
-        static_cast<__nv_bfloat16*>(g), ldg, static_cast<const __nv_bfloat16*>(h), ldh, B, H / 8);
-  else
-    k_tanh_bwd<<<grid_for((size_t)B * H / 4), kT, 0, s>>>(static_cast<float*>(g), ldg,
-                                                          static_cast<const float*>(h), ldh, B,
-                                                          H / 4);
   return cudaGetLastError();
 }
 

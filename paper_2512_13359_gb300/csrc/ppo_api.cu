@@ -201,10 +201,11 @@ ppo::LossHp loss_hp(const auv_ppo* p) {
 // operand is B (K-major unless transposed) and second A (K-major when
 // transposed).
 cudaError_t gemm(auv_ppo* p, bool ta, bool tb, int m, int n, int k, const void* A, int lda,
-                 const void* B, int ldb, void* C, int ldc, bool c32, cudaStream_t s) {
+                 const void* B, int ldb, void* C, int ldc, bool c32, cudaStream_t s,
+                 const auv::gemm::Epilogue& epi = auv::gemm::Epilogue()) {
   const auv::gemm::Operand a = {B, ldb, tb}, b = {A, lda, !ta};
   return auv::gemm::launch(static_cast<auv::gemm::Prec>(p->cfg.precision), n, m, k, a, b, C, ldc,
-                           p->bf16 && !c32, 0.0f, p->gws, p->gws_bytes, p->st, s);
+                           p->bf16 && !c32, 0.0f, p->gws, p->gws_bytes, p->st, s, epi);
 }
 
 // Workspace of every product the learner runs (both networks).
@@ -240,16 +241,14 @@ int forward(auv_ppo* p, int net, cudaStream_t s) {
   const char* w = weights_for_gemm(p, net);
   const char *w1 = w, *w2 = w + (size_t)d.H * d.Dp * es, *w3 = w2 + (size_t)d.H * d.Hp * es;
   cudaError_t e;
+  // the hidden layers' tanh in the products' epilogues
+  const auv::gemm::Epilogue act = {auv::gemm::kEpiTanh};
   if ((e = gemm(p, true, false, d.H, d.B, d.Dp, w1, d.Dp, p->X, d.Dp, p->h1[net],
-                 d.Ha, false, s)))
+                 d.Ha, false, s, act)))
     return cuda_fail(p, e, "forward layer 1");
-  if ((e = ppo::launch_tanh_fwd(p->bf16, p->h1[net], d.Ha, d.B, d.H, s)))
-    return cuda_fail(p, e, "tanh 1");
   if ((e = gemm(p, true, false, d.H, d.B, d.Hp, w2, d.Hp, p->h1[net], d.Ha,
-                 p->h2[net], d.Ha, false, s)))
+                 p->h2[net], d.Ha, false, s, act)))
     return cuda_fail(p, e, "forward layer 2");
-  if ((e = ppo::launch_tanh_fwd(p->bf16, p->h2[net], d.Ha, d.B, d.H, s)))
-    return cuda_fail(p, e, "tanh 2");
   if ((e = gemm(p, true, false, p->out[net], d.B, d.Hp, w3, d.Hp, p->h2[net], d.Ha,
                  p->y[net], ld_head(p, net), true, s)))
     return cuda_fail(p, e, "forward layer 3");
@@ -286,17 +285,17 @@ int backward(auv_ppo* p, int net, const void* gy, cudaStream_t s) {
       return cuda_fail(p, e, "gradient W1");
     return AUV_OK;
   }
-  if ((e = gemm(p, false, false, d.H, d.B, out, w3, d.Hp, gy, ldy, gz2, d.H, false, s)))
+  // input gradients with tanh' in the epilogues (gz1 overwrites H2, which no
+  // later product reads)
+  const auv::gemm::Epilogue d2 = {auv::gemm::kEpiDtanh, p->h2[net], d.Ha};
+  const auv::gemm::Epilogue d1 = {auv::gemm::kEpiDtanh, p->h1[net], d.Ha};
+  if ((e = gemm(p, false, false, d.H, d.B, out, w3, d.Hp, gy, ldy, gz2, d.H, false, s, d2)))
     return cuda_fail(p, e, "gradient H2");
-  if ((e = ppo::launch_tanh_bwd(p->bf16, gz2, d.H, p->h2[net], d.Ha, d.B, d.H, s)))
-    return cuda_fail(p, e, "tanh' 2");
   if ((e = gemm(p, false, true, d.Hp, d.H, d.B, p->h1[net], d.Ha, gz2, d.H, g2, d.Hp,
                  true, s)))
     return cuda_fail(p, e, "gradient W2");
-  if ((e = gemm(p, false, false, d.H, d.B, d.H, w2, d.Hp, gz2, d.H, gz1, d.Ha, false, s)))
+  if ((e = gemm(p, false, false, d.H, d.B, d.H, w2, d.Hp, gz2, d.H, gz1, d.Ha, false, s, d1)))
     return cuda_fail(p, e, "gradient H1");
-  if ((e = ppo::launch_tanh_bwd(p->bf16, gz1, d.Ha, p->h1[net], d.Ha, d.B, d.H, s)))
-    return cuda_fail(p, e, "tanh' 1");
   if ((e = gemm(p, false, true, d.Dp, d.H, d.B, p->X, d.Dp, gz1, d.Ha, g1, d.Dp,
                  true, s)))
     return cuda_fail(p, e, "gradient W1");

@@ -10,12 +10,17 @@
 // runs in the k_shac_* kernels of k_adjoint.cu; the policy network's dense
 // products run in the library's GEMM (k_gemm.cu: tcgen05 with tf32 operands,
 // or fp32 on the CUDA cores) on the augmented layout of the PPO learner (a
-// constant-1 input column carries each bias).  Forward: for each
+// constant-1 input column carries each bias; tanh and tanh' run in the
+// products' epilogues).  Forward: for each
 // step, observation -> policy GEMMs (activations kept for every step) ->
 // action and physics (the env advances).  Backward, t = T-1 .. 0: physics
 // VJP of step t (the state adjoint lam and the head gradient), the policy's
-// backward (weight gradients accumulated over steps, input gradient), then
-// the observation VJP into lam.  The terminal critic seeds lam with
+// input gradients, then the observation VJP into lam.  The weight gradients
+// sum over steps as well as envs, so they wait for a group of steps whose
+// layer gradients fit 1 GiB and then run as three products over all of its
+// rows: one per step each was a sixth of the group's work per launch, with its
+// own split-K partials (65,536 envs x 32 steps, tf32: a quarter of the
+// window's time).  The terminal critic seeds lam with
 // coef_V dV(o(x_T))/dx_T through the value network's input gradient.
 #include <algorithm>
 #include <cstdio>
@@ -42,10 +47,11 @@ struct Gemm {
   Status* st;
   cudaStream_t s;
   cudaError_t operator()(bool ta, bool tb, int m, int n, int k, const float* A, int lda,
-                         const float* B, int ldb, float* C, int ldc, float beta = 0.0f) const {
+                         const float* B, int ldb, float* C, int ldc, float beta = 0.0f,
+                         const gemm::Epilogue& epi = gemm::Epilogue()) const {
     const gemm::Operand a = {B, ldb, tb}, b = {A, lda, !ta};
     return gemm::launch(tf32 ? gemm::kTf32 : gemm::kFp32, n, m, k, a, b, C, ldc, false, beta, ws,
-                        ws_bytes, st, s);
+                        ws_bytes, st, s, epi);
   }
 };
 
@@ -77,9 +83,13 @@ Layout layout(int n, int T, int H, bool paper) {
   L.o_H1 = take(T * N * L.Hp * 4);
   L.o_H2 = take(T * N * L.Hp * 4);
   L.o_Y = take(T * N * kLdy * 4);
-  L.o_G = take(N * H * 4);
+  // dL/dZ2, dL/dZ1 and dL/dY of the steps whose weight gradients run together
+  const size_t group = ((size_t)1 << 30) / (N * (2 * (size_t)H + kLdy) * 4);
+  L.G = (int)std::max<size_t>(1, std::min<size_t>(group, (size_t)T));
+  L.o_G2 = take(L.G * N * H * 4);
+  L.o_G1 = take(L.G * N * H * 4);
+  L.o_gY = take(L.G * N * kLdy * 4);
   L.o_GX = take(N * L.Dp * 4);
-  L.o_gY = take(N * kLdy * 4);
   L.o_lam = take((size_t)L.S * N * 4);
   L.o_done = take(T * N);
   L.o_rew = take(T * N * 4);
@@ -94,9 +104,14 @@ Layout layout(int n, int T, int H, bool paper) {
   // the GEMM workspace of the largest product (policy and value networks)
   size_t gws = 0;
   for (int o : {L.out, 1}) {
-    const int shapes[9][3] = {{n, H, L.Dp}, {n, H, L.Hp}, {n, o, L.Hp},   {o, L.Hp, n},    {n, H, o},
-                              {H, L.Hp, n}, {n, H, H},    {H, L.Dp, n}, {n, L.Dp, H}};
+    const int shapes[6][3] = {{n, H, L.Dp}, {n, H, L.Hp}, {n, o, L.Hp},
+                              {n, H, o},    {n, H, H},    {n, L.Dp, H}};
     for (const auto& sh : shapes) gws = std::max(gws, gemm::workspace_bytes(sh[0], sh[1], sh[2]));
+  }
+  for (int steps : {L.G, T % L.G}) {   // weight gradients: full groups, the last one
+    const int shapes[3][3] = {{L.out, L.Hp, steps * n}, {H, L.Hp, steps * n}, {H, L.Dp, steps * n}};
+    for (const auto& sh : shapes)
+      if (steps) gws = std::max(gws, gemm::workspace_bytes(sh[0], sh[1], sh[2]));
   }
   L.o_gws = take(gws);
   L.gws_bytes = gws;
@@ -125,8 +140,8 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
   const int n = L.n, T = L.T, H = L.H, Dp = L.Dp, Hp = L.Hp;
   const size_t N = (size_t)n;
   auto F = [&](size_t o) { return reinterpret_cast<float*>(base + o); };
-  float *X = F(L.o_X), *H1 = F(L.o_H1), *H2 = F(L.o_H2), *Y = F(L.o_Y), *G = F(L.o_G),
-        *GX = F(L.o_GX), *gY = F(L.o_gY), *lam = F(L.o_lam), *rew = F(L.o_rew),
+  float *X = F(L.o_X), *H1 = F(L.o_H1), *H2 = F(L.o_H2), *Y = F(L.o_Y), *G2 = F(L.o_G2),
+        *G1 = F(L.o_G1), *GX = F(L.o_GX), *gY = F(L.o_gY), *lam = F(L.o_lam), *rew = F(L.o_rew),
         *VH1 = F(L.o_VH1), *VH2 = F(L.o_VH2), *V = F(L.o_V), *gYv = F(L.o_gYv),
         *wp = F(L.o_wp), *wv = F(L.o_wv), *gp = F(L.o_gp), *sc = F(L.o_sc);
   uint8_t* done = reinterpret_cast<uint8_t*>(base + L.o_done);
@@ -156,13 +171,16 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
     return cfail(e, "value weights");
   if ((e = cudaMemsetAsync(gp, 0, L.n_aug_p * 4, s))) return cfail(e, "clear gradient");
 
+  const gemm::Epilogue act = {gemm::kEpiTanh};
+  auto dact = [&](const float* h) { return gemm::Epilogue{gemm::kEpiDtanh, h, Hp}; };
+
   // ---- forward ----
   for (int t = 0; t < T; ++t) {
     if ((e = launch_obs(M, B, SCs(t), Xs(t), Dp, obs_out, t, s))) return cfail(e, "observation");
-    if ((e = gemm(T_, N_, H, n, Dp, w1, Dp, Xs(t), Dp, H1s(t), Hp))) return cfail(e, "policy 1");
-    if ((e = ppo::launch_tanh_fwd(false, H1s(t), Hp, n, H, s))) return cfail(e, "tanh");
-    if ((e = gemm(T_, N_, H, n, Hp, w2, Hp, H1s(t), Hp, H2s(t), Hp))) return cfail(e, "policy 2");
-    if ((e = ppo::launch_tanh_fwd(false, H2s(t), Hp, n, H, s))) return cfail(e, "tanh");
+    if ((e = gemm(T_, N_, H, n, Dp, w1, Dp, Xs(t), Dp, H1s(t), Hp, 0.0f, act)))
+      return cfail(e, "policy 1");
+    if ((e = gemm(T_, N_, H, n, Hp, w2, Hp, H1s(t), Hp, H2s(t), Hp, 0.0f, act)))
+      return cfail(e, "policy 2");
     if ((e = gemm(T_, N_, out, n, Hp, w3, Hp, H2s(t), Hp, Ys(t), kLdy)))
       return cfail(e, "policy 3");
     if ((e = launch_step(M, B, Ys(t), kLdy, t_g0 + (uint64_t)t, rew + (size_t)t * N,
@@ -173,37 +191,40 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
   // ---- terminal critic: lam = coef_V dV(o(x_T))/dx_T ----
   if (value) {
     if ((e = launch_obs(M, B, nullptr, Xs(T), Dp, nullptr, 0, s))) return cfail(e, "observation");
-    if ((e = gemm(T_, N_, H, n, Dp, v1, Dp, Xs(T), Dp, VH1, Hp))) return cfail(e, "value 1");
-    if ((e = ppo::launch_tanh_fwd(false, VH1, Hp, n, H, s))) return cfail(e, "tanh");
-    if ((e = gemm(T_, N_, H, n, Hp, v2, Hp, VH1, Hp, VH2, Hp))) return cfail(e, "value 2");
-    if ((e = ppo::launch_tanh_fwd(false, VH2, Hp, n, H, s))) return cfail(e, "tanh");
+    if ((e = gemm(T_, N_, H, n, Dp, v1, Dp, Xs(T), Dp, VH1, Hp, 0.0f, act))) return cfail(e, "value 1");
+    if ((e = gemm(T_, N_, H, n, Hp, v2, Hp, VH1, Hp, VH2, Hp, 0.0f, act))) return cfail(e, "value 2");
     if ((e = gemm(T_, N_, 1, n, Hp, v3, Hp, VH2, Hp, V, kLdv))) return cfail(e, "value 3");
     if ((e = launch_fill_col(n, gYv, kLdv, coef_V, s))) return cfail(e, "critic seed");
-    if ((e = gemm(N_, N_, H, n, 1, v3, Hp, gYv, kLdv, G, H))) return cfail(e, "value dH2");
-    if ((e = ppo::launch_tanh_bwd(false, G, H, VH2, Hp, n, H, s))) return cfail(e, "tanh'");
-    if ((e = gemm(N_, N_, H, n, H, v2, Hp, G, H, VH2, Hp))) return cfail(e, "value dH1");
-    if ((e = ppo::launch_tanh_bwd(false, VH2, Hp, VH1, Hp, n, H, s))) return cfail(e, "tanh'");
+    if ((e = gemm(N_, N_, H, n, 1, v3, Hp, gYv, kLdv, G2, H, 0.0f, dact(VH2))))
+      return cfail(e, "value dH2");
+    if ((e = gemm(N_, N_, H, n, H, v2, Hp, G2, H, VH2, Hp, 0.0f, dact(VH1))))
+      return cfail(e, "value dH1");
     if ((e = gemm(N_, N_, Dp, n, H, v1, Dp, VH2, Hp, GX, Dp))) return cfail(e, "value dX");
     if ((e = launch_obs_vjp(M, B, nullptr, GX, Dp, lam, s))) return cfail(e, "observation VJP");
   }
   if (J && (e = launch_objective(n, T, rew, coef, value ? V : nullptr, kLdv, coef_V, J, s)))
     return cfail(e, "objective");
   // ---- backward through the window ----
-  for (int t = T - 1; t >= 0; --t) {
-    if ((e = launch_bwd(M, SCs(t), Ys(t), kLdy, done + (size_t)t * N, t_g0 + (uint64_t)t,
-                        coef + t, lam, gY, s)))
-      return cfail(e, "step VJP");
-    if ((e = gemm(N_, T_, Hp, out, n, H2s(t), Hp, gY, kLdy, g3, Hp, 1.0f)))
+  for (int t1 = T; t1 > 0; t1 -= L.G) {
+    const int t0 = std::max(0, t1 - L.G);
+    for (int t = t1 - 1; t >= t0; --t) {
+      const size_t k = (size_t)(t - t0) * N;   // first row of step t in the group's arrays
+      float *g2t = G2 + k * H, *g1t = G1 + k * H, *gyt = gY + k * kLdy;
+      if ((e = launch_bwd(M, SCs(t), Ys(t), kLdy, done + (size_t)t * N, t_g0 + (uint64_t)t, coef + t,
+                          lam, gyt, s)))
+        return cfail(e, "step VJP");
+      if ((e = gemm(N_, N_, H, n, out, w3, Hp, gyt, kLdy, g2t, H, 0.0f, dact(H2s(t)))))
+        return cfail(e, "dH2");
+      if ((e = gemm(N_, N_, H, n, H, w2, Hp, g2t, H, g1t, H, 0.0f, dact(H1s(t)))))
+        return cfail(e, "dH1");
+      if ((e = gemm(N_, N_, Dp, n, H, w1, Dp, g1t, H, GX, Dp))) return cfail(e, "dX");
+      if ((e = launch_obs_vjp(M, B, SCs(t), GX, Dp, lam, s))) return cfail(e, "observation VJP");
+    }
+    const int rows = (t1 - t0) * n;
+    if ((e = gemm(N_, T_, Hp, out, rows, H2s(t0), Hp, gY, kLdy, g3, Hp, 1.0f)))
       return cfail(e, "dW3");
-    if ((e = gemm(N_, N_, H, n, out, w3, Hp, gY, kLdy, G, H))) return cfail(e, "dH2");
-    if ((e = ppo::launch_tanh_bwd(false, G, H, H2s(t), Hp, n, H, s))) return cfail(e, "tanh'");
-    if ((e = gemm(N_, T_, Hp, H, n, H1s(t), Hp, G, H, g2, Hp, 1.0f))) return cfail(e, "dW2");
-    if ((e = gemm(N_, N_, H, n, H, w2, Hp, G, H, H2s(t), Hp))) return cfail(e, "dH1");
-    if ((e = ppo::launch_tanh_bwd(false, H2s(t), Hp, H1s(t), Hp, n, H, s)))
-      return cfail(e, "tanh'");
-    if ((e = gemm(N_, T_, Dp, H, n, Xs(t), Dp, H2s(t), Hp, g1, Dp, 1.0f))) return cfail(e, "dW1");
-    if ((e = gemm(N_, N_, Dp, n, H, w1, Dp, H2s(t), Hp, GX, Dp))) return cfail(e, "dX");
-    if ((e = launch_obs_vjp(M, B, SCs(t), GX, Dp, lam, s))) return cfail(e, "observation VJP");
+    if ((e = gemm(N_, T_, Hp, H, rows, H1s(t0), Hp, G2, H, g2, Hp, 1.0f))) return cfail(e, "dW2");
+    if ((e = gemm(N_, T_, Dp, H, rows, Xs(t0), Dp, G1, H, g1, Dp, 1.0f))) return cfail(e, "dW1");
   }
   if ((e = ppo::launch_convert(grad, gp, D, Dp, H, Hp, out, false, s)))
     return cfail(e, "gradient layout");

@@ -1,7 +1,7 @@
 """The exact-fp32 network kernels (csrc/k_fp32.cu) at the edges of their tiles.
 
-A rollout's tile holds 8, 16 or 32 envs depending on the batch (8 and 16 rows
-per SM are the lines), with sums in one order whatever the tile: envs of a
+A rollout's tile holds 8, 16 or 32 envs depending on the batch (8, 16 and 32
+rows per SM are the lines), with sums in one order whatever the tile: envs of a
 small batch must equal the same envs of a large one bit for bit, and the
 oracle's trajectory within the fp32 tolerance of the other rollout tests
 (1e-5 relative of max(|x|, 1): 32-bit rounding over a few steps).
@@ -33,7 +33,7 @@ def test_rollout_tiles(model, heads, hidden):
     from paper_2512_13359_gb300 import workloads as W
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     T, ref = 4, None
-    for n in (1, 9, 8 * sms + 1, 16 * sms + 1):   # one lane; a ragged 8-tile; ragged 16- and 32-tiles
+    for n in (1, 9, 8 * sms + 1, 16 * sms + 1, 32 * sms + 1):   # one lane; ragged 8-, 16- and 32-tiles, one and two CTAs an SM
         w, pw, vw, env = make(auvenv, W, model, hidden, n, heads)
         traj = env.alloc_traj(T)
         env.rollout(T, traj)

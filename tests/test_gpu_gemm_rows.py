@@ -1,0 +1,65 @@
+"""auv_gemm where its dispatch changes kernels: products over many rows with a short contraction (at least 8 row
+tiles of 128 and at most 9 K-chunks of 128 bytes), fp32 results stored as boxes where rows and N are whole 16-byte pieces, and tf32
+operands read along their samples, in place or, when their rows do not start on 16 bytes, through a copy.
+
+Against float64 of the same operands; tolerances as in test_gpu_gemm.py, as a fraction of sum_k |A(m,k) B(n,k)|:
+fp32 sums of exact bf16 products 1e-5, tf32 operands rounded to nearest (2^-11 each) 3e-3, bf16 results half an ulp."""
+import pytest
+
+from parity_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+TOL = {"bf16": 1e-5, "tf32": 3e-3}
+
+
+def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=3):
+    from paper_2512_13359_gb300 import auvenv
+    g = torch.Generator(device="cuda").manual_seed(M + 3 * N + 7 * K)
+    dt = torch.bfloat16 if prec == "bf16" else torch.float32
+
+    def operand(rows, mn, pad):
+        inner, outer = (rows, K) if mn else (K, rows)
+        align = 8 if prec == "bf16" else 4
+        ld = -(-inner // align) * align + pad
+        t = torch.randn((outer, ld), generator=g, device="cuda").to(dt)
+        v = t[:, :inner].double()
+        return t, ld, v.T if mn else v
+
+    A, lda, a = operand(M, a_mn, pad_a)
+    B, ldb, b = operand(N, b_mn, pad_b)
+    C = torch.full((M, N + pad_c), 7.0, device="cuda", dtype=torch.bfloat16 if c_bf16 else torch.float32)
+    ws = torch.empty(auvenv.lib().auv_gemm_workspace_bytes(M, N, K) // 4 + 1, device="cuda")
+    st = auvenv.gemm(prec, M, N, K, A, lda, a_mn, B, ldb, b_mn, C, N + pad_c, 0.0, ws)
+    ref, scale = a @ b.T, a.abs() @ b.abs().T
+    tol = TOL[prec] * scale + 1e-30 + (2.0 ** -8 * ref.abs() if c_bf16 else 0.0)
+    assert st.cpu().tolist() == [0, 0, 0, 0]
+    assert bool(((C[:, :N].double() - ref).abs() <= tol).all())
+    assert bool((C[:, N:] == 7.0).all())
+
+
+@pytest.mark.parametrize("prec", ["bf16", "tf32"])
+@pytest.mark.parametrize("M,N,K,b_mn", [
+    (1023, 256, 264, False), (1024, 256, 264, False), (1025, 129, 17, True),   # the row line; two 128-wide tiles
+    (2000, 64, 288, False), (2000, 64, 289, False), (2000, 64, 576, True), (2000, 64, 577, True),  # chunk lines
+    (1100, 8, 1, True)])
+def test_short_contractions(prec, M, N, K, b_mn):
+    run(need_gpu(), prec, M, N, K, False, b_mn)
+    run(need_gpu(), prec, M, N, K, False, b_mn, pad_c=4 + -N % 4)   # 16-byte rows: results stored as boxes
+
+
+@pytest.mark.parametrize("prec,c_bf16", [("bf16", True), ("bf16", False), ("tf32", False)])
+@pytest.mark.parametrize("b_mn", [False, True])
+def test_wide_tiles(prec, c_bf16, b_mn):
+    torch = need_gpu()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for rows in (128 * (sms // 2), 128 * (sms // 2) + 1, 128 * 2 * sms + 5):
+        run(torch, prec, rows, 250, 40, False, b_mn, c_bf16)
+        run(torch, prec, rows, 252, 40, False, b_mn, c_bf16, pad_c=4)
+
+
+@pytest.mark.parametrize("M,N,K", [(256, 264, 5000), (16, 264, 32 * 9 + 1), (130, 24, 33), (1, 1, 1), (33, 290, 700)])
+@pytest.mark.parametrize("pad_a,pad_b", [(0, 0), (1, 0), (0, 2), (3, 1)])
+def test_tf32_along_samples(M, N, K, pad_a, pad_b):
+    run(need_gpu(), "tf32", M, N, K, True, True, False, pad_a, pad_b)
+    run(need_gpu(), "tf32", M, N, K, False, True, False, 0, pad_b)
+    run(need_gpu(), "tf32", M, N, K, True, False, False, pad_a, 0)
