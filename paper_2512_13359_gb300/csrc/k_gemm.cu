@@ -23,8 +23,8 @@
 //    MN-major operands only with the 128-byte swizzle of 32-byte pieces
 //    (4 K rows, 512 bytes, a group): its tensor maps use that swizzle.
 //
-// fp32 operands without tensor cores (the exact mode): a register-blocked CUDA-core
-// kernel with the same operand layouts and the same split-K.
+// fp32 operands without tensor cores (the exact mode): register-blocked CUDA-core
+// kernels with the same operand layouts and the same split-K.
 //
 // Split-K: partial tiles go to ws[z][M_pad][N_pad] (fp32); k_reduce adds
 // them in a fixed order (eight interleaved partial sums over z, then those
@@ -736,108 +736,315 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   }
 }
 
-// fp32 CUDA-core GEMM: a BM x 128 tile of C per CTA (BM = 128, or 32 for
-// the few-row weight gradients of the output layers), 256 threads as 16 x 16
-// with BM/16 x 8 outputs each (BM = 128: rows ty*4 .. +3 and 64 + ty*4 .. +3,
-// columns likewise, so shared-memory reads are float4; BM = 32: rows ty*2,
-// ty*2 + 1), K in slices of 8 through double-buffered shared memory that
-// holds both operands M/N-fastest (As[k][m], Bs[k][n]) whichever way they
-// are stored.  Rows are padded by 4 floats: the K-major loads' stores (8 k of
-// 4 rows per warp) then land in 32 distinct banks, and row starts stay
-// 16-byte aligned.
-template <int BM, bool A_MN, bool B_MN>
-__global__ void __launch_bounds__(256, 2)
-k_gemm_fp32(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B,
-            int ldb, int chunks_per_split, void* C, int ldc, float beta, float* ws, int m_pad,
-            int n_pad, int epi, const float* __restrict__ aux, int ld_aux) {
-  constexpr int RM = BM / 16, QA = BM / 32;
-  __shared__ __align__(16) float As[2][8][BM + 4];
-  __shared__ __align__(16) float Bs[2][8][132];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * 128;
-  const int k_begin = blockIdx.z * chunks_per_split * 8;
-  const int k_end = min(K, k_begin + chunks_per_split * 8);
-  // element e of a ROWS x 8 slice: (row, k) with consecutive threads along
-  // the stored-contiguous index
-  auto coord = [](int e, int rows, bool mn, int& r, int& kk) {
-    if (mn) { kk = e / rows; r = e % rows; } else { r = e >> 3; kk = e & 7; }
-  };
-  auto load = [&](const float* X, int ld, bool mn, int rows, int r0, int R, int kb, float* v, int q_n) {
+// ---------------------------------------------------------------------------
+// fp32 on the CUDA cores.  Every output is a chain of FMAs in k, or, where K is
+// split, such a chain per split, the splits' sums added in order: the same
+// bits whichever kernel runs (a closed loop amplifies a changed rounding).
+//
+// Slices of 16 k are copied to shared memory as they are stored (cp.async, 16
+// bytes where rows allow it): K-major operands as [row][16] padded to 20
+// floats, read four k at a time, MN-major ones as [k][row], read four rows at
+// a time; both without bank conflicts.
+// ---------------------------------------------------------------------------
+constexpr int kSl = 16, kSlPad = kSl + 4;
+
+struct F32Args {
+  int M, N, K;
+  const float *A, *B;
+  int lda, ldb;
+  int seg;                // k per split (a multiple of 8)
+  float* C;
+  int ldc;
+  float beta;
+  float* ws;              // split partials, or null (write C)
+  int m_pad, n_pad;
+  int epi;
+  const float* aux;
+  int ld_aux;
+};
+
+__device__ __forceinline__ void cp_async(float* dst, const float* src, int bytes, bool vec) {
+  const uint32_t d = tc::smem_u32(dst);
+  if (vec)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+
+// Copies of rows r0 .. r0 + ROWS - 1 (below R) of an operand, 16 k at a time
+// from k_begin (below k_end), into shared memory by NT threads; absent
+// elements become zero.  A thread's addresses are worked out once.
+template <int ROWS, bool MN, bool VEC, int NT>
+struct F32Loader {
+  static constexpr int W = VEC ? 4 : 1, kItems = ROWS * kSl / W, kPer = (kItems + NT - 1) / NT;
+  const float* src[kPer];
+  int off[kPer], kk[kPer], rows[kPer];   // shared-memory offset, k in the slice, rows below R
+  size_t step;
+  int k_end;
+
+  __device__ __forceinline__ void init(const float* X, int ld, int r0, int R, int k_begin, int k_end_, int t) {
+    k_end = k_end_;
+    step = MN ? (size_t)kSl * ld : kSl;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (q >= q_n) break;
-      int r, kk;
-      coord(tid + 256 * q, rows, mn, r, kk);
-      const int rr = r0 + r, k = kb + kk;
-      v[q] = (rr < R && k < k_end) ? (mn ? X[(size_t)k * ld + rr] : X[(size_t)rr * ld + k]) : 0.0f;
-    }
-  };
-  auto store = [&](float* S, int stride, bool mn, int rows, const float* v, int q_n) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (q >= q_n) break;
-      int r, kk;
-      coord(tid + 256 * q, rows, mn, r, kk);
-      S[kk * stride + r] = v[q];
-    }
-  };
-  float acc[RM][8] = {};
-  float va[4], vb[4];
-  int buf = 0;
-  if (k_begin < k_end) {
-    load(A, lda, A_MN, BM, m0, M, k_begin, va, QA);
-    load(B, ldb, B_MN, 128, n0, N, k_begin, vb, 4);
-    store(&As[0][0][0], BM + 4, A_MN, BM, va, QA);
-    store(&Bs[0][0][0], 132, B_MN, 128, vb, 4);
-  }
-  __syncthreads();
-  for (int kb = k_begin; kb < k_end; kb += 8) {
-    const bool more = kb + 8 < k_end;
-    if (more) {                                   // next slice in flight during this one
-      load(A, lda, A_MN, BM, m0, M, kb + 8, va, QA);
-      load(B, ldb, B_MN, 128, n0, N, kb + 8, vb, 4);
-    }
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      float a[RM];
-      if constexpr (BM == 128) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + ty * 4]);
-        a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-        a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
+    for (int i = 0; i < kPer; ++i) {
+      const int e = i * NT + t;
+      int r;
+      if (MN) {
+        kk[i] = e / (ROWS / W);
+        r = e % (ROWS / W) * W;
+        off[i] = kk[i] * (ROWS + 4) + r;
+        rows[i] = min(W, R - r0 - r);
+        src[i] = X + (size_t)(k_begin + kk[i]) * ld + r0 + r;
       } else {
-        const float2 a0 = *reinterpret_cast<const float2*>(&As[buf][kk][ty * 2]);
-        a[0] = a0.x; a[1] = a0.y;
+        r = e / (kSl / W);
+        kk[i] = e % (kSl / W) * W;
+        off[i] = r * kSlPad + kk[i];
+        rows[i] = r0 + r < R ? W : 0;
+        src[i] = X + (size_t)(r0 + r) * ld + k_begin + kk[i];
       }
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + tx * 4]);
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < RM; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      if (kItems % NT != 0 && e >= kItems) rows[i] = -W;   // no such item
     }
-    if (more) {
-      store(&As[buf ^ 1][0][0], BM + 4, A_MN, BM, va, QA);
-      store(&Bs[buf ^ 1][0][0], 132, B_MN, 128, vb, 4);
-    }
-    __syncthreads();
-    buf ^= 1;
   }
+  // The slice from k kb (the next one on every call); X: any address of the operand.
+  __device__ __forceinline__ void fetch(float* dst, const float* X, int kb) {
 #pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int m = m0 + (BM == 128 ? (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4) : ty * 2 + i);
+    for (int i = 0; i < kPer; ++i) {
+      if (kItems % NT == 0 || rows[i] > -W) {
+        int have = rows[i];
+        if (kb + kSl > k_end) have = MN ? (kb + kk[i] < k_end ? have : 0) : min(have, k_end - kb - kk[i]);
+        have = max(have, 0);
+        cp_async(dst + off[i], have ? src[i] : X, 4 * have, VEC);
+      }
+      src[i] += step;
+    }
+  }
+};
+
+template <int ROWS, bool MN>
+constexpr int f32_slice_floats() {
+  return MN ? kSl * (ROWS + 4) : ROWS * kSlPad;
+}
+
+// Rows of one thread: TM of them (4 per group), thread t of T along the tile.
+template <int T, bool MN>
+__device__ __forceinline__ int f32_row(int t, int i) {
+  return MN ? t * 4 + (i & 3) + (i >> 2) * 4 * T : t + T * i;
+}
+
+// acc += over k k0 .. k0 + 7 of a slice (TM x 8 outputs per thread).
+template <int BM, int BN, int TM, bool A_MN, bool B_MN>
+__device__ __forceinline__ void f32_mac8(const float* As, const float* Bs, int k0, int ty, int tx,
+                                         float (&acc)[TM][8]) {
+  constexpr int TY = BM / TM, TX = BN / 8;
+#pragma unroll
+  for (int q = 0; q < 8; q += 4) {
+    float a[TM][4];
+    if (A_MN) {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+        for (int g = 0; g < TM / 4; ++g) {
+          const float4 v = *reinterpret_cast<const float4*>(As + (k0 + q + kk) * (BM + 4) + ty * 4 + g * 4 * TY);
+          a[4 * g][kk] = v.x;
+          a[4 * g + 1][kk] = v.y;
+          a[4 * g + 2][kk] = v.z;
+          a[4 * g + 3][kk] = v.w;
+        }
+    } else {
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(As + (ty + TY * i) * kSlPad + k0 + q);
+        a[i][0] = v.x;
+        a[i][1] = v.y;
+        a[i][2] = v.z;
+        a[i][3] = v.w;
+      }
+    }
+    if (B_MN) {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const float* row = Bs + (k0 + q + kk) * (BN + 4) + tx * 4;
+        const float4 u = *reinterpret_cast<const float4*>(row);
+        const float4 v = *reinterpret_cast<const float4*>(row + 4 * TX);
+        const float b[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i][kk], b[j], acc[i][j]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 v = *reinterpret_cast<const float4*>(Bs + (tx + TX * j) * kSlPad + k0 + q);
+        const float b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(a[i][kk], b[kk], acc[i][j]);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void f32_store(const F32Args& a, int z, int m, int n, float x) {
+  if (m >= a.M || n >= a.N) return;
+  if (a.ws) {   // partials of the elements the reduction reads
+    a.ws[((size_t)z * a.m_pad + m) * a.n_pad + n] = x;
+    return;
+  }
+  float* c = a.C + (size_t)m * a.ldc + n;
+  const float h = a.epi == kEpiDtanh ? a.aux[(size_t)m * a.ld_aux + n] : 0.0f;
+  *c = a.beta != 0.0f ? fmaf(a.beta, *c, x) : epilogue(a.epi, x, h);
+}
+
+template <int BM, int BN>
+struct F32Tile {
+  static constexpr int TM = BM >= 128 ? 8 : 4;
+  static constexpr int kThreads = (BM / TM) * (BN / 8);
+  static constexpr int kStages = 3;
+  template <bool A_MN, bool B_MN>
+  static constexpr int smem_floats() {
+    return kStages * (f32_slice_floats<BM, A_MN>() + f32_slice_floats<BN, B_MN>());
+  }
+};
+
+// A BM x BN tile per CTA, TM x 8 outputs per thread, three slices in flight.
+// SEG: every split's chain in turn, its sum added to the total (blockIdx.z is
+// 0); else one split per blockIdx.z.  128 x 128 tiles for products that fill
+// the SMs (128 x 96 for 264 columns), 64 x 64 for batches of a few thousand
+// rows, 16 x 128 for the heads' weight gradients.  FMA issue and shared-memory
+// reads bound them (about half of the FP32 peak: 65,536 x 256 x 256 202 us).
+// Against scalar loads through registers: 256 x 264 x 131,072 1,090 -> 590 us,
+// 12 x 264 x 131,072 270 -> 90 us, 4,096 x 256 x 264 (five splits) 27 us and a
+// 14 us reduction -> 26 us.
+template <int BM, int BN, bool A_MN, bool B_MN, bool VEC, bool SEG>
+__global__ void __launch_bounds__((F32Tile<BM, BN>::kThreads), (BM >= 128 ? 2 : 3))
+k_gemm_fp32(const F32Args args) {
+  using TL = F32Tile<BM, BN>;
+  constexpr int TM = TL::TM, TY = BM / TM, TX = BN / 8, NT = TL::kThreads, S = TL::kStages;
+  constexpr int kA = f32_slice_floats<BM, A_MN>(), kB = f32_slice_floats<BN, B_MN>();
+  extern __shared__ __align__(16) float f32_smem[];
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+  const int k_begin = SEG ? 0 : blockIdx.z * args.seg;
+  const int k_end = SEG ? args.K : min(args.K, k_begin + args.seg);
+  F32Loader<BM, A_MN, VEC, NT> load_a;
+  F32Loader<BN, B_MN, VEC, NT> load_b;
+  load_a.init(args.A, args.lda, m0, args.M, k_begin, k_end, tid);
+  load_b.init(args.B, args.ldb, n0, args.N, k_begin, k_end, tid);
+  auto fetch = [&](int kb, int stage) {
+    if (kb < k_end) {
+      float* d = f32_smem + stage * (kA + kB);
+      load_a.fetch(d, args.A, kb);
+      load_b.fetch(d + kA, args.B, kb);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[TM][8] = {}, total[SEG ? TM : 1][SEG ? 8 : 1];
+  int seg_end = args.seg;
+  bool first = true;
+#pragma unroll
+  for (int s = 0; s < S - 1; ++s) fetch(k_begin + s * kSl, s);
+  int stage = 0;
+  for (int kb = k_begin; kb < k_end; kb += kSl) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+    __syncthreads();   // this slice has landed for everyone; the one before is consumed
+    fetch(kb + (S - 1) * kSl, stage == 0 ? S - 1 : stage - 1);
+    const float* As = f32_smem + stage * (kA + kB);
+#pragma unroll
+    for (int k8 = 0; k8 < kSl; k8 += 8) {
+      f32_mac8<BM, BN, TM, A_MN, B_MN>(As, As + kA, k8, ty, tx, acc);
+      if (SEG && kb + k8 + 8 == seg_end) {
+        seg_end += args.seg;
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            total[SEG ? i : 0][SEG ? j : 0] = first ? acc[i][j] : total[SEG ? i : 0][SEG ? j : 0] + acc[i][j];
+            acc[i][j] = 0.0f;
+          }
+        first = false;
+      }
+    }
+    stage = stage + 1 == S ? 0 : stage + 1;
+  }
+  const bool tail = SEG && seg_end - args.seg < args.K;   // the last split ends at K, not at its full length
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const int n = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
-      if (ws) {   // partials of the elements the reduction reads
-        if (m < M && n < N) ws[((size_t)blockIdx.z * m_pad + m) * n_pad + n] = acc[i][j];
-      } else if (m < M && n < N) {
-        float* c = static_cast<float*>(C) + (size_t)m * ldc + n;
-        const float h = epi == kEpiDtanh ? aux[(size_t)m * ld_aux + n] : 0.0f;
-        *c = beta != 0.0f ? fmaf(beta, *c, acc[i][j]) : epilogue(epi, acc[i][j], h);
-      }
+      float x = acc[i][j];
+      if (SEG) x = !tail ? total[SEG ? i : 0][SEG ? j : 0] : (first ? x : total[SEG ? i : 0][SEG ? j : 0] + x);
+      f32_store(args, blockIdx.z, m0 + f32_row<TY, A_MN>(ty, i), n0 + f32_row<TX, B_MN>(tx, j), x);
     }
+}
+
+// Narrow or few tiles: each warp computes a 32 x 32 block over one split with
+// slices of its own (no block-wide barrier in the loop).  WS = 8: the CTA's
+// warps take the splits (at most eight) of one block and add their sums in
+// order; WS = 1 (no split): eight blocks of 32 rows.
+constexpr int kWarpSlice = 2 * 32 * kSlPad;   // A and B slice floats of one warp (MN-major B: 16 x 36 fits)
+constexpr int kWarpStages = 2;
+constexpr int kWarpSmem = 8 * kWarpStages * kWarpSlice * 4;
+
+template <bool B_MN, bool VEC, int WS>
+__global__ void __launch_bounds__(256, 2) k_gemm_fp32_warps(const F32Args args) {
+  static_assert(f32_slice_floats<32, true>() <= 32 * kSlPad, "slice room");
+  extern __shared__ __align__(16) float f32_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 3, ty = lane >> 2;
+  const int m0 = (blockIdx.x * (8 / WS) + (WS == 1 ? warp : 0)) * 32, n0 = blockIdx.y * 32;
+  const int k_begin = WS == 1 ? 0 : warp * args.seg;
+  const int k_end = min(args.K, k_begin + args.seg);
+  float* mine = f32_smem + warp * kWarpStages * kWarpSlice;
+  F32Loader<32, false, VEC, 32> load_a;
+  F32Loader<32, B_MN, VEC, 32> load_b;
+  load_a.init(args.A, args.lda, m0, args.M, k_begin, k_end, lane);
+  load_b.init(args.B, args.ldb, n0, args.N, k_begin, k_end, lane);
+  auto fetch = [&](int kb, int stage) {
+    if (kb < k_end) {
+      float* d = mine + stage * kWarpSlice;
+      load_a.fetch(d, args.A, kb);
+      load_b.fetch(d + 32 * kSlPad, args.B, kb);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[4][8] = {};
+  fetch(k_begin, 0);
+  int stage = 0;
+  for (int kb = k_begin; kb < k_end; kb += kSl) {
+    fetch(kb + kSl, stage ^ 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    const float* As = mine + stage * kWarpSlice;
+    f32_mac8<32, 32, 4, false, B_MN>(As, As + 32 * kSlPad, 0, ty, tx, acc);
+    f32_mac8<32, 32, 4, false, B_MN>(As, As + 32 * kSlPad, 8, ty, tx, acc);
+    __syncwarp();   // the slice is read before the next copy overwrites it
+    stage ^= 1;
+  }
+  if (WS == 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        f32_store(args, 0, m0 + f32_row<8, false>(ty, i), n0 + f32_row<4, B_MN>(tx, j), acc[i][j]);
+    return;
+  }
+  // the splits' sums through shared memory, 33 floats a row, then in order
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  float* part = f32_smem + warp * 32 * 33;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) part[f32_row<8, false>(ty, i) * 33 + f32_row<4, B_MN>(tx, j)] = acc[i][j];
+  __syncthreads();
+  const int splits = (args.K + args.seg - 1) / args.seg;
+#pragma unroll
+  for (int e0 = 0; e0 < 4; ++e0) {
+    const int r = warp + 8 * e0;
+    float x = f32_smem[r * 33 + lane];
+    for (int z = 1; z < splits; ++z) x += f32_smem[(z * 32 + r) * 33 + lane];
+    f32_store(args, 0, m0 + r, n0 + lane, x);
   }
 }
 
@@ -1013,7 +1220,13 @@ struct Plan {
   int m_pad, n_pad;
   bool rows;             // many rows, few K-chunks: k_gemm_rows
   int half;              // its first chunk of the second accumulator, or 0
+  int fp32;              // Fp32Kernel
+  int segments;          // fp32: splits added inside the kernel (1: none)
 };
+
+// fp32 kernels: 128 x 128 tiles (partials in the workspace when split), 64 x
+// 64 tiles, the same with the splits in turn, or a warp per 32 x 32 block.
+enum Fp32Kernel { kFp32Large, kFp32Small, kFp32Seg, kFp32Warps };
 
 constexpr int kRowsMaxChunks = RowTile<true, false, 128>::kMaxChunks;
 
@@ -1024,6 +1237,8 @@ Plan plan(Prec prec, int M, int N, int K, bool a_kmajor) {
   Plan p;
   p.rows = false;
   p.half = 0;
+  p.fp32 = kFp32Large;
+  p.segments = 1;
   if (prec == kFp32) {
     p.bm = M <= 32 ? 32 : 128;
     p.bn = 128;
@@ -1053,6 +1268,19 @@ Plan plan(Prec prec, int M, int N, int K, bool a_kmajor) {
   want = std::max(1, std::min(want, p.chunks / 4));
   p.per_split = (p.chunks + want - 1) / want;
   p.splits = (p.chunks + p.per_split - 1) / p.per_split;
+  if (prec == kFp32 && a_kmajor && p.splits <= 8) {
+    // A product over rows: its few splits are added inside the kernel instead
+    // of through partials in memory (4,096 x 256 x 264, five splits: 27 us and
+    // a 14 us reduction).  A warp per block where the result is narrow or 64 x
+    // 64 tiles would leave SMs idle.
+    const long small = (long)((M + 63) / 64) * ((N + 63) / 64);
+    const int all = sm_count_dev();
+    p.segments = p.splits;
+    if (N <= 32 || (p.splits > 1 && small < all)) p.fp32 = kFp32Warps;
+    else if (p.splits > 1) p.fp32 = kFp32Seg;
+    else if (tiles < 2 * all) p.fp32 = kFp32Small;
+    p.splits = 1;
+  }
   if (p.rows) {   // nine chunks or fewer: at most two splits
     p.half = p.splits > 1 ? p.per_split : 0;
     p.splits = 1;
@@ -1123,6 +1351,51 @@ cudaError_t dispatch_rows(bool b_mn, const Plan& P, const CUtensorMap& ma, const
               : launch_rows<TF32, false, kNarrow>(P, ma, mb, a, s);
 }
 
+template <int BM, int BN, bool A_MN, bool B_MN, bool VEC, bool SEG>
+cudaError_t launch_fp32_tile(const Plan& P, const F32Args& a, cudaStream_t s) {
+  using TL = F32Tile<BM, BN>;
+  auto kern = k_gemm_fp32<BM, BN, A_MN, B_MN, VEC, SEG>;
+  constexpr int smem = TL::template smem_floats<A_MN, B_MN>() * 4;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, SEG ? 1 : P.splits), TL::kThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <bool B_MN, bool VEC>
+cudaError_t launch_fp32_warps(const Plan& P, const F32Args& a, cudaStream_t s) {
+  auto kern = P.segments > 1 ? k_gemm_fp32_warps<B_MN, VEC, 8> : k_gemm_fp32_warps<B_MN, VEC, 1>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kWarpSmem);
+  if (e != cudaSuccess) return e;
+  const int rows = P.segments > 1 ? 32 : 256;
+  kern<<<dim3((a.M + rows - 1) / rows, (a.N + 31) / 32), 256, kWarpSmem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <bool A_MN, bool B_MN, bool VEC>
+cudaError_t launch_fp32_any(const Plan& P, const F32Args& a, cudaStream_t s) {
+  if constexpr (!A_MN) {
+    if (P.fp32 == kFp32Warps) return launch_fp32_warps<B_MN, VEC>(P, a, s);
+    if (P.fp32 == kFp32Seg) return launch_fp32_tile<64, 64, A_MN, B_MN, VEC, true>(P, a, s);
+  }
+  if (a.M <= 16) return launch_fp32_tile<16, 128, A_MN, B_MN, VEC, false>(P, a, s);
+  if (P.fp32 == kFp32Small) return launch_fp32_tile<64, 64, A_MN, B_MN, VEC, false>(P, a, s);
+  // 264 augmented columns: three tiles of 96 instead of three of 128
+  if (a.N > 256 && a.N <= 288) return launch_fp32_tile<128, 96, A_MN, B_MN, VEC, false>(P, a, s);
+  return launch_fp32_tile<128, 128, A_MN, B_MN, VEC, false>(P, a, s);
+}
+
+cudaError_t launch_fp32(const Plan& P, const F32Args& a, bool a_mn, bool b_mn, cudaStream_t s) {
+  // 16-byte copies where every row of both operands starts on 16 bytes
+  const bool vec = ((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B)) & 15u) == 0 &&
+                   a.lda % 4 == 0 && a.ldb % 4 == 0;
+  if (a_mn)
+    return b_mn ? (vec ? launch_fp32_any<true, true, true>(P, a, s) : launch_fp32_any<true, true, false>(P, a, s))
+                : (vec ? launch_fp32_any<true, false, true>(P, a, s) : launch_fp32_any<true, false, false>(P, a, s));
+  return b_mn ? (vec ? launch_fp32_any<false, true, true>(P, a, s) : launch_fp32_any<false, true, false>(P, a, s))
+              : (vec ? launch_fp32_any<false, false, true>(P, a, s) : launch_fp32_any<false, false, false>(P, a, s));
+}
+
 bool tma_ok(const Operand& o, int es) {
   return (reinterpret_cast<uintptr_t>(o.ptr) & 15u) == 0 && ((size_t)o.ld * es) % 16 == 0;
 }
@@ -1181,23 +1454,10 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
   float* part = P.splits > 1 ? ws : nullptr;
   cudaError_t e = cudaSuccess;
   if (prec == kFp32) {
-    const dim3 grid(P.tiles_m, P.tiles_n, P.splits);
-    const float* a = static_cast<const float*>(A.ptr);
-    const float* b = static_cast<const float*>(B.ptr);
-#define AUV_FP32_GEMM(TM, AM, BM)                                                           \
-  k_gemm_fp32<TM, AM, BM><<<grid, 256, 0, s>>>(M, N, K, a, A.ld, b, B.ld, P.per_split, C, ldc, \
-                                               beta, part, P.m_pad, P.n_pad, (int)epi.kind, \
-                                               static_cast<const float*>(epi.aux), epi.ld_aux)
-#define AUV_FP32_MAJOR(TM)                                         \
-  if (A.mn_major && B.mn_major) AUV_FP32_GEMM(TM, true, true);     \
-  else if (A.mn_major) AUV_FP32_GEMM(TM, true, false);             \
-  else if (B.mn_major) AUV_FP32_GEMM(TM, false, true);             \
-  else AUV_FP32_GEMM(TM, false, false)
-    if (P.bm == 32) { AUV_FP32_MAJOR(32); }
-    else { AUV_FP32_MAJOR(128); }
-#undef AUV_FP32_MAJOR
-#undef AUV_FP32_GEMM
-    e = cudaGetLastError();
+    const F32Args a = {M,   N,       K,        static_cast<const float*>(A.ptr), static_cast<const float*>(B.ptr),
+                       A.ld, B.ld,   P.per_split * 8, static_cast<float*>(C), ldc, beta,
+                       part, P.m_pad, P.n_pad, (int)epi.kind, static_cast<const float*>(epi.aux), epi.ld_aux};
+    e = launch_fp32(P, a, A.mn_major, B.mn_major, s);
   } else {
     const bool tf32 = prec == kTf32;
     const int es = tf32 ? 4 : 2;

@@ -1,6 +1,8 @@
 """auv_gemm where its dispatch changes kernels: products over many rows with a short contraction (at least 8 row
 tiles of 128 and at most 9 K-chunks of 128 bytes), fp32 results stored as boxes where rows and N are whole 16-byte pieces, and tf32
-operands read along their samples, in place or, when their rows do not start on 16 bytes, through a copy.
+operands read along their samples, in place or, when their rows do not start on 16 bytes, through a copy; and the fp32
+CUDA-core kernels (a warp per block, splits in turn, 64- and 128-wide tiles, 16-row tiles, partials in memory), with
+16-byte and 4-byte copies.
 
 Against float64 of the same operands; tolerances as in test_gpu_gemm.py, as a fraction of sum_k |A(m,k) B(n,k)|:
 fp32 sums of exact bf16 products 1e-5, tf32 operands rounded to nearest (2^-11 each) 3e-3, bf16 results half an ulp."""
@@ -9,7 +11,7 @@ import pytest
 from parity_util import need_gpu
 
 pytestmark = pytest.mark.gpu
-TOL = {"bf16": 1e-5, "tf32": 3e-3}
+TOL = {"bf16": 1e-5, "tf32": 3e-3, "fp32": 1e-5}
 
 
 def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=3):
@@ -19,7 +21,7 @@ def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=
 
     def operand(rows, mn, pad):
         inner, outer = (rows, K) if mn else (K, rows)
-        align = 8 if prec == "bf16" else 4
+        align = {"bf16": 8, "tf32": 4, "fp32": 4}[prec]
         ld = -(-inner // align) * align + pad
         t = torch.randn((outer, ld), generator=g, device="cuda").to(dt)
         v = t[:, :inner].double()
@@ -63,3 +65,15 @@ def test_tf32_along_samples(M, N, K, pad_a, pad_b):
     run(need_gpu(), "tf32", M, N, K, True, True, False, pad_a, pad_b)
     run(need_gpu(), "tf32", M, N, K, False, True, False, 0, pad_b)
     run(need_gpu(), "tf32", M, N, K, True, False, False, pad_a, 0)
+
+
+@pytest.mark.parametrize("M,N,K,a_mn", [
+    (70, 40, 300, False), (33, 12, 264, False), (1, 1, 9, False),          # a warp per block and split
+    (20011, 24, 256, False), (300, 32, 24, False),                         # a warp per block, no split
+    (4090, 256, 264, False), (2500, 260, 40, False),                       # 64-wide tiles, splits in turn
+    (9800, 256, 24, False), (2003, 250, 17, False), (20000, 250, 264, False),  # 64- and 128-wide tiles
+    (40, 50, 2001, False), (12, 264, 5003, True), (16, 100, 24, True), (260, 264, 3000, True), (50, 24, 33, True)])
+@pytest.mark.parametrize("b_mn", [False, True])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_fp32_kernels(M, N, K, a_mn, b_mn, pad):
+    run(need_gpu(), "fp32", M, N, K, a_mn, b_mn, False, pad, pad)
