@@ -56,5 +56,20 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A, const Opera
                    int ldc, bool c_bf16, float beta, float* ws, size_t ws_bytes, Status* st,
                    cudaStream_t s, const Epilogue& epi = Epilogue());
 
+// Weight gradients of one step in one launch: C_i[M][N] = sum_{k < K} A_i(m, k)
+// B_i(n, k) for up to kMaxGroup items of bf16 operands stored along their
+// samples (MN-major, as TMA reads them), N <= 320, fp32 C.  ws: at least
+// group_workspace_bytes.
+constexpr int kMaxGroup = 6;
+struct GroupItem {
+  int M, N;
+  Operand A, B;
+  float* C;
+  int ldc;
+};
+size_t group_workspace_bytes(const GroupItem* items, int n, int K);
+cudaError_t launch_group(const GroupItem* items, int n, int K, float* ws, size_t ws_bytes, Status* st,
+                         cudaStream_t s);
+
 }  // namespace gemm
 }  // namespace auv

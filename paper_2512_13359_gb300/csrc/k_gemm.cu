@@ -1048,6 +1048,156 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32_warps(const F32Args args) 
   }
 }
 
+// ---------------------------------------------------------------------------
+// A step's weight gradients (bf16, both operands along the samples) in one
+// launch of at most one CTA per SM: each item's row tiles get CTAs in
+// proportion to the bytes a K-chunk of theirs moves, so that all finish
+// together.  They are bound by the reads (426 MB through L2 at 65,536 samples
+// of both networks), which six launches of their own left idle at each start
+// and end: 85 us and 19 us of reductions per step.
+// ---------------------------------------------------------------------------
+struct GroupMaps {
+  CUtensorMap a[kMaxGroup], b[kMaxGroup];
+};
+struct GroupArgs {
+  struct Item {
+    int M, N, splits, per_split, cta0;   // K-chunks per CTA; first CTA
+    float* ws;                           // [splits][M][n_pad]
+    int n_pad;
+    float* C;
+    int ldc;
+  } it[kMaxGroup];
+  int n, chunks;
+  Status* st;
+};
+
+struct GroupTile {
+  static constexpr int kBK = 64;
+  static constexpr uint32_t kBlock = kBK * 128;          // 64 K-rows of 128 bytes
+  static constexpr uint32_t kABytes = 2 * kBlock, kBBytes = 5 * kBlock, kStage = kABytes + kBBytes;
+  static constexpr int kStages = 3;
+  static constexpr uint32_t kSmem = kStages * kStage + 256 + 1024;
+};
+
+__global__ void __launch_bounds__(192, 1)
+k_gemm_group(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupArgs args) {
+  using TL = GroupTile;
+  constexpr int kStages = TL::kStages, kProducer = 4, kIssuer = 5;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~(uintptr_t)1023u);
+  Bars* bar = reinterpret_cast<Bars*>(smem + kStages * TL::kStage);
+  volatile int* abort = &bar->abort;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  int q = 0;
+  while (q + 1 < args.n && (int)blockIdx.x >= args.it[q + 1].cta0) ++q;
+  const GroupArgs::Item& it = args.it[q];
+  const int local = (int)blockIdx.x - it.cta0, z = local % it.splits, m0 = local / it.splits * kBM;
+  const int c0 = z * it.per_split, n_chunks = max(0, min(args.chunks, c0 + it.per_split) - c0);
+
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    tc::mbar_init(&bar->acc_full, 1);
+    bar->abort = 0;
+    tc::mbar_fence_init();
+  }
+  if (warp == kIssuer) {
+    tc::tmem_alloc(&bar->tmem_base, 512);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+
+  if (warp == kProducer) {
+    if ((tid & 31) == 0) {
+      const int na = min(2, (it.M - m0 + 63) / 64), nb = (it.N + 63) / 64;
+      int c = 0;
+      for (; c < n_chunks; ++c) {
+        const int s = c % kStages;
+        if (c >= kStages &&
+            !tc::mbar_wait(&bar->empty[s], (uint32_t)((c / kStages) - 1) & 1u, abort, kWaitLimitNs))
+          break;
+        uint8_t* dst = smem + s * TL::kStage;
+        const int k = (c0 + c) * TL::kBK;
+        tc::mbar_arrive_expect_tx(&bar->full[s], (na + nb) * TL::kBlock);
+        for (int j = 0; j < na; ++j)
+          tma_load_2d(dst + j * TL::kBlock, &maps.a[q], m0 + 64 * j, k, &bar->full[s]);
+        for (int j = 0; j < nb; ++j)
+          tma_load_2d(dst + TL::kABytes + j * TL::kBlock, &maps.b[q], 64 * j, k, &bar->full[s]);
+      }
+      if (*abort)   // the copies still in flight
+        for (int s = 0; s < kStages; ++s) {
+          const int fills = c / kStages + (s < c % kStages ? 1 : 0);
+          if (fills > 0) wait_landed(&bar->full[s], (uint32_t)(fills - 1) & 1u);
+        }
+    }
+    __syncwarp();
+  } else if (warp == kIssuer) {
+    if ((tid & 31) == 0) {
+      // columns in one MMA of up to 256, the rest in a second
+      const uint32_t id1 = idesc(false, true, true, kBM, min(256, (it.N + 15) / 16 * 16));
+      const uint32_t id2 = idesc(false, true, true, kBM, max(16, (it.N - 256 + 15) / 16 * 16));
+      const uint32_t base = tc::smem_u32(smem);
+      bool ok = true;
+      for (int c = 0; c < n_chunks && ok; ++c) {
+        const int s = c % kStages;
+        ok = tc::mbar_wait(&bar->full[s], (uint32_t)(c / kStages) & 1u, abort, kWaitLimitNs);
+        if (!ok) break;
+        tc::tc_fence_after();
+        const uint32_t a0 = base + s * TL::kStage, b0 = a0 + TL::kABytes;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const uint32_t acc = c > 0 || kk > 0 ? 1u : 0u;
+          const uint64_t da = desc_sw128(a0 + kk * 2048, TL::kBlock, 1024);
+          mma<false>(tmem, da, desc_sw128(b0 + kk * 2048, TL::kBlock, 1024), id1, acc);
+          if (it.N > 256)
+            mma<false>(tmem + 256, da, desc_sw128(b0 + 4 * TL::kBlock + kk * 2048, TL::kBlock, 1024), id2,
+                       acc);
+        }
+        tc::mma_commit(&bar->empty[s]);
+      }
+      tc::mma_commit(&bar->acc_full);
+      wait_landed(&bar->acc_full, 0);   // tensor memory is freed below
+    }
+    __syncwarp();
+  } else {
+    const bool ok = n_chunks > 0 && tc::mbar_wait(&bar->acc_full, 0, abort, kWaitLimitNs);
+    tc::tc_fence_after();
+    const int row = m0 + tid;
+    const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+    for (int nb = 0; nb < it.N; nb += 32) {
+      uint32_t acc[32];
+      tc::tmem_ld32(lane_addr + nb, acc);
+      tc::tmem_ld_wait(acc);
+      if (!ok) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = 0u;   // no K in range (or a timed-out wait)
+      }
+      if (row < it.M) {
+        float* dst = it.ws + ((size_t)z * it.M + row) * it.n_pad + nb;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) st_f32x8(dst + 8 * j, acc + 8 * j);
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && bar->abort) {
+    atomicAdd(&args.st->timeouts, 1);
+    atomicCAS(&args.st->code, 0, -4);
+  }
+  if (warp == kIssuer) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 512);
+  }
+}
+
 // C = beta C + sum_z ws[z], fp32 or bf16 output.  A weight gradient has a
 // few tens of thousands of elements and tens of splits, so one thread per
 // element summing every split in turn left the kernel bound by load latency
@@ -1058,13 +1208,14 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32_warps(const F32Args args) 
 // the order g = 0..7: a fixed order, the same on every run.
 constexpr int kRedGroups = 8;
 constexpr int kRedQuads = 32;
-__global__ void __launch_bounds__(kRedGroups * kRedQuads)
-k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int n_pad, void* C,
-         int ldc, int c_bf16, float beta, int epi, const void* __restrict__ aux, int ld_aux) {
+__device__ __forceinline__ void reduce_block(long block, int M, int N, int splits,
+                                             const float* __restrict__ ws, int m_pad, int n_pad, void* C,
+                                             int ldc, int c_bf16, float beta, int epi,
+                                             const void* __restrict__ aux, int ld_aux) {
   __shared__ float4 part[kRedGroups][kRedQuads];
   const int lane = threadIdx.x % kRedQuads, grp = threadIdx.x / kRedQuads;
-  const int qpr = (N + 3) / 4;   // groups of four per row (n_pad is a multiple of 128)
-  const long quad = (long)blockIdx.x * kRedQuads + lane;
+  const int qpr = (N + 3) / 4;   // groups of four per row (n_pad is a multiple of 32)
+  const long quad = block * kRedQuads + lane;
   const bool live = quad < (long)M * qpr;
   const int m = live ? (int)(quad / qpr) : 0, n = live ? (int)(quad % qpr) * 4 : 0;
   const size_t zs = (size_t)m_pad * n_pad;
@@ -1124,6 +1275,21 @@ k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int 
       *c = beta != 0.0f ? fmaf(beta, *c, x) : x;
     }
   }
+}
+
+__global__ void __launch_bounds__(kRedGroups * kRedQuads)
+k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int n_pad, void* C,
+         int ldc, int c_bf16, float beta, int epi, const void* __restrict__ aux, int ld_aux) {
+  reduce_block(blockIdx.x, M, N, splits, ws, m_pad, n_pad, C, ldc, c_bf16, beta, epi, aux, ld_aux);
+}
+
+// Every item of a group (blockIdx.y).
+__global__ void __launch_bounds__(kRedGroups * kRedQuads)
+k_reduce_group(const __grid_constant__ GroupArgs args) {
+  const GroupArgs::Item& it = args.it[blockIdx.y];
+  if ((long)blockIdx.x * kRedQuads >= (long)it.M * ((it.N + 3) / 4)) return;
+  reduce_block(blockIdx.x, it.M, it.N, it.splits, it.ws, it.M, it.n_pad, it.C, it.ldc, 0, 0.0f, kEpiNone,
+               nullptr, 0);
 }
 
 // An MN-major fp32 operand (element (r, k) at k * ld + r) copied K-major:
@@ -1498,6 +1664,82 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
   k_reduce<<<(unsigned)((quads + kRedQuads - 1) / kRedQuads), kRedGroups * kRedQuads, 0, s>>>(
       M, N, P.splits, part, P.m_pad, P.n_pad, C, ldc, c_bf16 ? 1 : 0, beta, (int)epi.kind, epi.aux,
       epi.ld_aux);
+  return cudaGetLastError();
+}
+
+namespace {
+
+// CTAs, K ranges and partials (floats of workspace) of a group.
+void plan_group(const GroupItem* items, int n, int K, GroupArgs* g, size_t* floats) {
+  const int sms = sm_count_dev();
+  g->n = n;
+  g->chunks = (K + GroupTile::kBK - 1) / GroupTile::kBK;
+  auto cost = [](const GroupItem& i) {   // 64-column blocks per K-chunk of a row tile
+    return std::min(2, (i.M + 63) / 64) + (i.N + 63) / 64;
+  };
+  long total = 0;
+  for (int k = 0; k < n; ++k) total += (long)cost(items[k]) * ((items[k].M + kBM - 1) / kBM);
+  int cta = 0;
+  *floats = 0;
+  for (int k = 0; k < n; ++k) {
+    GroupArgs::Item& it = g->it[k];
+    const int tiles = (items[k].M + kBM - 1) / kBM;
+    // at least two chunks per CTA
+    const int want = std::max(1, std::min((int)((long)sms * cost(items[k]) / total), g->chunks / 2));
+    it.M = items[k].M;
+    it.N = items[k].N;
+    it.per_split = (g->chunks + want - 1) / want;
+    it.splits = (g->chunks + it.per_split - 1) / it.per_split;
+    it.cta0 = cta;
+    cta += tiles * it.splits;
+    it.n_pad = (it.N + 31) / 32 * 32;
+    it.C = items[k].C;
+    it.ldc = items[k].ldc;
+    *floats += (size_t)it.splits * it.M * it.n_pad;
+  }
+}
+
+int group_ctas(const GroupArgs& g) {
+  const GroupArgs::Item& last = g.it[g.n - 1];
+  return last.cta0 + (last.M + kBM - 1) / kBM * last.splits;
+}
+
+}  // namespace
+
+size_t group_workspace_bytes(const GroupItem* items, int n, int K) {
+  GroupArgs g;
+  size_t floats = 0;
+  plan_group(items, n, K, &g, &floats);
+  return floats * sizeof(float);
+}
+
+cudaError_t launch_group(const GroupItem* items, int n, int K, float* ws, size_t ws_bytes, Status* st,
+                         cudaStream_t s) {
+  if (n < 1 || n > kMaxGroup || K < 1) return cudaErrorInvalidValue;
+  GroupArgs g;
+  GroupMaps maps;
+  size_t floats = 0;
+  plan_group(items, n, K, &g, &floats);
+  if (!ws || reinterpret_cast<uintptr_t>(ws) % 32 != 0 || ws_bytes < floats * sizeof(float))
+    return cudaErrorInvalidValue;
+  g.st = st;
+  unsigned blocks = 1;
+  for (int k = 0; k < n; ++k) {
+    const GroupItem& i = items[k];
+    if (i.M < 1 || i.N < 1 || i.N > 320 || !i.A.mn_major || !i.B.mn_major || !tma_ok(i.A, 2) ||
+        !tma_ok(i.B, 2) || !make_map(&maps.a[k], false, true, i.A.ptr, i.M, K, i.A.ld, GroupTile::kBK) ||
+        !make_map(&maps.b[k], false, true, i.B.ptr, i.N, K, i.B.ld, GroupTile::kBK))
+      return cudaErrorInvalidValue;
+    g.it[k].ws = ws;
+    ws += (size_t)g.it[k].splits * i.M * g.it[k].n_pad;
+    blocks = std::max(blocks, (unsigned)(((size_t)i.M * ((i.N + 3) / 4) + kRedQuads - 1) / kRedQuads));
+  }
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_group, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       GroupTile::kSmem);
+  if (e != cudaSuccess) return e;
+  k_gemm_group<<<group_ctas(g), 192, GroupTile::kSmem, s>>>(maps, g);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_reduce_group<<<dim3(blocks, n), kRedGroups * kRedQuads, 0, s>>>(g);
   return cudaGetLastError();
 }
 

@@ -264,27 +264,11 @@ int backward(auv_ppo* p, int net, const void* gy, cudaStream_t s) {
   float* g = p->g + net_offset(p, net);
   float *g1 = g, *g2 = g + (size_t)d.H * d.Dp, *g3 = g2 + (size_t)d.H * d.Hp;
   void* gz2 = p->gb[net];
-  void* gz1 = p->h2[net];       // H2 is dead once gZ2 exists
+  void* gz1 = p->h2[net];       // H2 is dead once gZ2 and gW3 exist
   cudaError_t e;
   if ((e = gemm(p, false, true, d.Hp, out, d.B, p->h2[net], d.Ha, gy, ldy, g3, d.Hp,
                  true, s)))
     return cuda_fail(p, e, "gradient W3");
-  if (p->eng) {
-    // gZ2 and gZ1 (into the dead H2) on the tensor-core engine, then the
-    // weight gradients of layers 2 and 1
-    if ((e = auv::launch_learn_backward_bf16(
-             net ? p->img_bv : p->img_bp, out, static_cast<const uint16_t*>(gy), ldy, (size_t)d.B,
-             static_cast<const uint16_t*>(p->h2[net]), static_cast<const uint16_t*>(p->h1[net]), d.Ha,
-             static_cast<uint16_t*>(gz2), d.H, static_cast<uint16_t*>(gz1), d.Ha, p->st, s)))
-      return cuda_fail(p, e, "engine backward");
-    if ((e = gemm(p, false, true, d.Hp, d.H, d.B, p->h1[net], d.Ha, gz2, d.H, g2, d.Hp,
-                   true, s)))
-      return cuda_fail(p, e, "gradient W2");
-    if ((e = gemm(p, false, true, d.Dp, d.H, d.B, p->X, d.Dp, gz1, d.Ha, g1, d.Dp,
-                   true, s)))
-      return cuda_fail(p, e, "gradient W1");
-    return AUV_OK;
-  }
   // input gradients with tanh' in the epilogues (gz1 overwrites H2, which no
   // later product reads)
   const auv::gemm::Epilogue d2 = {auv::gemm::kEpiDtanh, p->h2[net], d.Ha};
@@ -299,6 +283,50 @@ int backward(auv_ppo* p, int net, const void* gy, cudaStream_t s) {
   if ((e = gemm(p, false, true, d.Dp, d.H, d.B, p->X, d.Dp, gz1, d.Ha, g1, d.Dp,
                  true, s)))
     return cuda_fail(p, e, "gradient W1");
+  return AUV_OK;
+}
+
+// Weight gradients of both networks (engine path) as groups of products: the
+// heads', which read H2, or the hidden layers'.
+int weight_items(const auv_ppo* p, bool hidden, auv::gemm::GroupItem* items) {
+  const ppo::Dims& d = p->d;
+  int n = 0;
+  for (int net = d.value_only ? 1 : 0; net < 2; ++net) {
+    float* g = p->g + net_offset(p, net);
+    float *g1 = g, *g2 = g + (size_t)d.H * d.Dp, *g3 = g2 + (size_t)d.H * d.Hp;
+    const void *gy = net ? p->g_v : p->g_y, *gz1 = p->h2[net];
+    if (hidden) {
+      items[n++] = {d.H, d.Hp, {p->gb[net], d.H, true}, {p->h1[net], d.Ha, true}, g2, d.Hp};
+      items[n++] = {d.H, d.Dp, {gz1, d.Ha, true}, {p->X, d.Dp, true}, g1, d.Dp};
+    } else {
+      items[n++] = {p->out[net], d.Hp, {gy, ld_head(p, net), true}, {p->h2[net], d.Ha, true}, g3, d.Hp};
+    }
+  }
+  return n;
+}
+
+// The engine path's backward: the heads' weight gradients, gZ2 and gZ1 (over
+// the then dead H2) of each network on the tensor-core engine, and the hidden
+// layers' weight gradients.
+int backward_engine(auv_ppo* p, cudaStream_t s) {
+  const ppo::Dims& d = p->d;
+  auv::gemm::GroupItem items[auv::gemm::kMaxGroup];
+  cudaError_t e;
+  int n = weight_items(p, false, items);
+  if ((e = auv::gemm::launch_group(items, n, d.B, p->gws, p->gws_bytes, p->st, s)))
+    return cuda_fail(p, e, "gradient W3");
+  for (int net = d.value_only ? 1 : 0; net < 2; ++net) {
+    if ((e = auv::launch_learn_backward_bf16(
+             net ? p->img_bv : p->img_bp, p->out[net],
+             static_cast<const uint16_t*>(net ? p->g_v : p->g_y), ld_head(p, net), (size_t)d.B,
+             static_cast<const uint16_t*>(p->h2[net]), static_cast<const uint16_t*>(p->h1[net]), d.Ha,
+             static_cast<uint16_t*>(p->gb[net]), d.H, static_cast<uint16_t*>(p->h2[net]), d.Ha, p->st,
+             s)))
+      return cuda_fail(p, e, "engine backward");
+  }
+  n = weight_items(p, true, items);
+  if ((e = auv::gemm::launch_group(items, n, d.B, p->gws, p->gws_bytes, p->st, s)))
+    return cuda_fail(p, e, "gradients W2, W1");
   return AUV_OK;
 }
 
@@ -346,6 +374,7 @@ int grads_impl(auv_ppo* p, const auv_ppo_batch* b, float* acc, cudaStream_t s) {
   if ((e = ppo::launch_head(d, hp, p->y[0], p->y[1], p->smp, p->g_y, p->g_v, p->head_part, s)))
     return cuda_fail(p, e, "loss head");
   if ((e = ppo::launch_stats(d, hp, p->head_part, p->mb, acc, s))) return cuda_fail(p, e, "statistics");
+  if (p->eng) return backward_engine(p, s);
   if ((!d.value_only && (rc = backward(p, 0, p->g_y, s))) || (rc = backward(p, 1, p->g_v, s)))
     return rc;
   return AUV_OK;
@@ -479,7 +508,14 @@ int ppo_create(const auv_ppo_config* cfg, auv_ppo** out) {
   p->n_aug_all = p->n_aug[0] + p->n_aug[1];
   // the engine's networks: hidden 256, input <= 18, head <= 16 (2A <= 16)
   p->eng = p->bf16 && d.H == 256 && d.D <= auv::kObs && !(cfg->flags & AUV_PPO_GEMM_PATH);
-  const size_t gws_bytes = gemm_workspace(d, p->out);
+  size_t gws_bytes = gemm_workspace(d, p->out);
+  if (p->eng) {
+    auv::gemm::GroupItem items[auv::gemm::kMaxGroup];
+    for (bool hidden : {false, true}) {
+      const int n = weight_items(p, hidden, items);
+      gws_bytes = std::max(gws_bytes, auv::gemm::group_workspace_bytes(items, n, d.B));
+    }
+  }
   // one allocation, 256-byte aligned pieces
   const size_t B = (size_t)d.B, nb = (B + 255) / 256;
   size_t off = 0;
