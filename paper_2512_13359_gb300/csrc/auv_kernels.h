@@ -181,7 +181,6 @@ cudaError_t launch_gather(const Dims& d, const PermKey& k, const StepCtl* ctl, c
                           const float* act, const float* logp, const float* adv,
                           const float* ret, uint32_t N, const Sample& out, void* X,
                           cudaStream_t s);
-cudaError_t launch_step_advance(StepCtl* ctl, cudaStream_t s);
 // Sample-major copy of a batch for the gather: rows of sample_row_floats(D, A)
 // floats (obs, act, logp, adv, ret, zero padding), row r = t N + i; act,
 // logp and adv may be NULL (value-only).  D + A + 3 <= 80.
@@ -189,17 +188,33 @@ int sample_row_floats(int D, int A);
 cudaError_t launch_transpose_batch(int D, int A, uint32_t T, uint32_t N, const float* obs,
                                    const float* act, const float* logp, const float* adv,
                                    const float* ret, float* dst, cudaStream_t s);
-cudaError_t launch_gather_sm(const Dims& d, const PermKey& k, const StepCtl* ctl,
-                             const float* rows, const Sample& out, void* X, cudaStream_t s);
+// What every step of an epoch reads: the permuted row of each position, and
+// per minibatch the advantages' mean and 1 / (deviation + 1e-8).
+struct EpochPrep {
+  uint32_t* rows;   // [n_mb][B]
+  double* part;     // [n_mb][blocks][2]: sums of adv and adv^2
+  double* norm;     // [n_mb][2]
+};
+size_t epoch_prep_bytes(const Dims& d, size_t rows);   // for up to rows / B minibatches
+EpochPrep epoch_prep(const Dims& d, size_t rows, char* mem);
+cudaError_t launch_epoch_prep(const Dims& d, const PermKey& k, uint32_t n_mb, const float* rows,
+                              const EpochPrep& prep, cudaStream_t s);
+// The minibatch of step ctl->step from the sample-major copy (advantage
+// statistics: EpochPrep's).
+cudaError_t launch_gather_sm(const Dims& d, const StepCtl* ctl, const float* rows, const EpochPrep& prep,
+                             const Sample& out, void* X, cudaStream_t s);
 // y [B][ld_pol], v [B][ld_val] fp32 head outputs; g_y, g_v the same shapes.
-cudaError_t launch_head(const Dims& d, const LossHp& hp, const float* y, const float* v,
-                        const Sample& smp, void* g_y, void* g_v, float* part, cudaStream_t s);
+// norm: EpochPrep's, or NULL: from smp.adv_part.
+cudaError_t launch_head(const Dims& d, const LossHp& hp, const StepCtl* ctl, const double* norm,
+                        const float* y, const float* v, const Sample& smp, void* g_y, void* g_v, float* part,
+                        cudaStream_t s);
 cudaError_t launch_stats(const Dims& d, const LossHp& hp, const float* part, float* mb,
                          float* acc, cudaStream_t s);
-// wb (bf16 copy of w, may be NULL) is rewritten with the new weights.
+// wb (bf16 copy of w, may be NULL) is rewritten with the new weights; advance:
+// ctl moves on to the next step.
 // part: kNormBlocks + 3 floats (norm partials, then the step's scalars).
 cudaError_t launch_adam(float* w, const float* g, float* m, float* v, size_t n, float* part,
-                        const AdamHp& hp, const StepCtl* ctl, float* mb, float* acc, void* wb,
+                        const AdamHp& hp, StepCtl* ctl, float* mb, float* acc, void* wb, bool advance,
                         cudaStream_t s);
 cudaError_t launch_to_bf16(const float* w, void* wb, size_t n, cudaStream_t s);
 cudaError_t launch_finish(const float* acc, float* out, cudaStream_t s);

@@ -111,56 +111,66 @@ __device__ __forceinline__ uint16_t bf16_bits(float x) {
 // low part follows.  Above every network input width (<= 18).
 constexpr int kBiasCol = 30;
 
+// fp32 weights to pack, element (row, col) of layer l at Wl[row * sl + col], its
+// bias at bl[row * tl]: a flat [W1 | b1 | W2 | b2 | W3 | b3] vector, or the
+// learner's augmented layers, whose bias is a column of each row.
+struct WView {
+  const float *W1, *b1, *W2, *b2, *W3, *b3;
+  int s1, t1, s2, t2, s3, t3;
+};
+__host__ __device__ inline WView flat_view(const float* w, int in_dim, int out_dim) {
+  const float *b1 = w + kH * in_dim, *W2 = b1 + kH, *b2 = W2 + kH * kH, *W3 = b2 + kH;
+  return {w, b1, W2, b2, W3, W3 + out_dim * kH, in_dim, 1, kH, 1, kH, 1};
+}
+__host__ __device__ inline WView aug_view(const float* w, int in_dim, int in_p, int Hp) {
+  const float *W2 = w + kH * in_p, *W3 = W2 + kH * Hp;
+  return {w, w + in_dim, W2, W2 + kH, W3, W3 + kH, in_p, in_p, Hp, Hp, Hp, Hp};
+}
+
 // One thread per 16-byte piece of the W1/W2/W3 regions, then the vectors.
 // in_dim: network input width (18 or 12, <= 32); out_dim: 1 (value) or the
 // policy head width (<= 16; head rows out_dim..15 are packed as zeros).
-__device__ void pack_piece(const float* __restrict__ w, int in_dim, int out_dim,
+__device__ void pack_piece(const WView& w, int in_dim, int out_dim,
                            uint8_t* __restrict__ img, int piece) {
-  const float* W1 = w;
-  const float* b1 = W1 + kH * in_dim;
-  const float* W2 = b1 + kH;
-  const float* b2 = W2 + kH * kH;
-  const float* W3 = b2 + kH;
-  const float* b3 = W3 + out_dim * kH;
   const bool policy = out_dim > 1;
   const int n_w1 = kH * 4, n_w2 = 4 * kH * 8, n_w3 = policy ? 4 * kHeadOut * 8 : 0;
   uint16_t v[8];
   uint32_t off;
   if (piece < n_w1) {
     const int n = piece >> 2, p = piece & 3, q = p ^ ((n >> 1) & 3);
-    const uint16_t b_hi = bf16_bits(b1[n]);
-    const uint16_t b_lo = bf16_bits(b1[n] - __uint_as_float((uint32_t)b_hi << 16));
+    const uint16_t b_hi = bf16_bits(w.b1[n * w.t1]);
+    const uint16_t b_lo = bf16_bits(w.b1[n * w.t1] - __uint_as_float((uint32_t)b_hi << 16));
     for (int e = 0; e < 8; ++e) {
       const int k = 8 * q + e;
-      v[e] = k < in_dim ? bf16_bits(W1[n * in_dim + k])
+      v[e] = k < in_dim ? bf16_bits(w.W1[n * w.s1 + k])
                         : (k == kBiasCol ? b_hi : (k == kBiasCol + 1 ? b_lo : (uint16_t)0));
     }
     off = kOffW1 + n * 64 + p * 16;
   } else if (piece < n_w1 + n_w2) {
     const int id = piece - n_w1;
     const int a = id / (kH * 8), n = (id / 8) % kH, p = id & 7, q = p ^ (n & 7);
-    for (int e = 0; e < 8; ++e) v[e] = bf16_bits(W2[n * kH + 64 * a + 8 * q + e]);
+    for (int e = 0; e < 8; ++e) v[e] = bf16_bits(w.W2[n * w.s2 + 64 * a + 8 * q + e]);
     off = kOffW2 + a * (kH * 128) + n * 128 + p * 16;
   } else if (piece < n_w1 + n_w2 + n_w3) {
     const int id = piece - n_w1 - n_w2;
     const int a = id / (kHeadOut * 8), n = (id / 8) % kHeadOut, p = id & 7, q = p ^ (n & 7);
     for (int e = 0; e < 8; ++e)
-      v[e] = n < out_dim ? bf16_bits(W3[n * kH + 64 * a + 8 * q + e]) : (uint16_t)0;
+      v[e] = n < out_dim ? bf16_bits(w.W3[n * w.s3 + 64 * a + 8 * q + e]) : (uint16_t)0;
     off = kOffW3 + a * (kHeadOut * 128) + n * 128 + p * 16;
   } else {
     const int id = piece - n_w1 - n_w2 - n_w3;   // vector entries, one float each
     float* f = reinterpret_cast<float*>(img);
     if (policy) {
-      if (id < kH) f[(kOffB1P >> 2) + id] = b1[id];
-      else if (id < 2 * kH) f[(kOffB2P >> 2) + id - kH] = b2[id - kH];
+      if (id < kH) f[(kOffB1P >> 2) + id] = w.b1[id * w.t1];
+      else if (id < 2 * kH) f[(kOffB2P >> 2) + id - kH] = w.b2[(id - kH) * w.t2];
       else if (id < 2 * kH + kHeadOut)
-        f[(kOffB3P >> 2) + id - 2 * kH] = id - 2 * kH < out_dim ? b3[id - 2 * kH] : 0.0f;
+        f[(kOffB3P >> 2) + id - 2 * kH] = id - 2 * kH < out_dim ? w.b3[(id - 2 * kH) * w.t3] : 0.0f;
     } else {
-      if (id < kH) f[(kOffB1V >> 2) + id] = b1[id];
-      else if (id < 2 * kH) f[(kOffB2V >> 2) + id - kH] = b2[id - kH];
+      if (id < kH) f[(kOffB1V >> 2) + id] = w.b1[id * w.t1];
+      else if (id < 2 * kH) f[(kOffB2V >> 2) + id - kH] = w.b2[(id - kH) * w.t2];
       else if (id < 3 * kH)
-        f[(kOffW3V >> 2) + id - 2 * kH] = __uint_as_float((uint32_t)bf16_bits(W3[id - 2 * kH]) << 16);
-      else if (id == 3 * kH) f[kOffB3V >> 2] = b3[0];
+        f[(kOffW3V >> 2) + id - 2 * kH] = __uint_as_float((uint32_t)bf16_bits(w.W3[id - 2 * kH]) << 16);
+      else if (id == 3 * kH) f[kOffB3V >> 2] = w.b3[0];
     }
     return;
   }
@@ -172,13 +182,9 @@ __device__ void pack_piece(const float* __restrict__ w, int in_dim, int out_dim,
   *reinterpret_cast<uint4*>(img + off) = pk;
 }
 
-// Backward image of one network from its flat fp32 weights (the layout of
-// k_pack): one thread per 16-byte piece of the W1 slot (W3^T, K = 32 with the
+// Backward image of one network from its fp32 weights: one thread per 16-byte piece of the W1 slot (W3^T, K = 32 with the
 // columns from out_dim up zero) and of the W2 slot (W2^T).
-__device__ void pack_back_piece(const float* __restrict__ w, int in_dim, int out_dim,
-                                uint8_t* __restrict__ img, int piece) {
-  const float* W2 = w + kH * in_dim + kH;
-  const float* W3 = W2 + kH * kH + kH;
+__device__ void pack_back_piece(const WView& w, int out_dim, uint8_t* __restrict__ img, int piece) {
   const int n_w1 = kH * 4, n_w2 = 4 * kH * 8;
   uint16_t v[8];
   uint32_t off;
@@ -186,13 +192,13 @@ __device__ void pack_back_piece(const float* __restrict__ w, int in_dim, int out
     const int n = piece >> 2, p = piece & 3, q = p ^ ((n >> 1) & 3);
     for (int e = 0; e < 8; ++e) {
       const int k = 8 * q + e;
-      v[e] = k < out_dim ? bf16_bits(W3[k * kH + n]) : (uint16_t)0;
+      v[e] = k < out_dim ? bf16_bits(w.W3[k * w.s3 + n]) : (uint16_t)0;
     }
     off = kOffW1 + n * 64 + p * 16;
   } else if (piece < n_w1 + n_w2) {
     const int id = piece - n_w1;
     const int a = id / (kH * 8), n = (id / 8) % kH, p = id & 7, q = p ^ (n & 7);
-    for (int e = 0; e < 8; ++e) v[e] = bf16_bits(W2[(64 * a + 8 * q + e) * kH + n]);
+    for (int e = 0; e < 8; ++e) v[e] = bf16_bits(w.W2[(64 * a + 8 * q + e) * w.s2 + n]);
     off = kOffW2 + a * (kH * 128) + n * 128 + p * 16;
   } else {
     return;
@@ -214,20 +220,20 @@ constexpr int kBackPieces = kH * 4 + 4 * kH * 8;
 __global__ void k_pack(const float* __restrict__ w, int in_dim, int out_dim,
                        uint8_t* __restrict__ img) {
   const int piece = blockIdx.x * blockDim.x + threadIdx.x;
-  if (piece < (out_dim > 1 ? kPolPieces : kValPieces)) pack_piece(w, in_dim, out_dim, img, piece);
+  if (piece < (out_dim > 1 ? kPolPieces : kValPieces)) pack_piece(flat_view(w, in_dim, out_dim), in_dim, out_dim, img, piece);
 }
 
 __global__ void k_pack_back(const float* __restrict__ w, int in_dim, int out_dim,
                             uint8_t* __restrict__ img) {
   const int piece = blockIdx.x * blockDim.x + threadIdx.x;
-  if (piece < kBackPieces) pack_back_piece(w, in_dim, out_dim, img, piece);
+  if (piece < kBackPieces) pack_back_piece(flat_view(w, in_dim, out_dim), out_dim, img, piece);
 }
 
 // The learner's four images in one launch: blockIdx.y = 0 policy forward,
 // 1 value forward, 2 policy backward, 3 value backward (a NULL weight
 // pointer skips its images).
 struct LearnerImages {
-  const float* w[2];   // flat fp32 weights, policy and value
+  WView w[2];          // fp32 weights, policy and value
   int in_dim, out_dim[2];
   uint8_t* fwd[2];
   uint8_t* back[2];
@@ -235,11 +241,11 @@ struct LearnerImages {
 __global__ void k_pack_learner(const LearnerImages L) {
   const int job = blockIdx.y, net = job & 1;
   const int piece = blockIdx.x * blockDim.x + threadIdx.x;
-  if (!L.w[net]) return;
+  if (!L.w[net].W1) return;
   if (job < 2) {
     if (piece < (net ? kValPieces : kPolPieces)) pack_piece(L.w[net], L.in_dim, L.out_dim[net], L.fwd[net], piece);
   } else if (piece < kBackPieces) {
-    pack_back_piece(L.w[net], L.in_dim, L.out_dim[net], L.back[net], piece);
+    pack_back_piece(L.w[net], L.out_dim[net], L.back[net], piece);
   }
 }
 
@@ -1300,10 +1306,11 @@ cudaError_t launch_pack_back_bf16(int in_dim, int out_dim, const float* w_f32, v
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_learner_bf16(int in_dim, int policy_out, const float* wp_f32,
-                                     const float* wv_f32, void* wp_packed, void* wv_packed,
+cudaError_t launch_pack_learner_bf16(int in_dim, int in_p, int Hp, int policy_out, const float* wp_aug,
+                                     const float* wv_aug, void* wp_packed, void* wv_packed,
                                      void* bp_packed, void* bv_packed, cudaStream_t s) {
-  const LearnerImages L = {{wp_f32, wv_f32},
+  const LearnerImages L = {{wp_aug ? aug_view(wp_aug, in_dim, in_p, Hp) : WView{},
+                            wv_aug ? aug_view(wv_aug, in_dim, in_p, Hp) : WView{}},
                            in_dim,
                            {policy_out, 1},
                            {static_cast<uint8_t*>(wp_packed), static_cast<uint8_t*>(wv_packed)},

@@ -315,8 +315,6 @@ __global__ void __launch_bounds__(256) k_transpose_batch(int D, int A, int Ws, u
   }
 }
 
-// k_gather from the sample-major copy: one row of Ws floats per sample, read
-// in 16-byte pieces.
 // Eight consecutive X values as 16-byte stores (X rows are multiples of 8
 // elements, so every chunk starts on a 16-byte boundary).
 __device__ __forceinline__ void st_act8(__nv_bfloat16* p, const float v[8]) {
@@ -387,97 +385,134 @@ __device__ __forceinline__ void st_head16(float* p, const float v[16]) {
   st_row8(p + 8, w);
 }
 
-// One sample per thread: its whole row (Ws <= W floats) is loaded at once
-// and X is written in chunks of eight with vector stores; W is a
-// compile-time bound on the row, so the row lives in registers.
-template <typename TX, int W>
-__global__ void __launch_bounds__(kT) k_gather_sm(Dims d, PermKey key, const StepCtl* ctl,
-                                                  const float* __restrict__ rows, int Ws,
-                                                  Sample out, TX* __restrict__ X) {
+// The permuted rows of an epoch's first `count` positions, for all its
+// minibatches at once: the permutation is a chain of a few thousand cycles per
+// sample, which a single minibatch's threads left unhidden in every step's
+// gather.  A thread goes on to its next position as soon as its cycle walk
+// ends, so that a warp does not wait for its slowest lane at each (a walk takes
+// one step or two on average, the longest of 32 five).
+__global__ void __launch_bounds__(kT) k_epoch_rows(uint32_t count, PermKey key, uint32_t* __restrict__ rows) {
+  const uint32_t stride = gridDim.x * kT;
+  uint32_t pos = blockIdx.x * kT + threadIdx.x, x = pos;
+  while (pos < count) {
+    x = feistel(x, key);
+    if (x < key.m) {
+      rows[pos] = x;
+      pos += stride;
+      x = pos;
+    }
+  }
+}
+
+// Sums of a minibatch's (mb0 + blockIdx.y) advantages and their squares, in
+// fp64: a block takes kAdvPer samples, several per thread before the block's
+// tree (the GPU's fp64 pipe runs at a 64th of the fp32 rate).
+constexpr int kAdvPer = 8 * kT;
+__global__ void __launch_bounds__(kT) k_adv_sums(int B, uint32_t mb0, const float* __restrict__ rows, int Ws,
+                                                 int adv_at, EpochPrep prep) {
   __shared__ double sh[2 * (kT / 32)];
-  const int b = blockIdx.x * kT + threadIdx.x;
-  const unsigned long long epoch = ctl->epoch0 + ctl->step / ctl->n_mb;
-  const uint32_t start = (ctl->step % ctl->n_mb) * (uint32_t)d.B;
-  key.e0 = (uint32_t)epoch;
-  key.e1 = (uint32_t)(epoch >> 32);
+  const uint32_t mb = mb0 + blockIdx.y;
+  const int b0 = blockIdx.x * kAdvPer + threadIdx.x;
+  float a[kAdvPer / kT];
+#pragma unroll
+  for (int u = 0; u < kAdvPer / kT; ++u) {
+    const int b = b0 + u * kT;
+    a[u] = b < B ? __ldg(rows + (size_t)__ldg(prep.rows + (size_t)mb * (uint32_t)B + b) * Ws + adv_at) : 0.0f;
+  }
   double s[2] = {0.0, 0.0};
-  if (b < d.B) {
-    const uint32_t r = perm_index(start + (uint32_t)b, key);
-    const float4* src = reinterpret_cast<const float4*>(rows + (size_t)r * Ws);
-    float v[W];
 #pragma unroll
-    for (int q = 0; q < W / 4; ++q) {
-      float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (4 * q < Ws) t = __ldg(src + q);
-      v[4 * q] = t.x;
-      v[4 * q + 1] = t.y;
-      v[4 * q + 2] = t.z;
-      v[4 * q + 3] = t.w;
-    }
-    TX* x = X + (size_t)b * d.Dp;
-#pragma unroll
-    for (int c = 0; c < W / 8; ++c) {
-      if (8 * c < d.Dp) {
-        float x8[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int k = 8 * c + j;
-          x8[j] = k < d.D ? v[k] : (k == d.D ? 1.0f : 0.0f);
-        }
-        st_act8(x + 8 * c, x8);
-      }
-    }
-    // the fields after the observation sit at run-time offsets: read them
-    // from the row again (its sectors are in L1 from the loads above), so
-    // that v stays in registers
-    const float* f = rows + (size_t)r * Ws + d.D;
-    if (!d.value_only && d.A == 8) {
-      uint32_t w[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(__ldg(f + j));
-      st_row8(out.act + (size_t)b * 8, w);
-    } else if (!d.value_only) {
-      for (int j = 0; j < d.A; ++j) out.act[(size_t)b * d.A + j] = __ldg(f + j);
-    }
-    const float lp = __ldg(f + d.A), a = __ldg(f + d.A + 1);
-    out.ret[b] = __ldg(f + d.A + 2);
-    if (!d.value_only) {
-      out.logp[b] = lp;
-      out.adv[b] = a;
-      s[0] = a;
-      s[1] = (double)a * a;
-    }
+  for (int u = 0; u < kAdvPer / kT; ++u) {
+    s[0] += a[u];
+    s[1] = fma((double)a[u], (double)a[u], s[1]);
   }
   block_sum<2>(s, sh);
   if (threadIdx.x == 0) {
-    out.adv_part[2 * blockIdx.x] = s[0];
-    out.adv_part[2 * blockIdx.x + 1] = s[1];
+    double* part = prep.part + 2 * ((size_t)mb * gridDim.x + blockIdx.x);
+    part[0] = s[0];
+    part[1] = s[1];
+  }
+}
+
+// Mean and 1 / (deviation + 1e-8) of a minibatch from its blocks' sums, in one
+// order (blockDim.x = kT); written by thread 0.
+__device__ __forceinline__ void adv_norm(const double* part, int n_part, int B, double* sh, double* out) {
+  double s[2] = {0.0, 0.0};
+  for (int k = threadIdx.x; k < n_part; k += kT) {
+    s[0] += part[2 * k];
+    s[1] += part[2 * k + 1];
+  }
+  block_sum<2>(s, sh);
+  if (threadIdx.x == 0) {
+    const double mean = s[0] / B;
+    const double var = fmax((s[1] - s[0] * mean) / (B - 1), 0.0);
+    out[0] = mean;
+    out[1] = 1.0 / (sqrt(var) + 1e-8);
+  }
+}
+
+__global__ void __launch_bounds__(kT) k_adv_norm(int B, int n_part, EpochPrep prep) {
+  __shared__ double sh[2 * (kT / 32)];
+  adv_norm(prep.part + 2 * (size_t)blockIdx.x * n_part, n_part, B, sh, prep.norm + 2 * (size_t)blockIdx.x);
+}
+
+// The minibatch from the sample-major copy: a thread per 32 bytes of a
+// sample's row, its part of X and the fields that lie in it (65,536 samples:
+// 20 us when one thread worked out the permutation and moved a whole row, 6
+// here, and 3 a step for the epoch's preparation).
+template <typename TX>
+__global__ void __launch_bounds__(kT) k_gather_sm(Dims d, const StepCtl* ctl,
+                                                  const float* __restrict__ rows, int Ws,
+                                                  const uint32_t* __restrict__ perm, Sample out,
+                                                  TX* __restrict__ X) {
+  const unsigned nq = (unsigned)Ws / 8, t = blockIdx.x * kT + threadIdx.x;
+  const unsigned b = t / nq, q = t - b * nq;
+  if (b >= (unsigned)d.B) return;
+  const size_t first = (size_t)(ctl->step % ctl->n_mb) * (uint32_t)d.B;
+  const uint32_t r = __ldg(perm + first + b);
+  uint32_t w[8];
+  ld_row8(rows + (size_t)r * Ws + 8 * q, w);
+  float v[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(w[j]);
+  if (8 * (int)q < d.Dp) {
+    float x8[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = 8 * (int)q + j;
+      x8[j] = k < d.D ? v[j] : (k == d.D ? 1.0f : 0.0f);
+    }
+    st_act8(X + (size_t)b * d.Dp + 8 * q, x8);
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = 8 * (int)q + j - d.D;   // field after the observation
+    if (k < 0 || k > d.A + 2) continue;
+    if (k == d.A + 2) out.ret[b] = v[j];
+    else if (d.value_only) continue;
+    else if (k < d.A) out.act[(size_t)b * d.A + k] = v[j];
+    else if (k == d.A) out.logp[b] = v[j];
+    else out.adv[b] = v[j];
   }
 }
 
 // One thread per sample: log-density, ratio, clipped surrogate, value and
 // entropy terms, and dL/d(head) for both networks (already divided by B).
-// Every block first reduces the gather's advantage partial sums, in the same
-// order, so that all blocks normalise with the same mean and deviation.
+// The advantages' mean and deviation come from the epoch's preparation, or
+// every block reduces the gather's partial sums itself, in the same order.
 template <typename TG>
-__global__ void __launch_bounds__(kT) k_head(Dims d, LossHp hp, const float* __restrict__ y,
+__global__ void __launch_bounds__(kT) k_head(Dims d, LossHp hp, const StepCtl* ctl,
+                                             const double* __restrict__ epoch_norm,
+                                             const float* __restrict__ y,
                                              const float* __restrict__ v, Sample smp,
                                              int n_part, TG* __restrict__ g_y,
                                              TG* __restrict__ g_v, float* __restrict__ part) {
   __shared__ double shd[2 * (kT / 32)];
   __shared__ float shf[5 * (kT / 32)];
   __shared__ double norm[2];
-  double s[2] = {0.0, 0.0};
-  for (int k = threadIdx.x; k < n_part; k += kT) {
-    s[0] += smp.adv_part[2 * k];
-    s[1] += smp.adv_part[2 * k + 1];
-  }
-  block_sum<2>(s, shd);
-  if (threadIdx.x == 0) {
-    const double mean = s[0] / d.B;
-    const double var = fmax((s[1] - s[0] * mean) / (d.B - 1), 0.0);
-    norm[0] = mean;
-    norm[1] = 1.0 / (sqrt(var) + 1e-8);
+  if (epoch_norm) {
+    if (threadIdx.x < 2) norm[threadIdx.x] = epoch_norm[2 * (size_t)(ctl->step % ctl->n_mb) + threadIdx.x];
+  } else {
+    adv_norm(smp.adv_part, n_part, d.B, shd, norm);
   }
   __syncthreads();
   const int b = blockIdx.x * kT + threadIdx.x;
@@ -623,7 +658,12 @@ __global__ void __launch_bounds__(kT) k_adam_prep(float* __restrict__ part, Adam
 __global__ void __launch_bounds__(kT) k_adam(float* __restrict__ w, const float* __restrict__ g,
                                              float* __restrict__ m, float* __restrict__ v,
                                              size_t n, const float* __restrict__ part, AdamHp hp,
-                                             __nv_bfloat16* __restrict__ wb) {
+                                             __nv_bfloat16* __restrict__ wb, StepCtl* advance) {
+  // the step is over (k_adam_prep read the control): on to the next
+  if (advance && blockIdx.x == 0 && threadIdx.x == 0) {
+    advance->step += 1u;
+    advance->t += 1ull;
+  }
   const float scale = part[kNormBlocks];
   const float c1 = part[kNormBlocks + 1], c2 = part[kNormBlocks + 2];
   const float ib1 = 1.0f - hp.b1, ib2 = 1.0f - hp.b2;
@@ -643,11 +683,6 @@ __global__ void __launch_bounds__(kT) k_to_bf16(const float* __restrict__ w,
                                                 __nv_bfloat16* __restrict__ wb, size_t n) {
   for (size_t e = blockIdx.x * (size_t)kT + threadIdx.x; e < n; e += (size_t)gridDim.x * kT)
     wb[e] = __float2bfloat16_rn(w[e]);
-}
-
-__global__ void k_step_advance(StepCtl* ctl) {
-  ctl->step += 1u;
-  ctl->t += 1ull;
 }
 
 __global__ void k_finish(const float* __restrict__ acc, float* __restrict__ out) {
@@ -754,38 +789,56 @@ cudaError_t launch_transpose_batch(int D, int A, uint32_t T, uint32_t N, const f
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_sm(const Dims& d, const PermKey& k, const StepCtl* ctl,
-                             const float* rows, const Sample& out, void* X, cudaStream_t s) {
-  const unsigned nb = (d.B + kT - 1) / kT;
-  const int Ws = sample_row_floats(d.D, d.A);
-  if (Ws > kSmMaxW || d.Dp > Ws || d.Dp % 8 != 0 || reinterpret_cast<uintptr_t>(X) % 16 != 0 ||
-      reinterpret_cast<uintptr_t>(rows) % 16 != 0)
-    return cudaErrorInvalidValue;
-  if (d.bf16) {
-    __nv_bfloat16* xb = static_cast<__nv_bfloat16*>(X);
-    if (Ws <= 32) k_gather_sm<__nv_bfloat16, 32><<<nb, kT, 0, s>>>(d, k, ctl, rows, Ws, out, xb);
-    else k_gather_sm<__nv_bfloat16, kSmMaxW><<<nb, kT, 0, s>>>(d, k, ctl, rows, Ws, out, xb);
-  } else {
-    float* xf = static_cast<float*>(X);
-    if (Ws <= 32) k_gather_sm<float, 32><<<nb, kT, 0, s>>>(d, k, ctl, rows, Ws, out, xf);
-    else k_gather_sm<float, kSmMaxW><<<nb, kT, 0, s>>>(d, k, ctl, rows, Ws, out, xf);
+size_t epoch_prep_bytes(const Dims& d, size_t rows) {
+  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kAdvPer - 1) / kAdvPer;
+  return ((rows * 4 + 15) & ~(size_t)15) + n_mb * (nb + 1) * 2 * sizeof(double);
+}
+
+EpochPrep epoch_prep(const Dims& d, size_t rows, char* mem) {
+  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kAdvPer - 1) / kAdvPer;
+  double* part = reinterpret_cast<double*>(mem + ((rows * 4 + 15) & ~(size_t)15));
+  return {reinterpret_cast<uint32_t*>(mem), part, part + 2 * n_mb * nb};
+}
+
+cudaError_t launch_epoch_prep(const Dims& d, const PermKey& k, uint32_t n_mb, const float* rows,
+                              const EpochPrep& prep, cudaStream_t s) {
+  const size_t count = (size_t)n_mb * (size_t)d.B;   // at most T N <= 2^31
+  const size_t blocks = (count / 16 + kT - 1) / kT;  // 16 positions a thread, or more
+  k_epoch_rows<<<(unsigned)(blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks)), kT, 0, s>>>((uint32_t)count, k,
+                                                                                         prep.rows);
+  if (d.value_only) return cudaGetLastError();
+  const unsigned nb = ((unsigned)d.B + kAdvPer - 1) / kAdvPer;
+  for (uint32_t m0 = 0; m0 < n_mb; m0 += 65535u) {   // gridDim.y
+    const uint32_t m = n_mb - m0 < 65535u ? n_mb - m0 : 65535u;
+    k_adv_sums<<<dim3(nb, m), kT, 0, s>>>(d.B, m0, rows, sample_row_floats(d.D, d.A), d.D + d.A + 1, prep);
   }
+  k_adv_norm<<<n_mb, kT, 0, s>>>(d.B, (int)nb, prep);
   return cudaGetLastError();
 }
 
-cudaError_t launch_step_advance(StepCtl* ctl, cudaStream_t s) {
-  k_step_advance<<<1, 1, 0, s>>>(ctl);
+cudaError_t launch_gather_sm(const Dims& d, const StepCtl* ctl, const float* rows, const EpochPrep& prep,
+                             const Sample& out, void* X, cudaStream_t s) {
+  const int Ws = sample_row_floats(d.D, d.A);
+  if (Ws > kSmMaxW || d.Dp > Ws || d.Dp % 8 != 0 || reinterpret_cast<uintptr_t>(X) % 16 != 0)
+    return cudaErrorInvalidValue;
+  const size_t threads = (size_t)d.B * (Ws / 8);
+  const unsigned nb = (unsigned)((threads + kT - 1) / kT);
+  if (d.bf16)
+    k_gather_sm<<<nb, kT, 0, s>>>(d, ctl, rows, Ws, prep.rows, out, static_cast<__nv_bfloat16*>(X));
+  else
+    k_gather_sm<<<nb, kT, 0, s>>>(d, ctl, rows, Ws, prep.rows, out, static_cast<float*>(X));
   return cudaGetLastError();
 }
 
-cudaError_t launch_head(const Dims& d, const LossHp& hp, const float* y, const float* v,
-                        const Sample& smp, void* g_y, void* g_v, float* part, cudaStream_t s) {
+cudaError_t launch_head(const Dims& d, const LossHp& hp, const StepCtl* ctl, const double* norm,
+                        const float* y, const float* v, const Sample& smp, void* g_y, void* g_v, float* part,
+                        cudaStream_t s) {
   const int nb = (d.B + kT - 1) / kT;
   if (d.bf16)
-    k_head<<<nb, kT, 0, s>>>(d, hp, y, v, smp, nb, static_cast<__nv_bfloat16*>(g_y),
+    k_head<<<nb, kT, 0, s>>>(d, hp, ctl, norm, y, v, smp, nb, static_cast<__nv_bfloat16*>(g_y),
                              static_cast<__nv_bfloat16*>(g_v), part);
   else
-    k_head<<<nb, kT, 0, s>>>(d, hp, y, v, smp, nb, static_cast<float*>(g_y),
+    k_head<<<nb, kT, 0, s>>>(d, hp, ctl, norm, y, v, smp, nb, static_cast<float*>(g_y),
                              static_cast<float*>(g_v), part);
   return cudaGetLastError();
 }
@@ -797,11 +850,12 @@ cudaError_t launch_stats(const Dims& d, const LossHp& hp, const float* part, flo
 }
 
 cudaError_t launch_adam(float* w, const float* g, float* m, float* v, size_t n, float* part,
-                        const AdamHp& hp, const StepCtl* ctl, float* mb, float* acc, void* wb,
+                        const AdamHp& hp, StepCtl* ctl, float* mb, float* acc, void* wb, bool advance,
                         cudaStream_t s) {
   k_sumsq<<<kNormBlocks, kT, 0, s>>>(g, n, part);
   k_adam_prep<<<1, kT, 0, s>>>(part, hp, ctl, mb, acc);
-  k_adam<<<grid_for(n), kT, 0, s>>>(w, g, m, v, n, part, hp, static_cast<__nv_bfloat16*>(wb));
+  k_adam<<<grid_for(n), kT, 0, s>>>(w, g, m, v, n, part, hp, static_cast<__nv_bfloat16*>(wb),
+                                    advance ? ctl : nullptr);
   return cudaGetLastError();
 }
 

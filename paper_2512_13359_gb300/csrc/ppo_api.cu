@@ -18,8 +18,9 @@
 // backward buffer G [B][H] and the head output Y [B][ld].  Everything a step
 // touches is resident.  ppo_update adds one separate allocation: a
 // sample-major copy of its batch (rows of round8(D + A + 3) floats), made
-// once per call, from which every step gathers its minibatch; it grows when a
-// larger batch arrives and lives until ppo_destroy.
+// once per call, from which every step gathers its minibatch, with the
+// current epoch's permuted row numbers (4 bytes a row); it grows when a larger
+// batch arrives and lives until ppo_destroy.
 
 #include <algorithm>
 #include <cmath>
@@ -63,15 +64,17 @@ struct auv_ppo {
   size_t gws_bytes;
   // bf16 forward and backward-data on the tensor-core engine: packed images
   // of both networks (forward, and transposed for the backward), rebuilt
-  // from w every step, a flat staging copy and a status block
+  // from w every step, and a status block
   bool eng = false;
   void *img_p = nullptr, *img_v = nullptr, *img_bp = nullptr, *img_bv = nullptr;
-  float* flat_eng = nullptr;
   Status* st = nullptr;
   // sample-major copy of the batch of the current ppo_update (use_sm while
-  // that update's steps are enqueued); the step graph records which copy
+  // that update's steps are enqueued), then the current epoch's permuted row
+  // numbers and each minibatch's advantage mean and 1 / deviation (EpochPrep);
+  // the step graph records which copy
   float* sm_buf = nullptr;
   size_t sm_rows = 0;
+  ppo::EpochPrep prep = {};
   bool use_sm = false;
   const float* graph_sm = nullptr;
   uint64_t t, epoch;
@@ -346,18 +349,17 @@ int grads_impl(auv_ppo* p, const auv_ppo_batch* b, float* acc, cudaStream_t s) {
   const ppo::Dims& d = p->d;
   const uint32_t m = b->T * b->N;
   cudaError_t e =
-      p->use_sm ? ppo::launch_gather_sm(d, perm_key(p, m, 0), p->ctl, p->sm_buf, p->smp, p->X, s)
+      p->use_sm ? ppo::launch_gather_sm(d, p->ctl, p->sm_buf, p->prep, p->smp, p->X, s)
                 : ppo::launch_gather(d, perm_key(p, m, 0), p->ctl, b->obs, b->act, b->logp, b->adv,
                                      b->ret, b->N, p->smp, p->X, s);
   if (e != cudaSuccess) return cuda_fail(p, e, "gather");
   int rc;
   if (p->eng) {
-    // Both networks on the tensor-core engine: flat fp32 weights, packed bf16
-    // images, then one launch per network writing H1, H2 and the head.
-    if ((rc = convert(p, p->flat_eng, p->flat_eng + p->n_flat[0], p->w, false, s))) return rc;
-    if ((e = auv::launch_pack_learner_bf16(d.D, p->out[0], d.value_only ? nullptr : p->flat_eng,
-                                           p->flat_eng + p->n_flat[0], p->img_p, p->img_v,
-                                           p->img_bp, p->img_bv, s)))
+    // Both networks on the tensor-core engine: packed bf16 images, then one
+    // launch per network writing H1, H2 and the head.
+    if ((e = auv::launch_pack_learner_bf16(d.D, d.Dp, d.Hp, p->out[0], d.value_only ? nullptr : p->w,
+                                           p->w + p->n_aug[0], p->img_p, p->img_v, p->img_bp, p->img_bv,
+                                           s)))
       return cuda_fail(p, e, "pack engine weights");
     for (int net = d.value_only ? 1 : 0; net < 2; ++net) {
       if ((e = auv::launch_learn_forward_bf16(net == 0, net ? p->img_v : p->img_p, d.D, p->out[net],
@@ -371,7 +373,8 @@ int grads_impl(auv_ppo* p, const auv_ppo_batch* b, float* acc, cudaStream_t s) {
     return rc;
   }
   const ppo::LossHp hp = loss_hp(p);
-  if ((e = ppo::launch_head(d, hp, p->y[0], p->y[1], p->smp, p->g_y, p->g_v, p->head_part, s)))
+  if ((e = ppo::launch_head(d, hp, p->ctl, p->use_sm ? p->prep.norm : nullptr, p->y[0], p->y[1], p->smp,
+                            p->g_y, p->g_v, p->head_part, s)))
     return cuda_fail(p, e, "loss head");
   if ((e = ppo::launch_stats(d, hp, p->head_part, p->mb, acc, s))) return cuda_fail(p, e, "statistics");
   if (p->eng) return backward_engine(p, s);
@@ -381,7 +384,8 @@ int grads_impl(auv_ppo* p, const auv_ppo_batch* b, float* acc, cudaStream_t s) {
 }
 
 // Adam step t + 1 with t from the step control (the caller advances p->t).
-int apply_impl(auv_ppo* p, float* acc, cudaStream_t s) {
+// advance: the step control moves on to the next step.
+int apply_impl(auv_ppo* p, float* acc, bool advance, cudaStream_t s) {
   const auv_ppo_config& c = p->cfg;
   ppo::AdamHp hp;
   hp.lr = c.lr;
@@ -390,7 +394,7 @@ int apply_impl(auv_ppo* p, float* acc, cudaStream_t s) {
   hp.eps = c.adam_eps;
   hp.max_norm = c.max_grad_norm;
   cudaError_t e = ppo::launch_adam(p->w, p->g, p->m, p->v, p->n_aug_all, p->norm_part, hp, p->ctl,
-                                   p->mb, acc, p->wb, s);
+                                   p->mb, acc, p->wb, advance, s);
   return e == cudaSuccess ? AUV_OK : cuda_fail(p, e, "Adam");
 }
 
@@ -417,8 +421,7 @@ bool capture_step(auv_ppo* p, const auv_ppo_batch* b) {
   if (cudaStreamBeginCapture(p->gstream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
     return false;
   const bool ok = grads_impl(p, b, p->acc, p->gstream) == AUV_OK &&
-                  apply_impl(p, p->acc, p->gstream) == AUV_OK &&
-                  ppo::launch_step_advance(p->ctl, p->gstream) == cudaSuccess;
+                  apply_impl(p, p->acc, true, p->gstream) == AUV_OK;
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(p->gstream, &g);
   bool done = ok && e == cudaSuccess && g &&
@@ -539,7 +542,6 @@ int ppo_create(const auv_ppo_config* cfg, auv_ppo** out) {
                o_iv = take(p->eng ? auv::bf16_value_image_bytes() : 0),
                o_ibp = take(p->eng ? auv::bf16_back_image_bytes() : 0),
                o_ibv = take(p->eng ? auv::bf16_back_image_bytes() : 0),
-               o_fe = take(p->eng ? (p->n_flat[0] + p->n_flat[1]) * 4 : 0),
                o_st = take(sizeof(Status));
   size_t o_h1[2], o_h2[2], o_gb[2], o_y[2];
   for (int k = 0; k < 2; ++k) {
@@ -580,7 +582,6 @@ int ppo_create(const auv_ppo_config* cfg, auv_ppo** out) {
     p->img_v = base + o_iv;
     p->img_bp = base + o_ibp;
     p->img_bv = base + o_ibv;
-    p->flat_eng = reinterpret_cast<float*>(base + o_fe);
   }
   p->st = reinterpret_cast<Status*>(base + o_st);
   for (int k = 0; k < 2; ++k) {
@@ -726,7 +727,7 @@ int ppo_apply(auv_ppo* p, const float* grad, float* stats, void* stream) {
     if ((rc = convert(p, p->flat, p->flat + p->n_flat[0], p->g, true, s))) return rc;
   }
   if ((rc = set_ctl(p, p->epoch, 1u << 31, 0, p->t, s))) return rc;
-  if ((rc = apply_impl(p, nullptr, s))) return rc;
+  if ((rc = apply_impl(p, nullptr, false, s))) return rc;
   p->t += 1;
   if (stats) {
     cudaError_t e = cudaMemcpyAsync(stats + 5, p->mb + 5, 4, cudaMemcpyDeviceToDevice, s);
@@ -783,8 +784,13 @@ int ppo_update(auv_ppo* p, const auv_ppo_batch* batch, uint32_t epochs, uint32_t
     if (p->sm_buf) cudaFree(p->sm_buf);
     p->sm_buf = nullptr;
     p->sm_rows = 0;
-    if (cudaMalloc(&p->sm_buf, rows * ws * sizeof(float)) == cudaSuccess) p->sm_rows = rows;
-    else p->sm_buf = nullptr;
+    const size_t copy = (rows * ws * sizeof(float) + 255) & ~(size_t)255;
+    if (cudaMalloc(&p->sm_buf, copy + ppo::epoch_prep_bytes(p->d, rows)) == cudaSuccess) {
+      p->sm_rows = rows;
+      p->prep = ppo::epoch_prep(p->d, rows, reinterpret_cast<char*>(p->sm_buf) + copy);
+    } else {
+      p->sm_buf = nullptr;
+    }
     cudaGetLastError();
   }
   p->use_sm = p->sm_buf != nullptr;
@@ -816,11 +822,14 @@ int ppo_update(auv_ppo* p, const auv_ppo_batch* batch, uint32_t epochs, uint32_t
                                                      batch->ret, p->sm_buf, r)))
     return cuda_fail(p, e, "sample-major batch copy");
   for (uint64_t k = 0; k < steps; ++k) {
+    if (p->use_sm && k % n_minibatches == 0 &&
+        (e = ppo::launch_epoch_prep(p->d, perm_key(p, (uint32_t)rows, p->epoch + k / n_minibatches), n_minibatches,
+                                    p->sm_buf, p->prep, r)))
+      return cuda_fail(p, e, "epoch permutation");
     if (graph) {
       if ((e = cudaGraphLaunch(p->step_graph, r))) return cuda_fail(p, e, "launch step graph");
     } else {
-      if ((rc = grads_impl(p, batch, p->acc, r)) || (rc = apply_impl(p, p->acc, r))) return rc;
-      if ((e = ppo::launch_step_advance(p->ctl, r))) return cuda_fail(p, e, "advance step");
+      if ((rc = grads_impl(p, batch, p->acc, r)) || (rc = apply_impl(p, p->acc, true, r))) return rc;
     }
   }
   if (stats && (e = ppo::launch_finish(p->acc, stats, r)) != cudaSuccess)
