@@ -309,6 +309,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  pdl_enter();   // after the allocation: the next kernel's may not come first
   const uint32_t tmem = bar->tmem_base;
   const uint32_t s_base = tc::smem_u32(smem);
 
@@ -551,6 +552,7 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  pdl_enter();   // after the allocation: the next kernel's may not come first
   const uint32_t tmem = bar->tmem_base;
 
   if (warp == kProducer) {
@@ -1280,7 +1282,7 @@ __device__ __forceinline__ void reduce_block(long block, int M, int N, int split
 __global__ void __launch_bounds__(kRedGroups * kRedQuads)
 k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int n_pad, void* C,
          int ldc, int c_bf16, float beta, int epi, const void* __restrict__ aux, int ld_aux) {
-  reduce_block(blockIdx.x, M, N, splits, ws, m_pad, n_pad, C, ldc, c_bf16, beta, epi, aux, ld_aux);
+  reduce_block(blockIdx.x + pdl_enter(), M, N, splits, ws, m_pad, n_pad, C, ldc, c_bf16, beta, epi, aux, ld_aux);
 }
 
 // Every item of a group (blockIdx.y).
@@ -1465,8 +1467,7 @@ cudaError_t launch_tc(const Plan& P, const CUtensorMap& ma, const CUtensorMap& m
   auto kern = k_gemm_tc<TF32, A_MN, B_MN, BN>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::kSmem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(P.tiles_m, P.tiles_n, P.splits), 192, TL::kSmem, s>>>(ma, mb, a);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(P.tiles_m, P.tiles_n, P.splits), 192, TL::kSmem, s, ma, mb, a);
 }
 
 template <bool TF32, int BN>
@@ -1502,9 +1503,8 @@ cudaError_t launch_rows(const Plan& P, const CUtensorMap& ma, const CUtensorMap&
   }
   // every column tile on the same number of CTAs, at most kCtas per SM in all
   const int groups = std::max(1, std::min(P.tiles_m, sm_count_dev() * TL::kCtas / P.tiles_n));
-  kern<<<groups * P.tiles_n, TL::kThreads, smem, s>>>(ma, mb, mc, mx, a, P.tiles_m, P.tiles_n, stages,
-                                                      P.half, boxes ? 1 : 0);
-  return cudaGetLastError();
+  return launch_pdl(kern, groups * P.tiles_n, TL::kThreads, smem, s, ma, mb, mc, mx, a, P.tiles_m, P.tiles_n,
+                    stages, P.half, boxes ? 1 : 0);
 }
 
 template <bool TF32>
@@ -1661,10 +1661,9 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
   }
   if (e != cudaSuccess || !part) return e;
   const size_t quads = (size_t)M * ((N + 3) / 4);
-  k_reduce<<<(unsigned)((quads + kRedQuads - 1) / kRedQuads), kRedGroups * kRedQuads, 0, s>>>(
-      M, N, P.splits, part, P.m_pad, P.n_pad, C, ldc, c_bf16 ? 1 : 0, beta, (int)epi.kind, epi.aux,
-      epi.ld_aux);
-  return cudaGetLastError();
+  return launch_pdl(k_reduce, (unsigned)((quads + kRedQuads - 1) / kRedQuads), kRedGroups * kRedQuads, 0, s, M, N,
+                    P.splits, (const float*)part, P.m_pad, P.n_pad, C, ldc, c_bf16 ? 1 : 0, beta, (int)epi.kind,
+                    epi.aux, epi.ld_aux);
 }
 
 namespace {

@@ -77,3 +77,45 @@ def test_tf32_along_samples(M, N, K, pad_a, pad_b):
 @pytest.mark.parametrize("pad", [0, 1])
 def test_fp32_kernels(M, N, K, a_mn, b_mn, pad):
     run(need_gpu(), "fp32", M, N, K, a_mn, b_mn, False, pad, pad)
+
+
+@pytest.mark.parametrize("M", [1024, 5000, 40000])
+def test_products_that_feed_one_another(M):
+    """Launches that overlap the kernel before them: each product reads the
+    last one's result (rows kernel, then a contraction over the samples with
+    split partials and their reduction, whose result is the next product's
+    other operand, in place of one still being read), back to back, one at a
+    time, and replayed from a graph: the same bits."""
+    torch = need_gpu()
+    from paper_2512_13359_gb300 import auvenv
+    H = 256
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x0 = torch.randn((M, H), generator=g, device="cuda")
+    w0 = torch.randn((H, H), generator=g, device="cuda") / 16
+    x, y, w = (torch.empty_like(t) for t in (x0, x0, w0))
+    ws = torch.empty(max(auvenv.lib().auv_gemm_workspace_bytes(m, H, k) for m, k in ((M, H), (H, M))) // 4 + 1,
+                     device="cuda")
+    st = torch.zeros(4, dtype=torch.int32, device="cuda")
+
+    def chain(sync):
+        x.copy_(x0)
+        w.copy_(w0)
+        for _ in range(6):
+            for A, B, C, m, k, mn in ((x, w, y, M, H, False), (y, w, x, M, H, False), (x, y, w, H, M, True)):
+                auvenv.gemm("tf32", m, H, k, A, H, mn, B, H, mn, C, H, 0.0, ws, st)
+                sync()
+            w.mul_(1.0 / w.abs().max() / 16)   # another library's kernel between two of ours
+            sync()
+        return x.clone(), w.clone()
+
+    one = chain(torch.cuda.synchronize)
+    for _ in range(3):
+        assert all(torch.equal(a, b) for a, b in zip(one, chain(lambda: None)))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = chain(lambda: None)
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(one, out))
+    assert st.cpu().tolist() == [0, 0, 0, 0] and bool(torch.isfinite(one[0]).all())
