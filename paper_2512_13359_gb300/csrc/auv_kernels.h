@@ -87,16 +87,18 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
                char* base, uint64_t t_g0, const float* policy, const float* value,
                const float* coef, float coef_V, bool tf32, float* grad, float* J,
                float* obs_out, float* rew_out, uint8_t* done_out, cudaStream_t s, char* err);
+constexpr int kLdy = 16;   // floats of a policy head's row (2 x 8, or 2 x 6 padded)
+
 // obs_fm: optional [T][18][N] output of step t's observation.
-cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X, int ldx,
+cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X,
                        float* obs_fm, int t, cudaStream_t s);
-cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, int ldy, uint64_t t_g,
+cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, uint64_t t_g,
                         float* rew, uint8_t* done, Status* st, cudaStream_t s);
-cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y, int ldy,
+cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y,
                        const uint8_t* done, uint64_t t_g, const float* coef, float* lam,
                        float* gY, cudaStream_t s);
 cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* sc, const float* gX,
-                           int ldx, float* lam, cudaStream_t s);
+                           float* lam, cudaStream_t s);
 cudaError_t launch_objective(int n, int T, const float* rew, const float* coef, const float* V,
                              int ldv, float coef_V, float* J, cudaStream_t s);
 cudaError_t launch_fill_col(int n, float* buf, int ld, float v, cudaStream_t s);

@@ -505,6 +505,31 @@ __device__ __forceinline__ void store_lam(float* __restrict__ lam, size_t n, int
   for (int k = 0; k < 6; ++k) lam[(7 + k) * n + i] = lx.nu[k];
 }
 
+// A thread's row of a network input, head or their gradients, N floats from
+// p on (8, 16 or 24; rows are whole 32-byte sectors): a load or store per
+// sector.  Single floats a row apart cost a sector each: the observations of
+// 65,536 envs took 11.6 us (4.5 now), the step's VJP 18.1 us (15.5).
+template <int N>
+__device__ __forceinline__ void ld_row(const float* p, float* v) {
+#pragma unroll
+  for (int j = 0; j < N; j += 8)
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[j]), "=f"(v[j + 1]), "=f"(v[j + 2]), "=f"(v[j + 3]), "=f"(v[j + 4]), "=f"(v[j + 5]),
+          "=f"(v[j + 6]), "=f"(v[j + 7])
+        : "l"(p + j));
+}
+template <int N>
+__device__ __forceinline__ void st_row(float* p, const float* v) {
+#pragma unroll
+  for (int j = 0; j < N; j += 8)
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p + j), "f"(v[j]), "f"(v[j + 1]),
+                 "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]), "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
+                 : "memory");
+}
+// Floats of an observation's row (the observation, 1, zeros to a sector).
+constexpr int kLdx = (kObs + 8) / 8 * 8, kPaperLdx = (paper::kObs + 8) / 8 * 8;
+using shac::kLdy;
+
 // Reparameterised action a = mu + exp(clamp(ls)) eps from a policy head row.
 __device__ __forceinline__ void shac_action(const Model& M, const float* __restrict__ y,
                                             const float eps[kAct], float a[kAct],
@@ -519,33 +544,32 @@ __device__ __forceinline__ void shac_action(const Model& M, const float* __restr
 }
 
 // Observation row of the network input (augmented: 1 at column kObs, zeros
-// up to ldx) of each env's current state; with sc, also the step's scratch.
+// up to kLdx) of each env's current state; with sc, also the step's scratch.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs(const Model M, Buffers B,
                                                           float* __restrict__ sc,
-                                                          float* __restrict__ X, int ldx,
+                                                          float* __restrict__ X,
                                                           float* __restrict__ obs_fm, int t) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   Env e;
   load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   if (sc) save_step(sc, (size_t)M.n, i, e);
-  float o[kObs];
+  float o[kLdx];
   observe(e, o);
-  float* x = X + (size_t)i * ldx;
+  o[kObs] = 1.0f;
 #pragma unroll
-  for (int k = 0; k < kObs; ++k) x[k] = o[k];
-  x[kObs] = 1.0f;
-  for (int k = kObs + 1; k < ldx; ++k) x[k] = 0.0f;
+  for (int k = kObs + 1; k < kLdx; ++k) o[k] = 0.0f;
+  st_row<kLdx>(X + (size_t)i * kLdx, o);
   if (obs_fm) {
 #pragma unroll
     for (int k = 0; k < kObs; ++k) obs_fm[((size_t)t * kObs + k) * M.n + i] = o[k];
   }
 }
 
-// One closed-loop step from the policy head Y [N][ldy]: action, physics,
+// One closed-loop step from the policy head Y [N][kLdy]: action, physics,
 // episode bookkeeping; the env's buffers are advanced.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_step(const Model M, Buffers B,
-                                                           const float* __restrict__ Y, int ldy,
+                                                           const float* __restrict__ Y,
                                                            uint64_t t_g, float* __restrict__ rew,
                                                            uint8_t* __restrict__ done,
                                                            Status* st) {
@@ -557,7 +581,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step(const Model M, Buffer
   float eps[kAct], a[kAct], sig[kAct];
   bool in[kAct];
   action_noise(id, M.seed, t_g, eps);
-  shac_action(M, Y + (size_t)i * ldy, eps, a, sig, in);
+  float y[kLdy];
+  ld_row<kLdy>(Y + (size_t)i * kLdy, y);
+  shac_action(M, y, eps, a, sig, in);
   bool d;
   const float r = physics_step(M, id, e, a, &d);
   if (!env_finite(e)) flag_nan(st, i);
@@ -568,11 +594,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step(const Model M, Buffer
 
 // Backward of one closed-loop step: lam (dJ/d post-step state, [13][N]) is
 // replaced by dJ/d pre-step state through the physics, and the policy head's
-// gradient is written to gY [N][ldy] (mean, then the log-std head through
+// gradient is written to gY [N][kLdy] (mean, then the log-std head through
 // a = mu + sigma eps; zero where the clamp is active).
 __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
                                                           const float* __restrict__ sc,
-                                                          const float* __restrict__ Y, int ldy,
+                                                          const float* __restrict__ Y,
                                                           const uint8_t* __restrict__ done,
                                                           uint64_t t_g, const float* __restrict__ coef,
                                                           float* __restrict__ lam,
@@ -597,7 +623,9 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
   float eps[kAct], a[kAct], sig[kAct], a_c[kAct], tau[6], nup[6];
   bool in[kAct];
   action_noise(id, M.seed, t_g, eps);
-  shac_action(M, Y + (size_t)i * ldy, eps, a, sig, in);
+  float y[kLdy];
+  ld_row<kLdy>(Y + (size_t)i * kLdy, y);
+  shac_action(M, y, eps, a, sig, in);
   allocate(M, a, a_c, tau);
 #pragma unroll
   for (int k = 0; k < 6; ++k) nup[k] = es.nu[k];
@@ -611,7 +639,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
   for (int s = M.substeps - 1; s >= 0; --s) substep_vjp(M, es, xs[s], tau, lx, ltau);
 #pragma unroll
   for (int k = 0; k < 6; ++k) lx.nu[k] += lnup[k];
-  float* g = gY + (size_t)i * ldy;
+  float g[kLdy];
 #pragma unroll
   for (int k = 0; k < kAct; ++k) {
     float ga = la[k];
@@ -621,15 +649,15 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
     g[k] = ga;
     g[kAct + k] = in[k] ? ga * sig[k] * eps[k] : 0.0f;
   }
+  st_row<kLdy>(gY + (size_t)i * kLdy, g);
   store_lam(lam, n, i, lx);
 }
 
 // lam += (d obs / d state)^T gX at the state of scratch sc (or of the env's
-// buffers when sc is NULL); gX [N][ldx], first kObs columns.
+// buffers when sc is NULL); gX [N][kLdx], first kObs columns.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp(const Model M, Buffers B,
                                                               const float* __restrict__ sc,
-                                                              const float* __restrict__ gX,
-                                                              int ldx, float* __restrict__ lam) {
+                                                              const float* __restrict__ gX, float* __restrict__ lam) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
@@ -639,9 +667,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp(const Model M, Buf
   } else {
     load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   }
-  float lo[kObs];
-#pragma unroll
-  for (int k = 0; k < kObs; ++k) lo[k] = gX[(size_t)i * ldx + k];
+  float lo[kLdx];
+  ld_row<kLdx>(gX + (size_t)i * kLdx, lo);
   X lx;
   load_lam(lam, n, i, lx);
   obs_vjp(e, lo, lx);
@@ -987,11 +1014,11 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_paper_adjoint(
 
 // ---- SHAC in closed loop on the paper model ----
 
-// Observation row (12 + the constant 1, zeros up to ldx) of each env's state;
+// Observation row (12 + the constant 1, zeros up to kPaperLdx) of each env's state;
 // with sc, the step's scratch (its history mean from the env's state rows).
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_paper(const Model M, Buffers B,
                                                                 float* __restrict__ sc,
-                                                                float* __restrict__ X, int ldx,
+                                                                float* __restrict__ X,
                                                                 float* __restrict__ obs_fm,
                                                                 int t) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
@@ -999,13 +1026,12 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_paper(const Model M, B
   paper::Env e;
   paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   if (sc) paper_save_step(M, e, B.state, sc, (size_t)M.n, i);
-  float o[paper::kObs];
+  float o[kPaperLdx];
   paper::observe(e, o);
-  float* x = X + (size_t)i * ldx;
+  o[paper::kObs] = 1.0f;
 #pragma unroll
-  for (int k = 0; k < paper::kObs; ++k) x[k] = o[k];
-  x[paper::kObs] = 1.0f;
-  for (int k = paper::kObs + 1; k < ldx; ++k) x[k] = 0.0f;
+  for (int k = paper::kObs + 1; k < kPaperLdx; ++k) o[k] = 0.0f;
+  st_row<kPaperLdx>(X + (size_t)i * kPaperLdx, o);
   if (obs_fm) {
 #pragma unroll
     for (int k = 0; k < paper::kObs; ++k) obs_fm[((size_t)t * paper::kObs + k) * M.n + i] = o[k];
@@ -1027,8 +1053,7 @@ __device__ __forceinline__ void paper_shac_action(const Model& M, const float* _
 }
 
 __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, Buffers B,
-                                                                 const float* __restrict__ Y,
-                                                                 int ldy, uint64_t t_g,
+                                                                 const float* __restrict__ Y, uint64_t t_g,
                                                                  float* __restrict__ rew,
                                                                  uint8_t* __restrict__ done,
                                                                  Status* st) {
@@ -1040,7 +1065,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, 
   float eps[8], a[paper::kAct], sig[paper::kAct];
   bool in[paper::kAct];
   action_noise(id, M.seed, t_g, eps);
-  paper_shac_action(M, Y + (size_t)i * ldy, eps, a, sig, in);
+  float y[kLdy];
+  ld_row<kLdy>(Y + (size_t)i * kLdy, y);
+  paper_shac_action(M, y, eps, a, sig, in);
   bool d;
   const float r = paper::physics_step(M, id, e, a, paper::hist_rows(B.state, M.n, i), &d);
   if (!paper::env_finite(e)) flag_nan(st, i);
@@ -1052,7 +1079,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, 
 // Backward of one closed-loop paper step: lam [61][N] (rows 0..12 the pose
 // and velocity, 13.. the history) from post- to pre-step, head gradient gY.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
-    const Model M, const float* __restrict__ sc, const float* __restrict__ Y, int ldy,
+    const Model M, const float* __restrict__ sc, const float* __restrict__ Y,
     const uint8_t* __restrict__ done, uint64_t t_g, const float* __restrict__ coef,
     float* __restrict__ lam, float* __restrict__ gY) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
@@ -1074,14 +1101,17 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
   float eps[8], a[paper::kAct], sig[paper::kAct], la[paper::kAct];
   bool in[paper::kAct];
   action_noise(id, M.seed, t_g, eps);
-  paper_shac_action(M, Y + (size_t)i * ldy, eps, a, sig, in);
+  float y[kLdy];
+  ld_row<kLdy>(Y + (size_t)i * kLdy, y);
+  paper_shac_action(M, y, eps, a, sig, in);
   paper_step_vjp(M, sc, n, i, a, __ldg(coef), lx, lh, la);
-  float* g = gY + (size_t)i * ldy;
+  float g[kLdy] = {};
 #pragma unroll
   for (int k = 0; k < paper::kAct; ++k) {
     g[k] = la[k];
     g[paper::kAct + k] = in[k] ? la[k] * sig[k] * eps[k] : 0.0f;
   }
+  st_row<kLdy>(gY + (size_t)i * kLdy, g);
 #pragma unroll
   for (int k = 0; k < 3; ++k) lam[k * n + i] = lx.p[k];
 #pragma unroll
@@ -1096,8 +1126,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
 // lam (rows 0..12) += (d obs / d state)^T gX at the step's input (sc) or at
 // the env's current state (sc NULL).
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp_paper(
-    const Model M, Buffers B, const float* __restrict__ sc, const float* __restrict__ gX,
-    int ldx, float* __restrict__ lam) {
+    const Model M, Buffers B, const float* __restrict__ sc, const float* __restrict__ gX, float* __restrict__ lam) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
@@ -1109,9 +1138,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp_paper(
   } else {
     paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   }
-  float lo[paper::kObs];
-#pragma unroll
-  for (int k = 0; k < paper::kObs; ++k) lo[k] = gX[(size_t)i * ldx + k];
+  float lo[kPaperLdx];
+  ld_row<kPaperLdx>(gX + (size_t)i * kPaperLdx, lo);
   X lx;
   load_lam(lam, n, i, lx);
   paper_obs_vjp(e, lo, lx);
@@ -1131,40 +1159,40 @@ namespace shac {
 
 static unsigned blocks(int n) { return (n + kAdjThreads - 1) / kAdjThreads; }
 
-cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X, int ldx,
+cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X,
                        float* obs_fm, int t, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_obs_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, X, ldx, obs_fm, t);
+    k_shac_obs_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, X, obs_fm, t);
   else
-    k_shac_obs<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, X, ldx, obs_fm, t);
+    k_shac_obs<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, X, obs_fm, t);
   return cudaGetLastError();
 }
 
-cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, int ldy, uint64_t t_g,
+cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, uint64_t t_g,
                         float* rew, uint8_t* done, Status* st, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_step_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, ldy, t_g, rew, done, st);
+    k_shac_step_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st);
   else
-    k_shac_step<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, ldy, t_g, rew, done, st);
+    k_shac_step<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st);
   return cudaGetLastError();
 }
 
-cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y, int ldy,
+cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y,
                        const uint8_t* done, uint64_t t_g, const float* coef, float* lam,
                        float* gY, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_bwd_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, ldy, done, t_g, coef, lam, gY);
+    k_shac_bwd_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY);
   else
-    k_shac_bwd<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, ldy, done, t_g, coef, lam, gY);
+    k_shac_bwd<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY);
   return cudaGetLastError();
 }
 
 cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* sc, const float* gX,
-                           int ldx, float* lam, cudaStream_t s) {
+                           float* lam, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_obs_vjp_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, ldx, lam);
+    k_shac_obs_vjp_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, lam);
   else
-    k_shac_obs_vjp<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, ldx, lam);
+    k_shac_obs_vjp<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, lam);
   return cudaGetLastError();
 }
 

@@ -55,7 +55,6 @@ struct Gemm {
   }
 };
 
-constexpr int kLdy = 16;   // policy head row (2 x 8, or 2 x 6 padded)
 constexpr int kLdv = 8;    // value head row
 
 }  // namespace
@@ -176,21 +175,21 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
 
   // ---- forward ----
   for (int t = 0; t < T; ++t) {
-    if ((e = launch_obs(M, B, SCs(t), Xs(t), Dp, obs_out, t, s))) return cfail(e, "observation");
+    if ((e = launch_obs(M, B, SCs(t), Xs(t), obs_out, t, s))) return cfail(e, "observation");
     if ((e = gemm(T_, N_, H, n, Dp, w1, Dp, Xs(t), Dp, H1s(t), Hp, 0.0f, act)))
       return cfail(e, "policy 1");
     if ((e = gemm(T_, N_, H, n, Hp, w2, Hp, H1s(t), Hp, H2s(t), Hp, 0.0f, act)))
       return cfail(e, "policy 2");
     if ((e = gemm(T_, N_, out, n, Hp, w3, Hp, H2s(t), Hp, Ys(t), kLdy)))
       return cfail(e, "policy 3");
-    if ((e = launch_step(M, B, Ys(t), kLdy, t_g0 + (uint64_t)t, rew + (size_t)t * N,
+    if ((e = launch_step(M, B, Ys(t), t_g0 + (uint64_t)t, rew + (size_t)t * N,
                          done + (size_t)t * N, st, s)))
       return cfail(e, "step");
   }
   if ((e = cudaMemsetAsync(lam, 0, (size_t)L.S * N * 4, s))) return cfail(e, "clear adjoint");
   // ---- terminal critic: lam = coef_V dV(o(x_T))/dx_T ----
   if (value) {
-    if ((e = launch_obs(M, B, nullptr, Xs(T), Dp, nullptr, 0, s))) return cfail(e, "observation");
+    if ((e = launch_obs(M, B, nullptr, Xs(T), nullptr, 0, s))) return cfail(e, "observation");
     if ((e = gemm(T_, N_, H, n, Dp, v1, Dp, Xs(T), Dp, VH1, Hp, 0.0f, act))) return cfail(e, "value 1");
     if ((e = gemm(T_, N_, H, n, Hp, v2, Hp, VH1, Hp, VH2, Hp, 0.0f, act))) return cfail(e, "value 2");
     if ((e = gemm(T_, N_, 1, n, Hp, v3, Hp, VH2, Hp, V, kLdv))) return cfail(e, "value 3");
@@ -200,7 +199,7 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
     if ((e = gemm(N_, N_, H, n, H, v2, Hp, G2, H, VH2, Hp, 0.0f, dact(VH1))))
       return cfail(e, "value dH1");
     if ((e = gemm(N_, N_, Dp, n, H, v1, Dp, VH2, Hp, GX, Dp))) return cfail(e, "value dX");
-    if ((e = launch_obs_vjp(M, B, nullptr, GX, Dp, lam, s))) return cfail(e, "observation VJP");
+    if ((e = launch_obs_vjp(M, B, nullptr, GX, lam, s))) return cfail(e, "observation VJP");
   }
   if (J && (e = launch_objective(n, T, rew, coef, value ? V : nullptr, kLdv, coef_V, J, s)))
     return cfail(e, "objective");
@@ -210,7 +209,7 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
     for (int t = t1 - 1; t >= t0; --t) {
       const size_t k = (size_t)(t - t0) * N;   // first row of step t in the group's arrays
       float *g2t = G2 + k * H, *g1t = G1 + k * H, *gyt = gY + k * kLdy;
-      if ((e = launch_bwd(M, SCs(t), Ys(t), kLdy, done + (size_t)t * N, t_g0 + (uint64_t)t, coef + t,
+      if ((e = launch_bwd(M, SCs(t), Ys(t), done + (size_t)t * N, t_g0 + (uint64_t)t, coef + t,
                           lam, gyt, s)))
         return cfail(e, "step VJP");
       if ((e = gemm(N_, N_, H, n, out, w3, Hp, gyt, kLdy, g2t, H, 0.0f, dact(H2s(t)))))
@@ -218,7 +217,7 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
       if ((e = gemm(N_, N_, H, n, H, w2, Hp, g2t, H, g1t, H, 0.0f, dact(H1s(t)))))
         return cfail(e, "dH1");
       if ((e = gemm(N_, N_, Dp, n, H, w1, Dp, g1t, H, GX, Dp))) return cfail(e, "dX");
-      if ((e = launch_obs_vjp(M, B, SCs(t), GX, Dp, lam, s))) return cfail(e, "observation VJP");
+      if ((e = launch_obs_vjp(M, B, SCs(t), GX, lam, s))) return cfail(e, "observation VJP");
     }
     const int rows = (t1 - t0) * n;
     if ((e = gemm(N_, T_, Hp, out, rows, H2s(t0), Hp, gY, kLdy, g3, Hp, 1.0f)))
