@@ -912,9 +912,9 @@ def run_shac(args):
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak, "traffic": None, "peak_source": psrc,
                      "flops_per_env_step": fps},
-        # per step 5 launches forward and 5 backward; 13 around them; the three weight gradients of
+        # per step 4 launches forward and 4 backward; 12 around them; the three weight gradients of
         # each group of steps (1 GiB of layer gradients) with their reductions
-        "gpu_launches": args.steps * (10 * T + 13 + 6 * -(-T // max(1, min(T, 2 ** 30 // (n * (2 * H + 16) * 4))))),
+        "gpu_launches": args.steps * (8 * T + 12 + 6 * -(-T // max(1, min(T, 2 ** 30 // (n * (2 * H + 16) * 4))))),
         "clocks": None,
     }
     print(json.dumps(line), flush=True)

@@ -89,16 +89,29 @@ int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,
                float* obs_out, float* rew_out, uint8_t* done_out, cudaStream_t s, char* err);
 constexpr int kLdy = 16;   // floats of a policy head's row (2 x 8, or 2 x 6 padded)
 
-// obs_fm: optional [T][18][N] output of step t's observation.
+// Where a state's observation goes: the network input's rows X [N][D + 1
+// rounded up to 8] (NULL: nowhere), the step's scratch sc and step t of the
+// feature-major obs_fm [T][D][N] (either may be NULL).
+struct ObsRows {
+  float *X, *sc, *obs_fm;
+  int t;
+};
+// The gradient gX (NULL: none) of the observation of the state in scratch sc.
+struct ObsGrad {
+  const float *sc, *gX;
+};
+// Observation of the current states.
 cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X,
                        float* obs_fm, int t, cudaStream_t s);
+// One step, then the observation of the states it leads to.
 cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, uint64_t t_g,
-                        float* rew, uint8_t* done, Status* st, cudaStream_t s);
+                        float* rew, uint8_t* done, Status* st, const ObsRows& next, cudaStream_t s);
+// Adjoint of the observation of the states a step led to, then of that step.
 cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y,
                        const uint8_t* done, uint64_t t_g, const float* coef, float* lam,
-                       float* gY, cudaStream_t s);
-cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* sc, const float* gX,
-                           float* lam, cudaStream_t s);
+                       float* gY, const ObsGrad& next, cudaStream_t s);
+// Adjoint of the observation of the current states.
+cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* gX, float* lam, cudaStream_t s);
 cudaError_t launch_objective(int n, int T, const float* rew, const float* coef, const float* V,
                              int ldv, float coef_V, float* J, cudaStream_t s);
 cudaError_t launch_fill_col(int n, float* buf, int ld, float v, cudaStream_t s);

@@ -529,6 +529,45 @@ __device__ __forceinline__ void st_row(float* p, const float* v) {
 // Floats of an observation's row (the observation, 1, zeros to a sector).
 constexpr int kLdx = (kObs + 8) / 8 * 8, kPaperLdx = (paper::kObs + 8) / 8 * 8;
 using shac::kLdy;
+using shac::ObsGrad;
+using shac::ObsRows;
+
+// Values as they would be after a store and a load: what follows is rounded as
+// in a kernel of its own (no FMA across the two), whichever launch it is in.
+template <class E>
+__device__ __forceinline__ void settle(E& e) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) asm volatile("" : "+f"(e.p[k]));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) asm volatile("" : "+f"(e.q[k]));
+#pragma unroll
+  for (int k = 0; k < 6; ++k) asm volatile("" : "+f"(e.nu[k]));
+}
+template <class E>
+__device__ __forceinline__ void settle_goal(E& e) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) asm volatile("" : "+f"(e.pd[k]));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) asm volatile("" : "+f"(e.qd[k]));
+}
+
+// Observation row of the network input (augmented: 1 at column kObs, zeros up
+// to kLdx) of env i's state e; with sc also the step's scratch, with obs_fm
+// also the feature-major observation of step t.
+__device__ __forceinline__ void shac_obs_row(const Model& M, const Env& e, int i, float* __restrict__ sc,
+                                             float* __restrict__ X, float* __restrict__ obs_fm, int t) {
+  if (sc) save_step(sc, (size_t)M.n, i, e);
+  float o[kLdx];
+  observe(e, o);
+  o[kObs] = 1.0f;
+#pragma unroll
+  for (int k = kObs + 1; k < kLdx; ++k) o[k] = 0.0f;
+  st_row<kLdx>(X + (size_t)i * kLdx, o);
+  if (obs_fm) {
+#pragma unroll
+    for (int k = 0; k < kObs; ++k) obs_fm[((size_t)t * kObs + k) * M.n + i] = o[k];
+  }
+}
 
 // Reparameterised action a = mu + exp(clamp(ls)) eps from a policy head row.
 __device__ __forceinline__ void shac_action(const Model& M, const float* __restrict__ y,
@@ -543,8 +582,7 @@ __device__ __forceinline__ void shac_action(const Model& M, const float* __restr
   }
 }
 
-// Observation row of the network input (augmented: 1 at column kObs, zeros
-// up to kLdx) of each env's current state; with sc, also the step's scratch.
+// Observation rows of each env's current state.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs(const Model M, Buffers B,
                                                           float* __restrict__ sc,
                                                           float* __restrict__ X,
@@ -553,17 +591,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_obs(const Model M, Buffers
   if (i >= M.n) return;
   Env e;
   load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
-  if (sc) save_step(sc, (size_t)M.n, i, e);
-  float o[kLdx];
-  observe(e, o);
-  o[kObs] = 1.0f;
-#pragma unroll
-  for (int k = kObs + 1; k < kLdx; ++k) o[k] = 0.0f;
-  st_row<kLdx>(X + (size_t)i * kLdx, o);
-  if (obs_fm) {
-#pragma unroll
-    for (int k = 0; k < kObs; ++k) obs_fm[((size_t)t * kObs + k) * M.n + i] = o[k];
-  }
+  shac_obs_row(M, e, i, sc, X, obs_fm, t);
 }
 
 // One closed-loop step from the policy head Y [N][kLdy]: action, physics,
@@ -572,7 +600,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step(const Model M, Buffer
                                                            const float* __restrict__ Y,
                                                            uint64_t t_g, float* __restrict__ rew,
                                                            uint8_t* __restrict__ done,
-                                                           Status* st) {
+                                                           Status* st, ObsRows next) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   Env e;
@@ -590,6 +618,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step(const Model M, Buffer
   store_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   rew[i] = r;
   done[i] = d ? 1 : 0;
+  if (next.X) {
+    settle(e);
+    settle_goal(e);
+    shac_obs_row(M, e, i, next.sc, next.X, next.obs_fm, next.t);
+  }
 }
 
 // Backward of one closed-loop step: lam (dJ/d post-step state, [13][N]) is
@@ -602,7 +635,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
                                                           const uint8_t* __restrict__ done,
                                                           uint64_t t_g, const float* __restrict__ coef,
                                                           float* __restrict__ lam,
-                                                          float* __restrict__ gY) {
+                                                          float* __restrict__ gY, ObsGrad next) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
@@ -617,6 +650,14 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
     for (int k = 0; k < 6; ++k) lx.nu[k] = 0.f;
   } else {
     load_lam(lam, n, i, lx);
+    if (next.gX) {
+      Env e;
+      load_step(M, next.sc, n, i, e);
+      float lo[kLdx];
+      ld_row<kLdx>(next.gX + (size_t)i * kLdx, lo);
+      obs_vjp(e, lo, lx);
+      settle(lx);
+    }
   }
   Env es;
   load_step(M, sc, n, i, es);
@@ -653,20 +694,16 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_shac_bwd(const Model M,
   store_lam(lam, n, i, lx);
 }
 
-// lam += (d obs / d state)^T gX at the state of scratch sc (or of the env's
-// buffers when sc is NULL); gX [N][kLdx], first kObs columns.
+// lam += (d obs / d state)^T gX at the env's current state; gX [N][kLdx], first
+// kObs columns.
 __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp(const Model M, Buffers B,
-                                                              const float* __restrict__ sc,
-                                                              const float* __restrict__ gX, float* __restrict__ lam) {
+                                                              const float* __restrict__ gX,
+                                                              float* __restrict__ lam) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
   Env e;
-  if (sc) {
-    load_step(M, sc, n, i, e);
-  } else {
-    load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
-  }
+  load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   float lo[kLdx];
   ld_row<kLdx>(gX + (size_t)i * kLdx, lo);
   X lx;
@@ -1014,18 +1051,12 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_paper_adjoint(
 
 // ---- SHAC in closed loop on the paper model ----
 
-// Observation row (12 + the constant 1, zeros up to kPaperLdx) of each env's state;
-// with sc, the step's scratch (its history mean from the env's state rows).
-__global__ void __launch_bounds__(kAdjThreads) k_shac_obs_paper(const Model M, Buffers B,
-                                                                float* __restrict__ sc,
-                                                                float* __restrict__ X,
-                                                                float* __restrict__ obs_fm,
-                                                                int t) {
-  const int i = blockIdx.x * kAdjThreads + threadIdx.x;
-  if (i >= M.n) return;
-  paper::Env e;
-  paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
-  if (sc) paper_save_step(M, e, B.state, sc, (size_t)M.n, i);
+// Observation row (12 + the constant 1, zeros up to kPaperLdx) of env i's state
+// e; with sc, the step's scratch (its history mean from the env's state rows).
+__device__ __forceinline__ void paper_obs_row(const Model& M, const paper::Env& e, int i, const float* state,
+                                              float* sc, float* __restrict__ X, float* __restrict__ obs_fm,
+                                              int t) {
+  if (sc) paper_save_step(M, e, state, sc, (size_t)M.n, i);
   float o[kPaperLdx];
   paper::observe(e, o);
   o[paper::kObs] = 1.0f;
@@ -1038,8 +1069,18 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_obs_paper(const Model M, B
   }
 }
 
-// a = mu + exp(clamp(ls)) eps for the 6 wrench commands (eps: the first six
-// action normals).
+__global__ void __launch_bounds__(kAdjThreads) k_shac_obs_paper(const Model M, Buffers B,
+                                                                float* sc,
+                                                                float* __restrict__ X,
+                                                                float* __restrict__ obs_fm,
+                                                                int t) {
+  const int i = blockIdx.x * kAdjThreads + threadIdx.x;
+  if (i >= M.n) return;
+  paper::Env e;
+  paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
+  paper_obs_row(M, e, i, B.state, sc, X, obs_fm, t);
+}
+
 __device__ __forceinline__ void paper_shac_action(const Model& M, const float* __restrict__ y,
                                                   const float eps[8], float a[paper::kAct],
                                                   float sig[paper::kAct], bool in[paper::kAct]) {
@@ -1053,10 +1094,11 @@ __device__ __forceinline__ void paper_shac_action(const Model& M, const float* _
 }
 
 __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, Buffers B,
-                                                                 const float* __restrict__ Y, uint64_t t_g,
+                                                                 const float* __restrict__ Y,
+                                                                 uint64_t t_g,
                                                                  float* __restrict__ rew,
                                                                  uint8_t* __restrict__ done,
-                                                                 Status* st) {
+                                                                 Status* st, ObsRows next) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   paper::Env e;
@@ -1074,6 +1116,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, 
   paper::store_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   rew[i] = r;
   done[i] = d ? 1 : 0;
+  if (next.X) {
+    settle(e);
+    settle_goal(e);
+    paper_obs_row(M, e, i, B.state, next.sc, next.X, next.obs_fm, next.t);
+  }
 }
 
 // Backward of one closed-loop paper step: lam [61][N] (rows 0..12 the pose
@@ -1081,7 +1128,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_step_paper(const Model M, 
 __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
     const Model M, const float* __restrict__ sc, const float* __restrict__ Y,
     const uint8_t* __restrict__ done, uint64_t t_g, const float* __restrict__ coef,
-    float* __restrict__ lam, float* __restrict__ gY) {
+    float* __restrict__ lam, float* __restrict__ gY, ObsGrad next) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
@@ -1095,6 +1142,15 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
   for (int k = 0; k < 4; ++k) lx.q[k] = cut ? 0.f : lam[(3 + k) * n + i];
 #pragma unroll
   for (int k = 0; k < 6; ++k) lx.nu[k] = cut ? 0.f : lam[(7 + k) * n + i];
+  if (next.gX && !cut) {
+    paper::Env e;
+    int t_ep;
+    float mean[6], lo[kPaperLdx];
+    paper_load_step(next.sc, n, i, e, &t_ep, mean);
+    ld_row<kPaperLdx>(next.gX + (size_t)i * kPaperLdx, lo);
+    paper_obs_vjp(e, lo, lx);
+    settle(lx);
+  }
   for (int j = 0; j < paper::kHist; ++j)
 #pragma unroll
     for (int k = 0; k < 6; ++k) lh[j][k] = cut ? 0.f : lam[(13 + 6 * j + k) * n + i];
@@ -1123,21 +1179,15 @@ __global__ void __launch_bounds__(kAdjThreads) k_shac_bwd_paper(
     for (int k = 0; k < 6; ++k) lam[(13 + 6 * j + k) * n + i] = lh[j][k];
 }
 
-// lam (rows 0..12) += (d obs / d state)^T gX at the step's input (sc) or at
-// the env's current state (sc NULL).
-__global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp_paper(
-    const Model M, Buffers B, const float* __restrict__ sc, const float* __restrict__ gX, float* __restrict__ lam) {
+// lam (rows 0..12) += (d obs / d state)^T gX at the env's current state.
+__global__ void __launch_bounds__(kAdjThreads) k_shac_obs_vjp_paper(const Model M, Buffers B,
+                                                                    const float* __restrict__ gX,
+                                                                    float* __restrict__ lam) {
   const int i = blockIdx.x * kAdjThreads + threadIdx.x;
   if (i >= M.n) return;
   const size_t n = (size_t)M.n;
   paper::Env e;
-  if (sc) {
-    int t_ep;
-    float mean[6];
-    paper_load_step(sc, n, i, e, &t_ep, mean);
-  } else {
-    paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
-  }
+  paper::load_env(M, B.state, B.params, B.t_ep, B.episode, i, e);
   float lo[kPaperLdx];
   ld_row<kPaperLdx>(gX + (size_t)i * kPaperLdx, lo);
   X lx;
@@ -1169,30 +1219,29 @@ cudaError_t launch_obs(const Model& M, const Buffers& B, float* sc, float* X,
 }
 
 cudaError_t launch_step(const Model& M, const Buffers& B, const float* Y, uint64_t t_g,
-                        float* rew, uint8_t* done, Status* st, cudaStream_t s) {
+                        float* rew, uint8_t* done, Status* st, const ObsRows& next, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_step_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st);
+    k_shac_step_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st, next);
   else
-    k_shac_step<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st);
+    k_shac_step<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, Y, t_g, rew, done, st, next);
   return cudaGetLastError();
 }
 
 cudaError_t launch_bwd(const Model& M, const float* sc, const float* Y,
                        const uint8_t* done, uint64_t t_g, const float* coef, float* lam,
-                       float* gY, cudaStream_t s) {
+                       float* gY, const ObsGrad& next, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_bwd_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY);
+    k_shac_bwd_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY, next);
   else
-    k_shac_bwd<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY);
+    k_shac_bwd<<<blocks(M.n), kAdjThreads, 0, s>>>(M, sc, Y, done, t_g, coef, lam, gY, next);
   return cudaGetLastError();
 }
 
-cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* sc, const float* gX,
-                           float* lam, cudaStream_t s) {
+cudaError_t launch_obs_vjp(const Model& M, const Buffers& B, const float* gX, float* lam, cudaStream_t s) {
   if (M.model == 1)
-    k_shac_obs_vjp_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, lam);
+    k_shac_obs_vjp_paper<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, gX, lam);
   else
-    k_shac_obs_vjp<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, sc, gX, lam);
+    k_shac_obs_vjp<<<blocks(M.n), kAdjThreads, 0, s>>>(M, B, gX, lam);
   return cudaGetLastError();
 }
 
