@@ -155,15 +155,17 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       : "memory");
 }
 
-// Hidden layer epilogue for this thread's row: 256 accumulator columns at
-// col0 -> + bias -> tanh -> tf32, written back in place.  With `part` set,
-// each 32-column chunk is announced as soon as it is in tensor memory
-// (part[c], one arrival per thread), so that the next layer's K-slice c can
-// start while the later chunks are still being computed.
-__device__ __forceinline__ void hidden_epilogue(uint32_t lane_addr, uint32_t col0,
-                                                const float* bias, uint64_t* part = nullptr) {
+// Hidden layer epilogue for this thread's row: accumulator columns at col0,
+// in CHUNKS chunks of 32 -> + bias -> tanh -> tf32, written back in place.
+// Each chunk is announced as soon as it is in tensor memory (part[c], one
+// arrival per row), so that the next layer's K-slice c can start while the
+// later chunks are still being computed.  With STEP 2, two warpgroups share
+// it, `first` 0 and 1.
+template <int CHUNKS, int STEP>
+__device__ __forceinline__ void hidden_epilogue(uint32_t lane_addr, uint32_t col0, const float* bias,
+                                                uint64_t* part, int first) {
 #pragma unroll 1
-  for (int c = 0; c < kH / 32; ++c) {
+  for (int c = first; c < CHUNKS; c += STEP) {
     uint32_t acc[32];
     tc::tmem_ld32(lane_addr + col0 + 32 * c, acc);
     tc::tmem_ld_wait(acc);
@@ -172,13 +174,10 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t lane_addr, uint32_t col
       acc[j] = __float_as_uint(
           to_tf32(tc::tanh_f32(__uint_as_float(acc[j]) + bias[32 * c + j])));
     tmem_st32(lane_addr + col0 + 32 * c, acc);
-    if (part) {
-      tc::tmem_st_wait();
-      tc::tc_fence_before();
-      tc::mbar_arrive(&part[c]);
-    }
+    tc::tmem_st_wait();
+    tc::tc_fence_before();
+    tc::mbar_arrive(&part[c]);
   }
-  tc::tmem_st_wait();
 }
 
 // Gaussian head and the step's normals -> action and log-density (the fp32
@@ -343,7 +342,7 @@ k_rollout_tf32(const Model M, Buffers B, const uint8_t* __restrict__ image, Traj
       __syncwarp();
       if (!(ok = tc::mbar_wait(&bar->l1_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
-      hidden_epilogue(lane_addr, 0, bias, bar->h1_part);
+      hidden_epilogue<kSlices, 1>(lane_addr, 0, bias, bar->h1_part, 0);
       // The step's normals depend only on (env, seed, step): drawn here,
       // while layer 2's last MMAs run, instead of after the head.
       const uint32_t id = M.id_base + (uint32_t)i;
@@ -351,7 +350,7 @@ k_rollout_tf32(const Model M, Buffers B, const uint8_t* __restrict__ image, Traj
       if (active) action_noise(id, M.seed, t_g0 + (uint64_t)t, eps);
       if (!(ok = tc::mbar_wait(&bar->l2_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
-      hidden_epilogue(lane_addr, 256, bias + kH, bar->h2_part);
+      hidden_epilogue<kSlices, 1>(lane_addr, 256, bias + kH, bar->h2_part, 0);
       if (!(ok = tc::mbar_wait(&bar->l3_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
       uint32_t o3[16];
@@ -427,7 +426,29 @@ static_assert(kPSmem <= 227u * 1024u, "shared memory per CTA");
 constexpr uint32_t kColHalf = 256;   // this CTA's 128 columns of layer 2, then h2
 constexpr uint32_t kColPart = 384;   // partial head (16 columns)
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(160, 1)
+// The second epilogue warpgroup's share of every step (the two-CTA kernel:
+// 9,728 envs 8.17 -> 7.89 us a step.  One tile per CTA with twice the
+// epilogue gets slower by it, 8.33 -> 8.77 us: tanh throughput bounds it, and
+// chunks computed in pairs reach layer 2 later).  Neither l1_full nor
+// l2_full completes again before this group's arrivals of the step, so it
+// cannot miss a phase.
+__device__ __forceinline__ void epilogue_helper(PairBars* bar, uint32_t tmem, int warp, const float* b1,
+                                                const float* b2, int steps) {
+  volatile int* abort = &bar->abort;
+  const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  for (int t = 0; t < steps; ++t) {
+    const uint32_t ph = (uint32_t)t & 1u;
+    if (!tc::mbar_wait(&bar->l1_full, ph, abort, kWaitLimitNs)) break;
+    tc::tc_fence_after();
+    hidden_epilogue<kSlices, 2>(lane_addr, 0, b1, bar->h1_part, 1);
+    if (!tc::mbar_wait(&bar->l2_full, ph, abort, kWaitLimitNs)) break;
+    tc::tc_fence_after();
+    hidden_epilogue<4, 2>(lane_addr, kColHalf, b2, bar->h2_part, 1);
+  }
+}
+
+// (warps 0-3: env threads; 4: MMA issue; 5-8: the other half of the epilogues)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(288, 1)
 k_rollout_tf32_pair(const Model M, Buffers B, const uint8_t* __restrict__ image, Traj tr, int T,
                     uint64_t t_g0, Status* st) {
   extern __shared__ uint8_t smem_raw[];
@@ -517,6 +538,9 @@ k_rollout_tf32_pair(const Model M, Buffers B, const uint8_t* __restrict__ image,
       tc::mbar_wait(&bar->drain, 0, abort, kWaitLimitNs);
     }
     __syncwarp();
+  } else if (warp > 4) {
+    const float* bias = reinterpret_cast<const float*>(smem + kSB);
+    epilogue_helper(bar, tmem, warp, bias, bias + kH + 128 * rank, steps);
   } else {
     // ---- env threads (both CTAs; CTA 0 writes the trajectory) ----
     const int row = tid;
@@ -557,27 +581,14 @@ k_rollout_tf32_pair(const Model M, Buffers B, const uint8_t* __restrict__ image,
       __syncwarp();
       if (!(ok = tc::mbar_wait(&bar->l1_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
-      hidden_epilogue(lane_addr, 0, bias, bar->h1_part);
+      hidden_epilogue<kSlices, 2>(lane_addr, 0, bias, bar->h1_part, 0);
       const uint32_t id = M.id_base + (uint32_t)i;
       float eps[kAct];
       if (active) action_noise(id, M.seed, t_g0 + (uint64_t)t, eps);
       if (!(ok = tc::mbar_wait(&bar->l2_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
       // this CTA's 128 columns of h2: four chunks, each announced to layer 3
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        uint32_t acc[32];
-        const float* b2 = bias + kH + 128 * rank + 32 * c;
-        tc::tmem_ld32(lane_addr + kColHalf + 32 * c, acc);
-        tc::tmem_ld_wait(acc);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          acc[j] = __float_as_uint(to_tf32(tc::tanh_f32(__uint_as_float(acc[j]) + b2[j])));
-        tmem_st32(lane_addr + kColHalf + 32 * c, acc);
-        tc::tmem_st_wait();
-        tc::tc_fence_before();
-        tc::mbar_arrive(&bar->h2_part[c]);
-      }
+      hidden_epilogue<4, 2>(lane_addr, kColHalf, bias + kH + 128 * rank, bar->h2_part, 0);
       if (!(ok = tc::mbar_wait(&bar->l3_full, ph, abort, kWaitLimitNs))) break;
       tc::tc_fence_after();
       uint32_t p3[16];
@@ -665,7 +676,7 @@ cudaError_t launch_rollout_tf32(const Model& M, const Buffers& B, const void* pa
     e = cudaFuncSetAttribute(k_rollout_tf32_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kPSmem);
     if (e != cudaSuccess) return e;
-    k_rollout_tf32_pair<<<2 * grid, 160, kPSmem, s>>>(M, B, static_cast<const uint8_t*>(packed),
+    k_rollout_tf32_pair<<<2 * grid, 288, kPSmem, s>>>(M, B, static_cast<const uint8_t*>(packed),
                                                       tr, T, t_g0, st);
     return cudaGetLastError();
   }
