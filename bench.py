@@ -666,7 +666,10 @@ def run_ppo(args):
         bound, psrc = "tensor", (f"bf16 sustained, {src}" + ("" if ratio == 1.0 else
                                  " x tf32/bf16 nominal 1.1/2.25"))
     st = stats.cpu().numpy().tolist()
-    launches_per_step = 1 + 10 + 1 + 1 + 14 + 2     # gather, fwd, head, stats, bwd, norm+Adam
+    # gather, forward, head, stats, backward, norm + Adam (3); on the bf16 engine with its images packed and the
+    # weight gradients in two groups with their reductions, else one product per layer and direction.  Three launches
+    # an epoch draw its rows and advantage statistics.
+    launches_per_step = 1 + 1 + 2 + 2 + 2 + 4 + 3 if args.ppo_precision == "bf16" else 1 + 6 + 2 + 10 + 3
     line = {
         "metric": "PPO update samples/s", "value": samples / (step_ms * 1e-3),
         "unit": "samples/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -682,7 +685,7 @@ def run_ppo(args):
                      "frac": achieved / peak, "traffic": None, "peak_source": psrc,
                      "flops_per_sample": fps},
         "update_stats": dict(zip(auvenv.PPO_STAT_NAMES, st)),
-        "gpu_launches": args.steps * args.epochs * n_mb * launches_per_step,
+        "gpu_launches": args.steps * args.epochs * (n_mb * launches_per_step + 3),
         "clocks": clock_info,
     }
     print(json.dumps(line), flush=True)

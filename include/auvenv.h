@@ -506,8 +506,8 @@ int ppo_apply(auv_ppo* p, const float* grad, float* stats, void* stream);
  * `stream`; the weights (ppo_get_weights, or the pointers of ppo_weights) are
  * the updated ones once it completes.  Each call first copies the batch into
  * a sample-major buffer (T * N rows of round8(obs_dim + act_dim + 3) floats,
- * one coalesced pass) from which every step gathers its minibatch; the
- * learner allocates that buffer the first time it sees a batch of more rows
+ * one coalesced pass) from which every step gathers its minibatch, with 4
+ * more bytes a row for the epoch's permutation; the learner allocates that buffer the first time it sees a batch of more rows
  * than the last (the one allocation after ppo_create) and frees it in
  * ppo_destroy.  If the allocation fails the steps gather from the batch's
  * own arrays.
@@ -589,7 +589,8 @@ int env_adjoint(auv_env* env, int T, const float* act, const float* coef, const 
  * between steps, as env_adjoint's does); 1 <= T <= AUV_ADJOINT_MAX_T, at most
  * AUV_ADJOINT_MAX_SUBSTEPS substeps, hidden a multiple of 8 up to 1024.
  * The first call at a given (N, T) allocates the window's workspace
- * (activations of every step: about T N (2 hidden + 80) floats).
+ * (activations of every step: about T N (2 hidden + 80) floats; and the layer
+ * gradients of one step, or of as many steps as fit 1 GiB).
  */
 int env_shac_window(auv_env* env, const float* policy, const float* value, int T,
                     const float* coef, float coef_V, uint32_t precision, float* grad,
