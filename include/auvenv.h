@@ -621,7 +621,8 @@ int env_inverse_allocate(auv_env* env, int n, const float* wrench, float* cmd, v
  * act[t][.][i], rew / done = [t][i], next_obs = obs[t+1][.][i] (last_obs for
  * t = T-1: the observation after the last step).  After an auto-reset the
  * next observation is the new episode's first: a time-limit end is stored
- * as a terminal transition (done = 1).  Inputs are the rollout's arrays in
+ * as a terminal transition (done = 1).  When T x N exceeds the capacity the
+ * newest `capacity` transitions remain.  Inputs are the rollout's arrays in
  * device memory: obs [T][D][N], act [T][A][N], rew [T][N] fp32, done [T][N]
  * u8, last_obs [D][N].  head and size advance on the host at the call.
  *

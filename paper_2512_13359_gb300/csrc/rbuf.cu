@@ -53,13 +53,17 @@ constexpr size_t insert_smem(int tile, int D, int A) {
 // once.  HBM-bound by the copies in flight: 65,536 envs x 16 steps (304 MB at 18
 // + 8 features) took 126 us with one tile per step through registers and a
 // division per stored element, 65 us here (4.7 TB/s).
-template <int TILE>
+//
+// SKIP: the first `skip` envs of step 0 are not stored, so that a call with more
+// transitions than the ring has slots writes each slot once (blocks run in no
+// order): the newest C of them.
+template <int TILE, bool SKIP>
 __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, int A,
                                                    const float* __restrict__ obs,
                                                    const float* __restrict__ act,
                                                    const float* __restrict__ rew,
                                                    const uint8_t* __restrict__ done,
-                                                   const float* __restrict__ last_obs,
+                                                   const float* __restrict__ last_obs, int skip,
                                                    uint64_t head, uint64_t C,
                                                    float* __restrict__ s_obs,
                                                    float* __restrict__ s_act,
@@ -101,6 +105,7 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
   for (int t = t0; t < t1; ++t) {
     float r = 0.0f;
     uint8_t d = 0;
+    const int j0 = SKIP && t == 0 ? min(max(skip - i0, 0), cnt) : 0;   // the tile's first env to store
     if (tid < cnt) {
       r = __ldg(rew + (size_t)t * n + i0 + tid);
       d = __ldg(done + (size_t)t * n + i0 + tid);
@@ -111,9 +116,9 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
     const uint64_t slot0 = (head + (uint64_t)t * n + (uint64_t)i0) % C;
     const bool flat = slot0 + (uint64_t)cnt <= C;     // the tile's slots do not wrap
     const float *o0 = obs_tile(t), *o1 = obs_tile(t + 1), *at = act_tile(t);
-    int j = tid / D, k = tid % D;
+    int j = j0 + tid / D, k = tid % D;
 #pragma unroll 4
-    for (int e = tid; e < cnt * D; e += kInThreads) {
+    for (int e = j0 * D + tid; e < cnt * D; e += kInThreads) {
       const size_t dst = flat ? slot0 * D + e : (slot0 + j) % C * D + k;
       s_obs[dst] = o0[k * S + j];
       s_next[dst] = o1[k * S + j];
@@ -124,10 +129,10 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
         ++j;
       }
     }
-    j = tid / A;
+    j = j0 + tid / A;
     k = tid % A;
 #pragma unroll 4
-    for (int e = tid; e < cnt * A; e += kInThreads) {
+    for (int e = j0 * A + tid; e < cnt * A; e += kInThreads) {
       s_act[flat ? slot0 * A + e : (slot0 + j) % C * A + k] = at[k * S + j];
       j += aj;
       k += ak;
@@ -136,7 +141,7 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
         ++j;
       }
     }
-    if (tid < cnt) {
+    if (tid >= j0 && tid < cnt) {
       const uint64_t slot = flat ? slot0 + tid : (slot0 + tid) % C;
       s_rew[slot] = r;
       s_done[slot] = d;
@@ -415,15 +420,21 @@ int rbuf_insert(auv_rbuf* r, int T, int N, const float* obs, const float* act, c
   const bool wide = auv::insert_smem(64, D, A) <= 48 * 1024;
   const int tile = wide ? 64 : 32;
   const size_t smem = auv::insert_smem(tile, D, A);
-  auto kern = wide ? auv::k_rb_insert<64> : auv::k_rb_insert<32>;
+  // more transitions than slots: the newest C of them, from env `skip` of step t0
+  const uint64_t added = (uint64_t)T * (uint64_t)N;
+  const uint64_t lost = added > r->C ? added - r->C : 0;
+  const int t0 = (int)(lost / (uint64_t)N), skip = (int)(lost % (uint64_t)N), steps = T - t0;
+  const size_t o = (size_t)t0 * (size_t)N;
+  auto kern = wide ? (skip ? auv::k_rb_insert<64, true> : auv::k_rb_insert<64, false>)
+                   : (skip ? auv::k_rb_insert<32, true> : auv::k_rb_insert<32, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel attributes");
-  const dim3 grid((N + tile - 1) / tile, (T + auv::kSteps - 1) / auv::kSteps);
+  const dim3 grid((N + tile - 1) / tile, (steps + auv::kSteps - 1) / auv::kSteps);
   kern<<<grid, auv::kInThreads, smem, static_cast<cudaStream_t>(stream)>>>(
-      T, N, D, A, obs, act, rew, done, last_obs, r->head, r->C, r->obs, r->act, r->rew, r->next, r->done);
+      steps, N, D, A, obs + o * D, act + o * A, rew + o, done + o, last_obs, skip, (r->head + o) % r->C, r->C, r->obs,
+      r->act, r->rew, r->next, r->done);
   e = cudaGetLastError();
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel");
-  const uint64_t added = (uint64_t)T * (uint64_t)N;
   r->head = (r->head + added) % r->C;
   r->size = r->size + added < r->C ? r->size + added : r->C;
   return AUV_OK;

@@ -30,3 +30,29 @@ def test_insert_and_sample(D, A, N):
     assert np.array_equal(out["idx"].cpu().numpy(), want["idx"].astype(np.int32))
     for k in ("obs", "act", "rew", "next_obs", "done"):
         assert np.array_equal(out[k].cpu().numpy(), want[k]), k
+
+
+@pytest.mark.parametrize("D,A", [(18, 8), (130, 3)])
+@pytest.mark.parametrize("N,T,C", [
+    (65, 3, 64), (130, 1, 129), (1, 40, 7),      # C one below a multiple of N; a tile of one env
+    (200, 2, 5), (33, 17, 1),                    # C far below a tile
+    (100, 9, 450), (64, 24, 64 * 16 + 10),       # the first stored env in mid-step; whole blocks of steps dropped
+])
+def test_insert_more_than_the_ring_holds(D, A, N, T, C):
+    """Several transitions of one insert share a slot: the newest of them stays, whole."""
+    torch = need_gpu()
+    from oracle import offpolicy_oracle as F
+    from paper_2512_13359_gb300 import auvenv
+    rb, ref = auvenv.ReplayBuffer(D, A, C), F.ReplayBuffer(D, A, C)
+    rng = np.random.default_rng(N + T)
+    for steps in (1, T, T):   # the first moves head off slot 0
+        x = (rng.normal(size=(steps, D, N)), rng.normal(size=(steps, A, N)), rng.normal(size=(steps, N)),
+             rng.random((steps, N)) < 0.2, rng.normal(size=(D, N)))
+        x = [v.astype(np.uint8 if v.dtype == bool else np.float32) for v in x]
+        rb.insert(*(torch.from_numpy(v).cuda() for v in x))
+        ref.insert(*x)
+        assert rb.size == (ref.size, ref.head)
+        B = 8 * C + 64   # every slot is drawn (but for chance)
+        out, want = rb.sample(B, seed=7, draw=steps, with_idx=True), ref.sample(7, steps, B)
+        for k in ("obs", "act", "rew", "next_obs", "done"):
+            assert np.array_equal(out[k].cpu().numpy(), want[k]), k
