@@ -1052,24 +1052,32 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32_warps(const F32Args args) 
 
 // ---------------------------------------------------------------------------
 // A step's weight gradients (bf16, both operands along the samples) in one
-// launch of at most one CTA per SM: each item's row tiles get CTAs in
-// proportion to the bytes a K-chunk of theirs moves, so that all finish
-// together.  They are bound by the reads (426 MB through L2 at 65,536 samples
-// of both networks), which six launches of their own left idle at each start
-// and end: 85 us and 19 us of reductions per step.
+// launch of at most one CTA per SM.  The work is cut into units, a 128-row tile
+// of an item over one K range of it; the ranges are those of the item's product
+// launched alone (group_ranges), so that a gradient has the same bits whatever
+// shares its launch.  CTA c takes wide units (more than 192 columns) c, c + G,
+// ... and narrow ones from the other end, a wide and a narrow one in turn: each
+// kind has its own columns of tensor memory, so one unit's partials are read
+// out under the next one's MMAs, and the reads, which bound the kernel, stay
+// even over the SMs (426 MB through L2 at 65,536 samples of both networks).
+// 32 PPO steps of 65,536 samples: 9.08 ms with a launch per product, 8.17 here
+// (8.00 with longer ranges, fewer partials and a third of the chains, whose
+// sums are others).
 // ---------------------------------------------------------------------------
 struct GroupMaps {
   CUtensorMap a[kMaxGroup], b[kMaxGroup];
 };
 struct GroupArgs {
   struct Item {
-    int M, N, splits, per_split, cta0;   // K-chunks per CTA; first CTA
-    float* ws;                           // [splits][M][n_pad]
+    int M, N, splits, per_split;   // K ranges, K-chunks in each
+    int unit0;                     // its first unit of its kind
+    float* ws;                     // [splits][M][n_pad]
     int n_pad;
     float* C;
     int ldc;
   } it[kMaxGroup];
   int n, chunks;
+  int units[2];                    // wide, narrow
   Status* st;
 };
 
@@ -1079,7 +1087,42 @@ struct GroupTile {
   static constexpr uint32_t kABytes = 2 * kBlock, kBBytes = 5 * kBlock, kStage = kABytes + kBBytes;
   static constexpr int kStages = 3;
   static constexpr uint32_t kSmem = kStages * kStage + 256 + 1024;
+  static constexpr int kNarrow = 192;                    // columns of a narrow unit, at most
+  static constexpr uint32_t kNarrowCol = 512 - kNarrow;  // its accumulator's first column
 };
+
+struct GroupBars {
+  uint64_t full[GroupTile::kStages], empty[GroupTile::kStages];
+  uint64_t acc_full[2], acc_empty[2];                    // wide, narrow accumulator
+  uint64_t done;
+  uint32_t tmem_base;
+  int abort;
+};
+
+// The j-th unit of this CTA: its kind (j odd: narrow), item, row tile, K range.
+struct GroupUnit {
+  int kind, q, m0, z, c0, n_chunks;
+};
+__device__ __forceinline__ bool group_unit(const GroupArgs& args, int j, GroupUnit* u) {
+  const int G = (int)gridDim.x;
+  u->kind = j & 1;
+  const int index = (u->kind ? G - 1 - (int)blockIdx.x : (int)blockIdx.x) + (j >> 1) * G;
+  if (index >= args.units[u->kind]) return false;
+  u->q = -1;
+  for (int k = 0; k < args.n; ++k)
+    if ((args.it[k].N <= GroupTile::kNarrow ? 1 : 0) == u->kind && index >= args.it[k].unit0) u->q = k;
+  const GroupArgs::Item& it = args.it[u->q];
+  const int local = index - it.unit0;
+  u->z = local % it.splits;
+  u->m0 = local / it.splits * kBM;
+  u->c0 = u->z * it.per_split;
+  u->n_chunks = min(args.chunks, u->c0 + it.per_split) - u->c0;
+  return true;
+}
+// Units of the CTA that takes most, empty places included.
+__device__ __forceinline__ int group_turns(const GroupArgs& args) {
+  return 2 * ((max(args.units[0], args.units[1]) + (int)gridDim.x - 1) / (int)gridDim.x);
+}
 
 __global__ void __launch_bounds__(192, 1)
 k_gemm_group(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupArgs args) {
@@ -1088,21 +1131,21 @@ k_gemm_group(const __grid_constant__ GroupMaps maps, const __grid_constant__ Gro
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~(uintptr_t)1023u);
-  Bars* bar = reinterpret_cast<Bars*>(smem + kStages * TL::kStage);
+  GroupBars* bar = reinterpret_cast<GroupBars*>(smem + kStages * TL::kStage);
   volatile int* abort = &bar->abort;
   const int tid = threadIdx.x, warp = tid >> 5;
-  int q = 0;
-  while (q + 1 < args.n && (int)blockIdx.x >= args.it[q + 1].cta0) ++q;
-  const GroupArgs::Item& it = args.it[q];
-  const int local = (int)blockIdx.x - it.cta0, z = local % it.splits, m0 = local / it.splits * kBM;
-  const int c0 = z * it.per_split, n_chunks = max(0, min(args.chunks, c0 + it.per_split) - c0);
+  const int turns = group_turns(args);
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       tc::mbar_init(&bar->full[s], 1);
       tc::mbar_init(&bar->empty[s], 1);
     }
-    tc::mbar_init(&bar->acc_full, 1);
+    for (int k = 0; k < 2; ++k) {
+      tc::mbar_init(&bar->acc_full[k], 1);
+      tc::mbar_init(&bar->acc_empty[k], 4);
+    }
+    tc::mbar_init(&bar->done, 1);
     bar->abort = 0;
     tc::mbar_fence_init();
   }
@@ -1117,75 +1160,102 @@ k_gemm_group(const __grid_constant__ GroupMaps maps, const __grid_constant__ Gro
 
   if (warp == kProducer) {
     if ((tid & 31) == 0) {
-      const int na = min(2, (it.M - m0 + 63) / 64), nb = (it.N + 63) / 64;
-      int c = 0;
-      for (; c < n_chunks; ++c) {
-        const int s = c % kStages;
-        if (c >= kStages &&
-            !tc::mbar_wait(&bar->empty[s], (uint32_t)((c / kStages) - 1) & 1u, abort, kWaitLimitNs))
-          break;
-        uint8_t* dst = smem + s * TL::kStage;
-        const int k = (c0 + c) * TL::kBK;
-        tc::mbar_arrive_expect_tx(&bar->full[s], (na + nb) * TL::kBlock);
-        for (int j = 0; j < na; ++j)
-          tma_load_2d(dst + j * TL::kBlock, &maps.a[q], m0 + 64 * j, k, &bar->full[s]);
-        for (int j = 0; j < nb; ++j)
-          tma_load_2d(dst + TL::kABytes + j * TL::kBlock, &maps.b[q], 64 * j, k, &bar->full[s]);
+      int s = 0, fill = 0;   // next stage, and how often the ring has gone round
+      bool ok = true;
+      GroupUnit u;
+      for (int j = 0; j < turns && ok; ++j) {
+        if (!group_unit(args, j, &u)) continue;
+        const GroupArgs::Item& it = args.it[u.q];
+        const int na = min(2, (it.M - u.m0 + 63) / 64), nb = (it.N + 63) / 64;
+        for (int c = 0; c < u.n_chunks; ++c) {
+          ok = fill == 0 || tc::mbar_wait(&bar->empty[s], (uint32_t)(fill - 1) & 1u, abort, kWaitLimitNs);
+          if (!ok) break;
+          uint8_t* dst = smem + s * TL::kStage;
+          const int k = (u.c0 + c) * TL::kBK;
+          tc::mbar_arrive_expect_tx(&bar->full[s], (na + nb) * TL::kBlock);
+          for (int i = 0; i < na; ++i)
+            tma_load_2d(dst + i * TL::kBlock, &maps.a[u.q], u.m0 + 64 * i, k, &bar->full[s]);
+          for (int i = 0; i < nb; ++i)
+            tma_load_2d(dst + TL::kABytes + i * TL::kBlock, &maps.b[u.q], 64 * i, k, &bar->full[s]);
+          if (++s == kStages) {
+            s = 0;
+            ++fill;
+          }
+        }
       }
       if (*abort)   // the copies still in flight
-        for (int s = 0; s < kStages; ++s) {
-          const int fills = c / kStages + (s < c % kStages ? 1 : 0);
-          if (fills > 0) wait_landed(&bar->full[s], (uint32_t)(fills - 1) & 1u);
+        for (int q = 0; q < kStages; ++q) {
+          const int fills = fill + (q < s ? 1 : 0);
+          if (fills > 0) wait_landed(&bar->full[q], (uint32_t)(fills - 1) & 1u);
         }
     }
     __syncwarp();
   } else if (warp == kIssuer) {
     if ((tid & 31) == 0) {
-      // columns in one MMA of up to 256, the rest in a second
-      const uint32_t id1 = idesc(false, true, true, kBM, min(256, (it.N + 15) / 16 * 16));
-      const uint32_t id2 = idesc(false, true, true, kBM, max(16, (it.N - 256 + 15) / 16 * 16));
       const uint32_t base = tc::smem_u32(smem);
+      int s = 0;
+      uint32_t phase = 0;
       bool ok = true;
-      for (int c = 0; c < n_chunks && ok; ++c) {
-        const int s = c % kStages;
-        ok = tc::mbar_wait(&bar->full[s], (uint32_t)(c / kStages) & 1u, abort, kWaitLimitNs);
-        if (!ok) break;
-        tc::tc_fence_after();
-        const uint32_t a0 = base + s * TL::kStage, b0 = a0 + TL::kABytes;
+      GroupUnit u;
+      for (int j = 0; j < turns && ok; ++j) {
+        if (!group_unit(args, j, &u)) continue;
+        const int N = args.it[u.q].N, use = j >> 1;   // use: of this kind's accumulator
+        // columns in one MMA of up to 256, the rest in a second
+        const uint32_t id1 = idesc(false, true, true, kBM, min(256, (N + 15) / 16 * 16));
+        const uint32_t id2 = idesc(false, true, true, kBM, max(16, (N - 256 + 15) / 16 * 16));
+        const uint32_t d = tmem + (u.kind ? TL::kNarrowCol : 0u);
+        ok = use == 0 || tc::mbar_wait(&bar->acc_empty[u.kind], (uint32_t)(use - 1) & 1u, abort, kWaitLimitNs);
+        if (ok) tc::tc_fence_after();
+        for (int c = 0; c < u.n_chunks && ok; ++c) {
+          ok = tc::mbar_wait(&bar->full[s], phase, abort, kWaitLimitNs);
+          if (!ok) break;
+          tc::tc_fence_after();
+          const uint32_t a0 = base + s * TL::kStage, b0 = a0 + TL::kABytes;
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint32_t acc = c > 0 || kk > 0 ? 1u : 0u;
-          const uint64_t da = desc_sw128(a0 + kk * 2048, TL::kBlock, 1024);
-          mma<false>(tmem, da, desc_sw128(b0 + kk * 2048, TL::kBlock, 1024), id1, acc);
-          if (it.N > 256)
-            mma<false>(tmem + 256, da, desc_sw128(b0 + 4 * TL::kBlock + kk * 2048, TL::kBlock, 1024), id2,
-                       acc);
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint32_t acc = c > 0 || kk > 0 ? 1u : 0u;
+            const uint64_t da = desc_sw128(a0 + kk * 2048, TL::kBlock, 1024);
+            mma<false>(d, da, desc_sw128(b0 + kk * 2048, TL::kBlock, 1024), id1, acc);
+            if (N > 256)
+              mma<false>(d + 256, da, desc_sw128(b0 + 4 * TL::kBlock + kk * 2048, TL::kBlock, 1024), id2, acc);
+          }
+          tc::mma_commit(&bar->empty[s]);
+          if (++s == kStages) {
+            s = 0;
+            phase ^= 1u;
+          }
         }
-        tc::mma_commit(&bar->empty[s]);
+        if (ok) tc::mma_commit(&bar->acc_full[u.kind]);
       }
-      tc::mma_commit(&bar->acc_full);
-      wait_landed(&bar->acc_full, 0);   // tensor memory is freed below
+      tc::mma_commit(&bar->done);
+      wait_landed(&bar->done, 0);   // tensor memory is freed below
     }
     __syncwarp();
   } else {
-    const bool ok = n_chunks > 0 && tc::mbar_wait(&bar->acc_full, 0, abort, kWaitLimitNs);
-    tc::tc_fence_after();
-    const int row = m0 + tid;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
+    GroupUnit u;
+    for (int j = 0; j < turns; ++j) {
+      if (!group_unit(args, j, &u)) continue;
+      const GroupArgs::Item& it = args.it[u.q];
+      const bool ok = tc::mbar_wait(&bar->acc_full[u.kind], (uint32_t)(j >> 1) & 1u, abort, kWaitLimitNs);
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      tc::tc_fence_after();
+      const int row = u.m0 + tid;
+      const uint32_t col = u.kind ? TL::kNarrowCol : 0u;
 #pragma unroll 1
-    for (int nb = 0; nb < it.N; nb += 32) {
-      uint32_t acc[32];
-      tc::tmem_ld32(lane_addr + nb, acc);
-      tc::tmem_ld_wait(acc);
-      if (!ok) {
+      for (int nb = 0; nb < it.N; nb += 32) {
+        uint32_t acc[32];
+        tc::tmem_ld32(lane_addr + col + nb, acc);
+        tc::tmem_ld_wait(acc);
+        if (row < it.M) {
+          float* dst = it.ws + ((size_t)u.z * it.M + row) * it.n_pad + nb;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0u;   // no K in range (or a timed-out wait)
+          for (int i = 0; i < 4; ++i) st_f32x8(dst + 8 * i, acc + 8 * i);
+        }
       }
-      if (row < it.M) {
-        float* dst = it.ws + ((size_t)z * it.M + row) * it.n_pad + nb;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) st_f32x8(dst + 8 * j, acc + 8 * j);
-      }
+      tc::tc_fence_before();
+      __syncwarp();
+      if ((tid & 31) == 0) tc::mbar_arrive(&bar->acc_empty[u.kind]);
     }
   }
   tc::tc_fence_before();
@@ -1668,39 +1738,35 @@ cudaError_t launch(Prec prec, int M, int N, int K, const Operand& A_in, const Op
 
 namespace {
 
-// CTAs, K ranges and partials (floats of workspace) of a group.
+// K ranges of one item, as its product alone is split over the SMs: 128-row
+// tiles of all columns, but three tiles of 128 columns where a few rows meet
+// more than 256, at least four chunks a range.
+void group_ranges(const GroupItem& i, int chunks, int* splits, int* per_split) {
+  const int sms = sm_count_dev(), tiles = (i.M + kBM - 1) / kBM * (i.M <= kBM && i.N > 256 ? 3 : 1);
+  const int want = std::max(1, std::min(tiles >= sms / 2 ? 1 : (sms + tiles - 1) / tiles, chunks / 4));
+  *per_split = (chunks + want - 1) / want;
+  *splits = (chunks + *per_split - 1) / *per_split;
+}
+
+// Units, K ranges and partials (floats of workspace) of a group.
 void plan_group(const GroupItem* items, int n, int K, GroupArgs* g, size_t* floats) {
-  const int sms = sm_count_dev();
   g->n = n;
   g->chunks = (K + GroupTile::kBK - 1) / GroupTile::kBK;
-  auto cost = [](const GroupItem& i) {   // 64-column blocks per K-chunk of a row tile
-    return std::min(2, (i.M + 63) / 64) + (i.N + 63) / 64;
-  };
-  long total = 0;
-  for (int k = 0; k < n; ++k) total += (long)cost(items[k]) * ((items[k].M + kBM - 1) / kBM);
-  int cta = 0;
+  g->units[0] = g->units[1] = 0;
   *floats = 0;
   for (int k = 0; k < n; ++k) {
     GroupArgs::Item& it = g->it[k];
-    const int tiles = (items[k].M + kBM - 1) / kBM;
-    // at least two chunks per CTA
-    const int want = std::max(1, std::min((int)((long)sms * cost(items[k]) / total), g->chunks / 2));
     it.M = items[k].M;
     it.N = items[k].N;
-    it.per_split = (g->chunks + want - 1) / want;
-    it.splits = (g->chunks + it.per_split - 1) / it.per_split;
-    it.cta0 = cta;
-    cta += tiles * it.splits;
+    group_ranges(items[k], g->chunks, &it.splits, &it.per_split);
+    int& units = g->units[it.N <= GroupTile::kNarrow ? 1 : 0];
+    it.unit0 = units;
+    units += (it.M + kBM - 1) / kBM * it.splits;
     it.n_pad = (it.N + 31) / 32 * 32;
     it.C = items[k].C;
     it.ldc = items[k].ldc;
     *floats += (size_t)it.splits * it.M * it.n_pad;
   }
-}
-
-int group_ctas(const GroupArgs& g) {
-  const GroupArgs::Item& last = g.it[g.n - 1];
-  return last.cta0 + (last.M + kBM - 1) / kBM * last.splits;
 }
 
 }  // namespace
@@ -1736,7 +1802,7 @@ cudaError_t launch_group(const GroupItem* items, int n, int K, float* ws, size_t
   cudaError_t e = cudaFuncSetAttribute(k_gemm_group, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        GroupTile::kSmem);
   if (e != cudaSuccess) return e;
-  k_gemm_group<<<group_ctas(g), 192, GroupTile::kSmem, s>>>(maps, g);
+  k_gemm_group<<<std::min(sm_count_dev(), g.units[0] + g.units[1]), 192, GroupTile::kSmem, s>>>(maps, g);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_reduce_group<<<dim3(blocks, n), kRedGroups * kRedQuads, 0, s>>>(g);
   return cudaGetLastError();

@@ -405,31 +405,46 @@ __global__ void __launch_bounds__(kT) k_epoch_rows(uint32_t count, PermKey key, 
 }
 
 // Sums of a minibatch's (mb0 + blockIdx.y) advantages and their squares, in
-// fp64: a block takes kAdvPer samples, several per thread before the block's
-// tree (the GPU's fp64 pipe runs at a 64th of the fp32 rate).
-constexpr int kAdvPer = 8 * kT;
+// fp64, a pair for every kT consecutive samples, added in block_sum's order:
+// the partial sums of k_gather, bit for bit.  A block takes kAdvSets such sets;
+// a warp adds its 2 kAdvSets sums together, halving the sums a lane holds with
+// the lanes they come from, 9 fp64 additions a lane where one tree per sum
+// takes 5 each (the GPU's fp64 pipe runs at a 64th of the fp32 rate).
+constexpr int kAdvSets = 8;
 __global__ void __launch_bounds__(kT) k_adv_sums(int B, uint32_t mb0, const float* __restrict__ rows, int Ws,
-                                                 int adv_at, EpochPrep prep) {
-  __shared__ double sh[2 * (kT / 32)];
+                                                 int adv_at, int n_part, EpochPrep prep) {
+  __shared__ double sh[kT / 32][2 * kAdvSets];
   const uint32_t mb = mb0 + blockIdx.y;
-  const int b0 = blockIdx.x * kAdvPer + threadIdx.x;
-  float a[kAdvPer / kT];
+  const int set0 = blockIdx.x * kAdvSets, b0 = set0 * kT + threadIdx.x;
+  double s[2 * kAdvSets];
 #pragma unroll
-  for (int u = 0; u < kAdvPer / kT; ++u) {
+  for (int u = 0; u < kAdvSets; ++u) {
     const int b = b0 + u * kT;
-    a[u] = b < B ? __ldg(rows + (size_t)__ldg(prep.rows + (size_t)mb * (uint32_t)B + b) * Ws + adv_at) : 0.0f;
+    const float a = b < B ? __ldg(rows + (size_t)__ldg(prep.rows + (size_t)mb * (uint32_t)B + b) * Ws + adv_at) : 0.0f;
+    s[2 * u] = a;
+    s[2 * u + 1] = (double)a * a;
   }
-  double s[2] = {0.0, 0.0};
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int u = 0; u < kAdvPer / kT; ++u) {
-    s[0] += a[u];
-    s[1] = fma((double)a[u], (double)a[u], s[1]);
+  for (int o = 16, have = 2 * kAdvSets; o > 1; o >>= 1, have >>= 1) {   // the lower lanes keep the first half
+#pragma unroll
+    for (int k = 0; k < have / 2; ++k) {
+      const double mine = l & o ? s[k + have / 2] : s[k], other = l & o ? s[k] : s[k + have / 2];
+      s[k] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, o);
+    }
   }
-  block_sum<2>(s, sh);
-  if (threadIdx.x == 0) {
-    double* part = prep.part + 2 * ((size_t)mb * gridDim.x + blockIdx.x);
-    part[0] = s[0];
-    part[1] = s[1];
+  s[0] += __shfl_xor_sync(0xFFFFFFFFu, s[0], 1);   // sum l / 2 of the warp
+  if ((l & 1) == 0) sh[w][l >> 1] = s[0];
+  __syncthreads();
+  if (threadIdx.x < 2 * kAdvSets && set0 + (int)threadIdx.x / 2 < n_part) {
+    double v[kT / 32];
+#pragma unroll
+    for (int k = 0; k < kT / 32; ++k) v[k] = sh[k][threadIdx.x];
+#pragma unroll
+    for (int o = kT / 64; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) v[k] += v[k + o];
+    prep.part[2 * ((size_t)mb * n_part + set0) + threadIdx.x] = v[0];
   }
 }
 
@@ -790,12 +805,12 @@ cudaError_t launch_transpose_batch(int D, int A, uint32_t T, uint32_t N, const f
 }
 
 size_t epoch_prep_bytes(const Dims& d, size_t rows) {
-  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kAdvPer - 1) / kAdvPer;
+  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kT - 1) / kT;
   return ((rows * 4 + 15) & ~(size_t)15) + n_mb * (nb + 1) * 2 * sizeof(double);
 }
 
 EpochPrep epoch_prep(const Dims& d, size_t rows, char* mem) {
-  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kAdvPer - 1) / kAdvPer;
+  const size_t n_mb = rows / (size_t)d.B, nb = ((size_t)d.B + kT - 1) / kT;
   double* part = reinterpret_cast<double*>(mem + ((rows * 4 + 15) & ~(size_t)15));
   return {reinterpret_cast<uint32_t*>(mem), part, part + 2 * n_mb * nb};
 }
@@ -807,10 +822,11 @@ cudaError_t launch_epoch_prep(const Dims& d, const PermKey& k, uint32_t n_mb, co
   k_epoch_rows<<<(unsigned)(blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks)), kT, 0, s>>>((uint32_t)count, k,
                                                                                          prep.rows);
   if (d.value_only) return cudaGetLastError();
-  const unsigned nb = ((unsigned)d.B + kAdvPer - 1) / kAdvPer;
+  const unsigned nb = ((unsigned)d.B + kT - 1) / kT;
   for (uint32_t m0 = 0; m0 < n_mb; m0 += 65535u) {   // gridDim.y
     const uint32_t m = n_mb - m0 < 65535u ? n_mb - m0 : 65535u;
-    k_adv_sums<<<dim3(nb, m), kT, 0, s>>>(d.B, m0, rows, sample_row_floats(d.D, d.A), d.D + d.A + 1, prep);
+    k_adv_sums<<<dim3((nb + kAdvSets - 1) / kAdvSets, m), kT, 0, s>>>(d.B, m0, rows, sample_row_floats(d.D, d.A),
+                                                                      d.D + d.A + 1, (int)nb, prep);
   }
   k_adv_norm<<<n_mb, kT, 0, s>>>(d.B, (int)nb, prep);
   return cudaGetLastError();

@@ -77,3 +77,45 @@ def test_grouped_weight_gradients(D, A, B, value_only):
         err = np.abs(g[0][sl] - g[1][sl]).max() / scale
         print(f"[grouped D={D} B={B}] {err:.2e}")
         assert err <= 4 * GRAD_TOL["bf16"]
+
+
+@pytest.mark.parametrize("D,A,B", [(18, 8, 2), (12, 6, 255), (18, 8, 257), (7, 3, 5000), (18, 8, 30011)])
+def test_a_gradient_does_not_depend_on_its_launch(D, A, B):
+    """The K ranges of a weight gradient are its own product's: the value network's gradient has the same bits alone
+    and in one launch with the policy's."""
+    torch = need_gpu()
+    H, T, N = 256, 16, 2048
+    pw, vw = _weights(D, H, A, seed=3)
+    traj = _dev(torch, _traj(8, T, N, D, A))
+    g = []
+    for value_only in (False, True):
+        L = _learner(D, A, H, B, "bf16", value_only=value_only)
+        L.set_weights(pw, vw)
+        grad = torch.empty(L.n_policy + L.n_value, device="cuda")
+        L.grads({k: traj[k] for k in ("obs", "ret")} if value_only else traj, 0, 0, grad=grad)
+        assert L.status().code == 0
+        g.append(to_np(grad)[L.n_policy:])
+    assert np.abs(g[0]).max() > 0 and np.array_equal(g[0], g[1])
+
+
+@pytest.mark.parametrize("precision,H,B,mb", [
+    ("fp32", 32, 255, 3), ("fp32", 32, 257, 2), ("tf32", 64, 2049, 2), ("bf16", 256, 4097, 2), ("bf16", 256, 700, 5)])
+def test_prepared_advantage_sums_are_the_minibatch_calls(precision, H, B, mb):
+    """Advantages far from zero: the variance is what is left of sums 10^10 times as large, so that it shows any other
+    order of the fp64 additions.  The weights are the same bits as after the per-minibatch calls."""
+    torch = need_gpu()
+    D, A, T, N = 18, 8, 4, 2053
+    pw, vw = _weights(D, H, A, seed=5)
+    traj = _on_rollout_policy(_traj(6, T, N, D, A), pw, D, H, A)
+    traj["adv"] = (1000.0 + 0.01 * traj["adv"]).astype(np.float32)
+    traj = _dev(torch, traj)
+    a, b = (_learner(D, A, H, B, precision) for _ in range(2))
+    for q in (a, b):
+        q.set_weights(pw, vw)
+    a.update(traj, 2, mb)
+    for e in range(2):
+        for j in range(mb):
+            b.grads(traj, e, j)
+            b.apply()
+    for x, y in zip(a.get_weights(), b.get_weights()):
+        assert np.array_equal(x, y)
