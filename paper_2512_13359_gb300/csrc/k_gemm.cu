@@ -97,6 +97,14 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
   }
 }
 
+// Wait with the limit whatever the abort flag says (copies or MMAs still in flight
+// when a wait has given up: nothing may land after the CTA has left).
+__device__ __forceinline__ void wait_landed(uint64_t* b, uint32_t phase) {
+  const uint64_t t0 = tc::global_timer_ns();
+  while (!tc::mbar_test(b, phase) && tc::global_timer_ns() - t0 < kWaitLimitNs) {
+  }
+}
+
 struct TcArgs {
   int M, N, K;
   int chunks_per_split;   // K chunks of BK per CTA along z
@@ -322,7 +330,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
       const int nb = min(BN / TL::kElemsPer128, (args.N - n0 + TL::kElemsPer128 - 1) / TL::kElemsPer128);
       const uint32_t bytes = (A_MN ? na * (TL::kBK * 128) : TL::kABytes) +
                              (B_MN ? nb * (TL::kBK * 128) : TL::kBBytes);
-      for (int c = 0; c < n_chunks; ++c) {
+      int c = 0;
+      for (; c < n_chunks; ++c) {
         const int s = c % kStages;
         if (c >= kStages &&
             !tc::mbar_wait(&bar->empty[s], (uint32_t)((c / kStages) - 1) & 1u, abort, kWaitLimitNs))
@@ -347,6 +356,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
                         &bar->full[s]);
         }
       }
+      if (*abort)   // the copies still in flight
+        for (int s = 0; s < kStages; ++s) {
+          const int fills = c / kStages + (s < c % kStages ? 1 : 0);
+          if (fills > 0) wait_landed(&bar->full[s], (uint32_t)(fills - 1) & 1u);
+        }
     }
     __syncwarp();
   } else if (warp == kIssuer) {
@@ -384,6 +398,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         tc::mma_commit(&bar->empty[s]);
       }
       tc::mma_commit(&bar->acc_full);
+      wait_landed(&bar->acc_full, 0);   // tensor memory is freed below
     }
     __syncwarp();
   } else {
@@ -502,13 +517,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void*
                    reinterpret_cast<uint64_t>(map)),
                "r"(tc::smem_u32(src)), "r"(x), "r"(y)
                : "memory");
-}
-
-// Wait with the limit whatever the abort flag says (copies still in flight).
-__device__ __forceinline__ void wait_landed(uint64_t* b, uint32_t phase) {
-  const uint64_t t0 = tc::global_timer_ns();
-  while (!tc::mbar_test(b, phase) && tc::global_timer_ns() - t0 < kWaitLimitNs) {
-  }
 }
 
 template <bool TF32, bool B_MN, int BN>
@@ -657,7 +665,9 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       const bool direct_aux = args.epi == kEpiDtanh && !box_aux && live;
       float h[32];
       if (direct_aux) load_aux32(args, (size_t)row, n0 + (warp >> 2) * 32, h);
-      ok = tc::mbar_wait(&bar->acc_full[item & 1], (uint32_t)(item / 2) & 1u, abort, kWaitLimitNs);
+      // (a wait that gave up is the whole warp's: what follows is warp-wide)
+      ok = __all_sync(0xFFFFFFFFu, tc::mbar_wait(&bar->acc_full[item & 1], (uint32_t)(item / 2) & 1u, abort,
+                                                 kWaitLimitNs));
       if (!ok) break;
       tc::tc_fence_after();
 #pragma unroll 1
@@ -676,7 +686,7 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             acc[q] = __float_as_uint(__uint_as_float(acc[q]) + __uint_as_float(b[q]));
         }
         if (box_aux) {
-          ok = tc::mbar_wait(&bar->aux[warp], aux_phase, abort, kWaitLimitNs);
+          ok = __all_sync(0xFFFFFFFFu, tc::mbar_wait(&bar->aux[warp], aux_phase, abort, kWaitLimitNs));
           if (!ok) break;
           aux_phase ^= 1u;
           aux_sent = false;
