@@ -29,7 +29,9 @@ namespace auv {
 // would not come back) and before its first access to global memory: it lets
 // the next kernel come and waits until the previous ones are complete, their
 // writes visible.  Returns zero, which the compiler does not know: addresses
-// that include it cannot be read ahead of the wait.
+// that include it cannot be read ahead of the wait.  What the previous kernels
+// write is read by ordinary loads: a constant one (.nc, __ldg) promises data that
+// does not change while the kernel is resident.
 __device__ __forceinline__ int pdl_enter() {
   int zero;
   asm volatile(

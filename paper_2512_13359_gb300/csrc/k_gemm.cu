@@ -131,8 +131,10 @@ __device__ __forceinline__ void st_f32x8(float* p, const uint32_t* v) {
                : "memory");
 }
 
+// (not .nc: a kernel that starts ahead of its predecessor's end may be resident
+// while that one writes the array)
 __device__ __forceinline__ void ld_f32x8(const float* p, float* v) {
-  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
       : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
       : "l"(p));
 }
@@ -209,21 +211,19 @@ __device__ __forceinline__ void store32(const TcArgs& a, const uint32_t (&acc)[3
 }
 
 // The tanh' activations of one row's 32 columns from nb (0 beyond N), all in
-// flight at once.
+// flight at once.  row includes pdl_enter()'s zero, so that no load comes ahead
+// of its wait.
 __device__ __forceinline__ void load_aux32(const TcArgs& a, size_t row, int nb, float (&h)[32]) {
   if (a.aux_vec && nb + 32 <= a.N) {
     if (a.c_bf16) {
-      const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.aux) +
-                                                      row * a.ld_aux + nb);
-      uint4 u[4];
+      const uint16_t* p = static_cast<const uint16_t*>(a.aux) + row * a.ld_aux + nb;
+      float w[16];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) u[g] = __ldg(p + g);
+      for (int g = 0; g < 2; ++g) ld_f32x8(reinterpret_cast<const float*>(p + 16 * g), w + 8 * g);
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const uint32_t w[4] = {u[g].x, u[g].y, u[g].z, u[g].w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          h[8 * g + j] = __uint_as_float(j & 1 ? w[j >> 1] & 0xFFFF0000u : w[j >> 1] << 16);
+      for (int j = 0; j < 32; ++j) {
+        const uint32_t u = __float_as_uint(w[j >> 1]);
+        h[j] = __uint_as_float(j & 1 ? u & 0xFFFF0000u : u << 16);
       }
     } else {
       const float* p = static_cast<const float*>(a.aux) + row * a.ld_aux + nb;
@@ -317,7 +317,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  pdl_enter();   // after the allocation: the next kernel's may not come first
+  const int zero = pdl_enter();   // after the allocation: the next kernel's may not come first
   const uint32_t tmem = bar->tmem_base;
   const uint32_t s_base = tc::smem_u32(smem);
 
@@ -403,7 +403,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     __syncwarp();
   } else {
     // ---- epilogue: one row per thread, BN columns in chunks of 32 ----
-    const int row = m0 + tid;
+    const int row = m0 + tid + zero;
     const bool epi = args.epi != kEpiNone && !args.ws && row < args.M;
     const bool dtanh = epi && args.epi == kEpiDtanh;
     // tanh': a chunk's activations are loaded while the accumulator is still
@@ -560,7 +560,7 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  pdl_enter();   // after the allocation: the next kernel's may not come first
+  const int zero = pdl_enter();   // after the allocation: the next kernel's may not come first
   const uint32_t tmem = bar->tmem_base;
 
   if (warp == kProducer) {
@@ -660,7 +660,7 @@ k_gemm_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if (box_aux && m_first < tiles_m) fetch_aux(m_first, warp >> 2);
     int item = 0;
     for (int m = m_first; m < tiles_m; m += m_step, ++item) {
-      const int row = m * kBM + rw + lane;
+      const int row = m * kBM + rw + lane + zero;
       const bool live = row < args.M;
       const bool direct_aux = args.epi == kEpiDtanh && !box_aux && live;
       float h[32];
@@ -1292,8 +1292,8 @@ constexpr int kRedGroups = 8;
 constexpr int kRedQuads = 32;
 __device__ __forceinline__ void reduce_block(long block, int M, int N, int splits,
                                              const float* __restrict__ ws, int m_pad, int n_pad, void* C,
-                                             int ldc, int c_bf16, float beta, int epi,
-                                             const void* __restrict__ aux, int ld_aux) {
+                                             int ldc, int c_bf16, float beta, int epi, const void* aux,
+                                             int ld_aux) {
   __shared__ float4 part[kRedGroups][kRedQuads];
   const int lane = threadIdx.x % kRedQuads, grp = threadIdx.x / kRedQuads;
   const int qpr = (N + 3) / 4;   // groups of four per row (n_pad is a multiple of 32)
@@ -1361,7 +1361,7 @@ __device__ __forceinline__ void reduce_block(long block, int M, int N, int split
 
 __global__ void __launch_bounds__(kRedGroups * kRedQuads)
 k_reduce(int M, int N, int splits, const float* __restrict__ ws, int m_pad, int n_pad, void* C,
-         int ldc, int c_bf16, float beta, int epi, const void* __restrict__ aux, int ld_aux) {
+         int ldc, int c_bf16, float beta, int epi, const void* aux, int ld_aux) {
   reduce_block(blockIdx.x + pdl_enter(), M, N, splits, ws, m_pad, n_pad, C, ldc, c_bf16, beta, epi, aux, ld_aux);
 }
 

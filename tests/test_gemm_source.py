@@ -33,3 +33,17 @@ def test_a_warp_gives_up_whole(kernel):
     assert "tmem_ld32" in epilogue
     for m in re.finditer(r"[^;]*mbar_wait\([^;]*;\s*if \(!([^;]*)\) break;", epilogue):
         assert "__all_sync" in m.group(0), m.group(0)
+
+
+def test_reads_stay_behind_the_wait_for_the_previous_kernel():
+    """A kernel that may start while its predecessor runs takes no operand by a read that the compiler may move ahead of
+    the wait, or that may be served from a cache that the predecessor's stores bypass: addresses carry pdl_enter()'s
+    zero, and no load is of the constant kind (.nc, __ldg)."""
+    assert not re.search(r"(?m)^\s*pdl_enter\(\);", SRC)
+    for kernel in ("k_gemm_tc", "k_gemm_rows"):
+        assert re.search(r"\bint row = [^;]*\+ zero;", _body(kernel)), kernel
+    tensor = SRC[:SRC.index("// fp32 on the CUDA cores.")] + SRC[SRC.index("void reduce_block("):]
+    assert ".nc." not in tensor and "__ldg" not in tensor
+    for name in ("reduce_block", "k_reduce"):
+        head = SRC[SRC.index(name + "("):]
+        assert "__restrict__ aux" not in head[:head.index("{")], name
