@@ -590,7 +590,8 @@ int env_adjoint(auv_env* env, int T, const float* act, const float* coef, const 
  * AUV_ADJOINT_MAX_SUBSTEPS substeps, hidden a multiple of 8 up to 1024.
  * The first call at a given (N, T) allocates the window's workspace
  * (activations of every step: about T N (2 hidden + 80) floats; and the layer
- * gradients of one step, or of as many steps as fit 1 GiB).
+ * gradients of as many steps as fit 1 GiB, of fewer if that cannot be had, of
+ * one at least).
  */
 int env_shac_window(auv_env* env, const float* policy, const float* value, int T,
                     const float* coef, float coef_V, uint32_t precision, float* grad,

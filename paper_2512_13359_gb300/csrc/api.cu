@@ -52,6 +52,7 @@ struct auv_env {
   // first use.
   char* shac_ws = nullptr;
   size_t shac_ws_bytes = 0;
+  size_t shac_group;        // bytes of a group's layer gradients, at most
   int shac_T = 0;
 };
 
@@ -379,6 +380,7 @@ int env_create(const auv_config* cfg, const auv_buffers* buf, auv_env** out) {
   if (!env) return fail(nullptr, AUV_ERR_INVALID, "out of host memory");
   std::memset(env, 0, sizeof(*env));
   env->last_copy = -1;
+  env->shac_group = (size_t)1 << 30;
   env->cfg = *cfg;
   env->model = build_model(cfg);
   env->buf.state = buf->state;
@@ -811,23 +813,31 @@ int env_shac_window(auv_env* env, const float* policy, const float* value, int T
       (rc = map_output(env, done_out, "done_out", 1, &done)))
     return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const auv::shac::Layout L = auv::shac::layout(env->model.n, T, H, is_paper(&env->cfg));
+  auto layout = [&] { return auv::shac::layout(env->model.n, T, H, is_paper(&env->cfg), env->shac_group); };
+  auv::shac::Layout L = layout();
   if (L.bytes > env->shac_ws_bytes || T != env->shac_T) {
+    env->shac_T = 0;
+    cudaError_t e;
     if (L.bytes > env->shac_ws_bytes) {
       if (env->shac_ws) {
-        cudaError_t e = cudaFree(env->shac_ws);
+        e = cudaFree(env->shac_ws);
         env->shac_ws = nullptr;
         env->shac_ws_bytes = 0;
         if (e != cudaSuccess) return cuda_fail(env, e, "free SHAC workspace");
       }
-      cudaError_t e = cudaMalloc(&env->shac_ws, L.bytes);
+      // fewer steps in a group where the device has no room for a full one
+      while ((e = cudaMalloc(&env->shac_ws, L.bytes)) == cudaErrorMemoryAllocation && L.G > 1) {
+        cudaGetLastError();
+        env->shac_group /= 4;
+        L = layout();
+      }
       if (e != cudaSuccess) {
         env->shac_ws = nullptr;
         return cuda_fail(env, e, "cudaMalloc(SHAC workspace)");
       }
       env->shac_ws_bytes = L.bytes;
     }
-    cudaError_t e = auv::shac::init(L, env->shac_ws, s);
+    e = auv::shac::init(L, env->shac_ws, s);
     if (e != cudaSuccess) return cuda_fail(env, e, "initialise SHAC workspace");
     env->shac_T = T;
   }

@@ -79,8 +79,9 @@ struct Layout {
       o_wp, o_wv, o_gp, o_sc, o_gws, gws_bytes, bytes;
 };
 // paper: the paper model (input 12, head 12, 61 adjoint rows), else Fossen
-// (18, 16, 13).
-Layout layout(int n, int T, int H, bool paper);
+// (18, 16, 13).  group_bytes: room for a group's layer gradients (one step's at
+// least).
+Layout layout(int n, int T, int H, bool paper, size_t group_bytes);
 cudaError_t init(const Layout& L, char* base, cudaStream_t s);
 // Returns AUV_OK or an AUV_ERR_* code with err set.
 int run_window(const Model& M, const Buffers& B, Status* st, const Layout& L,

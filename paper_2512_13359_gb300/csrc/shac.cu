@@ -20,8 +20,8 @@
 // for 65,536 envs x 32 steps (tf32), 4.69 -> 4.57 ms for 4,096 of the paper's
 // model (fp32).  The weight gradients
 // sum over steps as well as envs, so they wait for a group of steps whose
-// layer gradients fit 1 GiB and then run as three products over all of its
-// rows: one per step each was a sixth of the group's work per launch, with its
+// layer gradients fit 1 GiB (less, where the device has no room for that) and
+// then run as three products over all of its rows: one per step each was a sixth of the group's work per launch, with its
 // own split-K partials (65,536 envs x 32 steps, tf32: a quarter of the
 // window's time).  The terminal critic seeds lam with
 // coef_V dV(o(x_T))/dx_T through the value network's input gradient.
@@ -62,7 +62,7 @@ constexpr int kLdv = 8;    // value head row
 
 }  // namespace
 
-Layout layout(int n, int T, int H, bool paper) {
+Layout layout(int n, int T, int H, bool paper, size_t group_bytes) {
   Layout L;
   L.n = n;
   L.T = T;
@@ -86,7 +86,7 @@ Layout layout(int n, int T, int H, bool paper) {
   L.o_H2 = take(T * N * L.Hp * 4);
   L.o_Y = take(T * N * kLdy * 4);
   // dL/dZ2, dL/dZ1 and dL/dY of the steps whose weight gradients run together
-  const size_t group = ((size_t)1 << 30) / (N * (2 * (size_t)H + kLdy) * 4);
+  const size_t group = group_bytes / (N * (2 * (size_t)H + kLdy) * 4);
   L.G = (int)std::max<size_t>(1, std::min<size_t>(group, (size_t)T));
   L.o_G2 = take(L.G * N * H * 4);
   L.o_G1 = take(L.G * N * H * 4);

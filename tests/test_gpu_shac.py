@@ -298,3 +298,71 @@ def test_shac_window_tf32(oracle):
     jerr = np.abs(to_np(J) - Jr).max() / np.abs(Jr).max()
     print(f"[shac tf32] projected {worst:.3e}, J {jerr:.3e}")
     assert worst <= 5e-4 and jerr <= 5e-4        # measured 2.4e-5, 1.1e-5
+
+
+def _gradient(torch, w, T, precision="fp32"):
+    """Gradient and objectives of a window with a terminal critic from the envs' reset states."""
+    env = make_env(w, policy=False)
+    env.reset()
+    pw, vw = (torch.from_numpy(x).cuda() for x in (W.policy_weights(w, 0.05), W.value_weights(w, 0.1)))
+    coef = torch.full((T,), 1e-4, device="cuda")
+    grad, J = torch.empty_like(pw), torch.empty(w["n_envs"], device="cuda")
+    env.shac_window(pw, vw, coef, 1e-4, grad, J=J, precision=precision)
+    assert env.status().code == 0
+    env.close()
+    return to_np(grad).astype(np.float64), to_np(J)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32"])
+def test_shac_window_of_several_groups_of_steps(precision):
+    """A gradient is the sum of its env shards': 36,000 envs of width 256 take their 16 steps' weight gradients in two
+    groups (14 steps fit 1 GiB), shards of 12,000 in one.  The sums differ by their order (and the closed loop carries
+    the forward's: at most TF32's rounding of its operands, 2^-11, in tf32); a step left out or taken twice is a
+    sixteenth of the gradient."""
+    torch = need_gpu()
+    n, T, shards = 36000, 16, 3
+    w = W.workload("ppo_65536", n_envs=n, hidden=256, mlp="fp32")
+    grad, J = _gradient(torch, w, T, precision)
+    parts = [_gradient(torch, dict(w, n_envs=n // shards, env_id_base=r * (n // shards)), T, precision)
+             for r in range(shards)]
+    total = sum(p[0] for p in parts)
+    err = np.linalg.norm(grad - total) / np.linalg.norm(total)
+    print(f"[shac groups {precision}] {err:.2e}")
+    assert err <= {"fp32": 1e-5, "tf32": 2.0 ** -11}[precision]
+    assert np.abs(J - np.concatenate([p[1] for p in parts])).max() <= 1e-3 * np.abs(J).max()
+
+
+def test_shac_window_where_a_full_group_does_not_fit():
+    """The device has room for the window and a few steps' layer gradients, not for 1 GiB of them: the window runs, in
+    more groups."""
+    torch = need_gpu()
+    n, T = 36000, 16
+    w = W.workload("ppo_65536", n_envs=n, hidden=256, mlp="fp32")
+    _gradient(torch, dict(w, n_envs=64), T)   # (modules and torch's own allocations)
+    torch.cuda.synchronize()
+    probe = make_env(w, policy=False)
+    probe.reset()
+    pw, vw = (torch.from_numpy(x).cuda() for x in (W.policy_weights(w, 0.05), W.value_weights(w, 0.1)))
+    coef, grad = torch.full((T,), 1e-4, device="cuda"), torch.empty_like(pw)
+    before = torch.cuda.mem_get_info()[0]
+    probe.shac_window(pw, vw, coef, 1e-4, grad)
+    torch.cuda.synchronize()
+    want, need = to_np(grad).astype(np.float64), before - torch.cuda.mem_get_info()[0]
+    probe.close()
+    assert need > 1 << 30
+    env = make_env(w, policy=False)
+    env.reset()
+    torch.cuda.synchronize()
+    room = need - (512 << 20)   # half a full group
+    hold = []
+    while (free := torch.cuda.mem_get_info()[0]) > room + (8 << 20):
+        hold.append(torch.empty(min(free - room, 64 << 30), dtype=torch.uint8, device="cuda"))
+    try:
+        env.shac_window(pw, vw, coef, 1e-4, grad)
+        assert env.status().code == 0
+        got = to_np(grad).astype(np.float64)
+    finally:
+        del hold
+        env.close()
+        torch.cuda.empty_cache()
+    assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
