@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 TOL = {"bf16": 1e-5, "tf32": 3e-3, "fp32": 1e-5}
 
 
-def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=3):
+def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=3, beta=0.0):
     from paper_2512_13359_gb300 import auvenv
     g = torch.Generator(device="cuda").manual_seed(M + 3 * N + 7 * K)
     dt = torch.bfloat16 if prec == "bf16" else torch.float32
@@ -31,8 +31,13 @@ def run(torch, prec, M, N, K, a_mn, b_mn, c_bf16=False, pad_a=0, pad_b=0, pad_c=
     B, ldb, b = operand(N, b_mn, pad_b)
     C = torch.full((M, N + pad_c), 7.0, device="cuda", dtype=torch.bfloat16 if c_bf16 else torch.float32)
     ws = torch.empty(auvenv.lib().auv_gemm_workspace_bytes(M, N, K) // 4 + 1, device="cuda")
-    st = auvenv.gemm(prec, M, N, K, A, lda, a_mn, B, ldb, b_mn, C, N + pad_c, 0.0, ws)
+    if beta:
+        C[:, :N] = torch.randn((M, N), generator=g, device="cuda")
+    c0 = C[:, :N].double()
+    st = auvenv.gemm(prec, M, N, K, A, lda, a_mn, B, ldb, b_mn, C, N + pad_c, beta, ws)
     ref, scale = a @ b.T, a.abs() @ b.abs().T
+    if beta:
+        ref, scale = ref + beta * c0, scale + abs(beta) * c0.abs()
     tol = TOL[prec] * scale + 1e-30 + (2.0 ** -8 * ref.abs() if c_bf16 else 0.0)
     assert st.cpu().tolist() == [0, 0, 0, 0]
     assert bool(((C[:, :N].double() - ref).abs() <= tol).all())
@@ -57,6 +62,18 @@ def test_wide_tiles(prec, c_bf16, b_mn):
     for rows in (128 * (sms // 2), 128 * (sms // 2) + 1, 128 * 2 * sms + 5):
         run(torch, prec, rows, 250, 40, False, b_mn, c_bf16)
         run(torch, prec, rows, 252, 40, False, b_mn, c_bf16, pad_c=4)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "tf32"])
+@pytest.mark.parametrize("c_bf16", [False, True])
+@pytest.mark.parametrize("N", [16, 33, 128, 255, 256])
+@pytest.mark.parametrize("pad_c", [0, 1, 8])
+def test_result_added_to_what_is_there(prec, c_bf16, N, pad_c):
+    """beta, and rows of C off 16 bytes: columns read and written by a warp together, 8 rows at a time, the last tile 1,
+    7, 8 or 9 rows of its warp's 32."""
+    for M in (1025, 1024 + 39, 1024 + 72, 1024 + 105):
+        for beta in (0.0, -0.5):
+            run(need_gpu(), prec, M, N, 40, False, N % 2 == 1, c_bf16, pad_c=pad_c, beta=beta)
 
 
 @pytest.mark.parametrize("M,N,K", [(256, 264, 5000), (16, 264, 32 * 9 + 1), (130, 24, 33), (1, 1, 1), (33, 290, 700)])
