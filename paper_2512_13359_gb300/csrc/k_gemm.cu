@@ -990,13 +990,14 @@ struct F32Tile {
 
 // A BM x BN tile per CTA, TM x 8 outputs per thread, three slices in flight.
 // SEG: every split's chain in turn, its sum added to the total (blockIdx.z is
-// 0); else one split per blockIdx.z.  128 x 128 tiles for products that fill
-// the SMs (128 x 96 for 264 columns), 64 x 64 for batches of a few thousand
-// rows, 16 x 128 for the heads' weight gradients.  FMA issue and shared-memory
-// reads bound them (about half of the FP32 peak: 65,536 x 256 x 256 202 us).
-// Against scalar loads through registers: 256 x 264 x 131,072 1,090 -> 590 us,
-// 12 x 264 x 131,072 270 -> 90 us, 4,096 x 256 x 264 (five splits) 27 us and a
-// 14 us reduction -> 26 us.
+// 0); else one split per blockIdx.z.  FMA issue and shared-memory reads bound
+// them (half to two thirds of the FP32 peak).  64 x 64 tiles, three CTAs an SM,
+// serve most shapes: the 8 x 8 outputs of a 128 x 128 tile's thread leave few
+// registers, which K-major rows read four k at a time spill, and two CTAs an SM
+// finish in coarse waves (launch_fp32_any has the lines).  16- and 32-row tiles
+// for the heads' weight gradients.  Against scalar loads through registers:
+// 256 x 264 x 30,011 175 -> 113 us, 12 x 264 x 131,072 270 -> 90 us,
+// 4,096 x 256 x 264 (five splits) 27 us and a 14 us reduction -> 26 us.
 template <int BM, int BN, bool A_MN, bool B_MN, bool VEC, bool SEG>
 __global__ void __launch_bounds__((F32Tile<BM, BN>::kThreads), (BM >= 128 ? 2 : 3))
 k_gemm_fp32(const F32Args args) {
@@ -1057,6 +1058,83 @@ k_gemm_fp32(const F32Args args) {
       if (SEG) x = !tail ? total[SEG ? i : 0][SEG ? j : 0] : (first ? x : total[SEG ? i : 0][SEG ? j : 0] + x);
       f32_store(args, blockIdx.z, m0 + f32_row<TY, A_MN>(ty, i), n0 + f32_row<TX, B_MN>(tx, j), x);
     }
+}
+
+// Large products with rows off 16 bytes, which cp.async can only copy float by
+// float: a 128 x 128 tile per CTA, 8 x 8 outputs per thread, slices of 8 k
+// through registers into two buffers of [k][row] whichever way the operands are
+// stored (rows padded by 4 floats: the K-major stores, 8 k of 4 rows per warp,
+// land in 32 distinct banks).  30,011 x 1,024 x 1,032 from odd rows: 1.43 to
+// 1.47 ms, 1.67 to 1.72 in 64 x 64 tiles.
+template <bool A_MN, bool B_MN>
+__global__ void __launch_bounds__(256, 2) k_gemm_fp32_regs(const F32Args args) {
+  __shared__ __align__(16) float As[2][8][132];
+  __shared__ __align__(16) float Bs[2][8][132];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int m0 = blockIdx.x * 128, n0 = blockIdx.y * 128;
+  const int k_begin = blockIdx.z * args.seg, k_end = min(args.K, k_begin + args.seg);
+  // element e of a 128 x 8 slice, consecutive threads along the stored index
+  auto coord = [](int e, bool mn, int& r, int& kk) {
+    r = mn ? e % 128 : e >> 3;
+    kk = mn ? e / 128 : e & 7;
+  };
+  auto load = [&](const float* X, int ld, bool mn, int r0, int R, int kb, float (&v)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      int r, kk;
+      coord(tid + 256 * q, mn, r, kk);
+      const int rr = r0 + r, k = kb + kk;
+      v[q] = rr < R && k < k_end ? __ldg(mn ? X + (size_t)k * ld + rr : X + (size_t)rr * ld + k) : 0.0f;
+    }
+  };
+  auto store = [&](float (&S)[8][132], bool mn, const float (&v)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      int r, kk;
+      coord(tid + 256 * q, mn, r, kk);
+      S[kk][r] = v[q];
+    }
+  };
+  float acc[8][8] = {}, va[4], vb[4];
+  load(args.A, args.lda, A_MN, m0, args.M, k_begin, va);
+  load(args.B, args.ldb, B_MN, n0, args.N, k_begin, vb);
+  store(As[0], A_MN, va);
+  store(Bs[0], B_MN, vb);
+  __syncthreads();
+  int buf = 0;
+  for (int kb = k_begin; kb < k_end; kb += 8) {
+    const bool more = kb + 8 < k_end;
+    if (more) {   // the next slice in flight during this one
+      load(args.A, args.lda, A_MN, m0, args.M, kb + 8, va);
+      load(args.B, args.ldb, B_MN, n0, args.N, kb + 8, vb);
+    }
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      float a[8], b[8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 u = *reinterpret_cast<const float4*>(&As[buf][kk][64 * h + ty * 4]);
+        const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 * h + tx * 4]);
+        a[4 * h] = u.x, a[4 * h + 1] = u.y, a[4 * h + 2] = u.z, a[4 * h + 3] = u.w;
+        b[4 * h] = v.x, b[4 * h + 1] = v.y, b[4 * h + 2] = v.z, b[4 * h + 3] = v.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    if (more) {
+      store(As[buf ^ 1], A_MN, va);
+      store(Bs[buf ^ 1], B_MN, vb);
+    }
+    __syncthreads();
+    buf ^= 1;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      f32_store(args, blockIdx.z, m0 + f32_row<16, true>(ty, i), n0 + f32_row<16, true>(tx, j), acc[i][j]);
 }
 
 // Narrow or few tiles: each warp computes a 32 x 32 block over one split with
@@ -1542,9 +1620,9 @@ struct Plan {
   int segments;          // fp32: splits added inside the kernel (1: none)
 };
 
-// fp32 kernels: 128 x 128 tiles (partials in the workspace when split), 64 x
-// 64 tiles, the same with the splits in turn, or a warp per 32 x 32 block.
-enum Fp32Kernel { kFp32Large, kFp32Small, kFp32Seg, kFp32Warps };
+// fp32 kernels: a tile per CTA (partials in the workspace when split), the same
+// with the splits in turn, or a warp per 32 x 32 block.
+enum Fp32Kernel { kFp32Tiles, kFp32Seg, kFp32Warps };
 
 constexpr int kRowsMaxChunks = RowTile<true, false, 128>::kMaxChunks;
 
@@ -1555,7 +1633,7 @@ Plan plan(Prec prec, int M, int N, int K, bool a_kmajor) {
   Plan p;
   p.rows = false;
   p.half = 0;
-  p.fp32 = kFp32Large;
+  p.fp32 = kFp32Tiles;
   p.segments = 1;
   if (prec == kFp32) {
     p.bm = M <= 32 ? 32 : 128;
@@ -1588,16 +1666,18 @@ Plan plan(Prec prec, int M, int N, int K, bool a_kmajor) {
   p.splits = (p.chunks + p.per_split - 1) / p.per_split;
   if (prec == kFp32 && a_kmajor && p.splits <= 8) {
     // A product over rows: its few splits are added inside the kernel instead
-    // of through partials in memory (4,096 x 256 x 264, five splits: 27 us and
-    // a 14 us reduction).  A warp per block where the result is narrow or 64 x
-    // 64 tiles would leave SMs idle.
+    // of through partials in memory (4,096 x 256 x 264, five splits: 27 us and a
+    // 14 us reduction).  A warp per block where the result is narrow or 64 x 64
+    // tiles would leave SMs idle; a tile with the splits in turn while their
+    // chain is short (4,096 x 256 x 512 41 to 43 us, 45 to 47 as partials; but
+    // 4,096 x 512 x 520 103 us, 83, and 1,024^3 76 to 81 us, 69).
     const long small = (long)((M + 63) / 64) * ((N + 63) / 64);
-    const int all = sm_count_dev();
-    p.segments = p.splits;
-    if (N <= 32 || (p.splits > 1 && small < all)) p.fp32 = kFp32Warps;
-    else if (p.splits > 1) p.fp32 = kFp32Seg;
-    else if (tiles < 2 * all) p.fp32 = kFp32Small;
-    p.splits = 1;
+    const bool warps = N <= 32 || (p.splits > 1 && small < sm_count_dev());
+    if (warps || p.splits == 1 || K <= 512) {
+      p.segments = p.splits;
+      p.fp32 = warps ? kFp32Warps : (p.splits > 1 ? kFp32Seg : kFp32Tiles);
+      p.splits = 1;
+    }
   }
   if (p.rows) {   // nine chunks or fewer: at most two splits
     p.half = p.splits > 1 ? p.per_split : 0;
@@ -1672,8 +1752,10 @@ cudaError_t launch_fp32_tile(const Plan& P, const F32Args& a, cudaStream_t s) {
   using TL = F32Tile<BM, BN>;
   auto kern = k_gemm_fp32<BM, BN, A_MN, B_MN, VEC, SEG>;
   constexpr int smem = TL::template smem_floats<A_MN, B_MN>() * 4;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  if constexpr (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+  }
   kern<<<dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, SEG ? 1 : P.splits), TL::kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -1688,6 +1770,24 @@ cudaError_t launch_fp32_warps(const Plan& P, const F32Args& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <bool A_MN, bool B_MN>
+cudaError_t launch_fp32_regs(const Plan& P, const F32Args& a, cudaStream_t s) {
+  k_gemm_fp32_regs<A_MN, B_MN><<<dim3((a.M + 127) / 128, (a.N + 127) / 128, P.splits), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+// 64 x 64 tiles, but
+//  - up to 32 rows: tiles of 16 or 32 (24 x 264 x 30,000: 35 us, 62 in 128 rows);
+//  - 128 x 128 tiles: an MN-major A in three waves of them or more (30,011 x
+//    1,024 x 1,032 1.18 to 1.27 ms, 1.28 to 1.33 in 64 x 64 tiles; but 30,011 x
+//    256 x 264, 1.5 waves, 109 to 111 us, 97 to 99, and with a K-major A 122 to
+//    140 us, 103 to 105), or just one full wave of whole ones (128 x 128 x
+//    128,000 92 to 103 us, 101 to 109);
+//  - many rows of 257 to 288 columns: three column tiles of 96 instead of five of
+//    64 (30,011 x 264 x 256: 107 to 111 us, 113 to 117);
+//  - large products off 16 bytes: through registers (65,536 x 256 x 264 225 to 230
+//    us, 249 to 263 in 64 x 64 tiles; below half of that size the tiles are as
+//    fast or faster: 30,011 x 129 x 264 117 to 119 us, 95 to 98).
 template <bool A_MN, bool B_MN, bool VEC>
 cudaError_t launch_fp32_any(const Plan& P, const F32Args& a, cudaStream_t s) {
   if constexpr (!A_MN) {
@@ -1695,10 +1795,20 @@ cudaError_t launch_fp32_any(const Plan& P, const F32Args& a, cudaStream_t s) {
     if (P.fp32 == kFp32Seg) return launch_fp32_tile<64, 64, A_MN, B_MN, VEC, true>(P, a, s);
   }
   if (a.M <= 16) return launch_fp32_tile<16, 128, A_MN, B_MN, VEC, false>(P, a, s);
-  if (P.fp32 == kFp32Small) return launch_fp32_tile<64, 64, A_MN, B_MN, VEC, false>(P, a, s);
-  // 264 augmented columns: three tiles of 96 instead of three of 128
-  if (a.N > 256 && a.N <= 288) return launch_fp32_tile<128, 96, A_MN, B_MN, VEC, false>(P, a, s);
-  return launch_fp32_tile<128, 128, A_MN, B_MN, VEC, false>(P, a, s);
+  if (a.M <= 32) return launch_fp32_tile<32, 128, A_MN, B_MN, VEC, false>(P, a, s);
+  const int sms = sm_count_dev();
+  const long ctas = (long)((a.M + 127) / 128) * ((a.N + 127) / 128) * P.splits;   // of 128 x 128 tiles
+  const bool whole = a.M % 128 == 0 && a.N % 128 == 0 && ctas <= 2 * sms && ctas > 2 * sms * 9 / 10;
+  if constexpr ((A_MN && B_MN) || (VEC && (A_MN || B_MN))) {
+    if (whole || (A_MN && ctas > 6 * sms)) return launch_fp32_tile<128, 128, A_MN, B_MN, VEC, false>(P, a, s);
+  }
+  if constexpr (VEC) {
+    if (a.N > 256 && a.N <= 288 && a.M >= 128 * sms) return launch_fp32_tile<128, 96, A_MN, B_MN, VEC, false>(P, a, s);
+  } else if constexpr (!(A_MN && B_MN)) {
+    const long tiles = (long)((a.M + 63) / 64) * ((a.N + 63) / 64);
+    if (whole || (P.splits == 1 && tiles * a.K >= 500000)) return launch_fp32_regs<A_MN, B_MN>(P, a, s);
+  }
+  return launch_fp32_tile<64, 64, A_MN, B_MN, VEC, false>(P, a, s);
 }
 
 cudaError_t launch_fp32(const Plan& P, const F32Args& a, bool a_mn, bool b_mn, cudaStream_t s) {

@@ -89,11 +89,16 @@ def test_tf32_along_samples(M, N, K, pad_a, pad_b):
     (20011, 24, 256, False), (300, 32, 24, False),                         # a warp per block, no split
     (4090, 256, 264, False), (2500, 260, 40, False),                       # 64-wide tiles, splits in turn
     (9800, 256, 24, False), (2003, 250, 17, False), (20000, 250, 264, False),  # 64- and 128-wide tiles
-    (40, 50, 2001, False), (12, 264, 5003, True), (16, 100, 24, True), (260, 264, 3000, True), (50, 24, 33, True)])
+    (40, 50, 2001, False), (12, 264, 5003, True), (16, 100, 24, True), (260, 264, 3000, True), (50, 24, 33, True),
+    (17, 70, 4001, True), (32, 264, 3000, False), (33, 130, 3000, True),       # 32-row tiles and one row more
+    (2100, 260, 512, False), (2100, 260, 520, False),                          # the splits' chain: in turn, as partials
+    (19457, 288, 40, False), (19456, 257, 9, True), (19456, 289, 9, True),     # column tiles of 96
+    (128, 128, 128 * 304 * 4, True), (256, 256, 9000, True), (39000, 256, 9, True),   # 128-wide tiles of an MN-major A
+    (8000, 1030, 264, False), (8000, 1030, 260, True)])                        # through registers when off 16 bytes
 @pytest.mark.parametrize("b_mn", [False, True])
 @pytest.mark.parametrize("pad", [0, 1])
 def test_fp32_kernels(M, N, K, a_mn, b_mn, pad):
-    run(need_gpu(), "fp32", M, N, K, a_mn, b_mn, False, pad, pad)
+    run(need_gpu(), "fp32", M, N, K, a_mn, b_mn, False, pad, pad, beta=0.5 if M % 2 else 0.0)
 
 
 @pytest.mark.parametrize("M", [1024, 5000, 40000])
