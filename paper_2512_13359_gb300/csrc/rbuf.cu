@@ -13,18 +13,20 @@
 // Sampling draws indices from a counter-based generator (Philox4x32-10 at
 // counter (b, 0x52420000, draw), key = seed; index = floor(word * size /
 // 2^32)) and gathers the rows.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <new>
 
+#include "auv_bf16.h"
 #include "auv_kernels.h"
 #include "auvenv.h"
 
 struct auv_rbuf {
   uint32_t D, A;
   uint64_t C;
-  int device;
+  int device, sms;
   char* mem;
   float *obs, *act, *rew, *next;
   uint8_t* done;
@@ -37,7 +39,7 @@ namespace auv {
 namespace {
 
 constexpr int kInThreads = 128;
-constexpr int kSteps = 8;                     // consecutive steps per block
+constexpr int kSteps = 8;                     // consecutive steps per block, at most
 constexpr int kObsTiles = 4, kActTiles = 3;   // rings in shared memory
 
 // Shared memory of an insert block: feature-major tiles, rows padded by one.
@@ -45,7 +47,7 @@ constexpr size_t insert_smem(int tile, int D, int A) {
   return sizeof(float) * (size_t)(tile + 1) * (kObsTiles * D + kActTiles * A);
 }
 
-// A block moves TILE consecutive envs of kSteps consecutive steps: the tiles'
+// A block moves TILE consecutive envs of `per` consecutive steps: the tiles'
 // feature rows are copied to shared memory as they come (cp.async, two steps
 // ahead of the one being stored), and a step's transitions leave in slot
 // order, consecutive threads on consecutive floats.  Step t + 1's observation
@@ -54,16 +56,18 @@ constexpr size_t insert_smem(int tile, int D, int A) {
 // + 8 features) took 126 us with one tile per step through registers and a
 // division per stored element, 65 us here (4.7 TB/s).
 //
-// SKIP: the first `skip` envs of step 0 are not stored, so that a call with more
+// The first `skip` envs of step 0 are not stored, so that a call with more
 // transitions than the ring has slots writes each slot once (blocks run in no
-// order): the newest C of them.
-template <int TILE, bool SKIP>
+// order): the newest C of them.  ANY: per and skip as given, else kSteps and 0
+// (known to the compiler: 65,536 x 16 transitions and a draw 80.5 us, 81.5 with
+// ANY).
+template <int TILE, bool ANY>
 __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, int A,
                                                    const float* __restrict__ obs,
                                                    const float* __restrict__ act,
                                                    const float* __restrict__ rew,
                                                    const uint8_t* __restrict__ done,
-                                                   const float* __restrict__ last_obs, int skip,
+                                                   const float* __restrict__ last_obs, int per_, int skip,
                                                    uint64_t head, uint64_t C,
                                                    float* __restrict__ s_obs,
                                                    float* __restrict__ s_act,
@@ -75,7 +79,7 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
   float* const acts = sm + kObsTiles * D * S;
   const size_t n = (size_t)N;
   const int i0 = blockIdx.x * TILE, cnt = min(TILE, N - i0);
-  const int t0 = blockIdx.y * kSteps, t1 = min(T, t0 + kSteps);
+  const int per = ANY ? per_ : kSteps, t0 = blockIdx.y * per, t1 = min(T, t0 + per);
   const int tid = threadIdx.x, lj = tid % TILE, lf = tid / TILE;   // loads: env, first feature
   auto copy_rows = [&](const float* src, int W, float* dst) {
     if (lj < cnt)
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kInThreads) k_rb_insert(int T, int N, int D, i
   for (int t = t0; t < t1; ++t) {
     float r = 0.0f;
     uint8_t d = 0;
-    const int j0 = SKIP && t == 0 ? min(max(skip - i0, 0), cnt) : 0;   // the tile's first env to store
+    const int j0 = ANY && t == 0 ? min(max(skip - i0, 0), cnt) : 0;   // the tile's first env to store
     if (tid < cnt) {
       r = __ldg(rew + (size_t)t * n + i0 + tid);
       d = __ldg(done + (size_t)t * n + i0 + tid);
@@ -372,6 +376,7 @@ int rbuf_create(uint32_t obs_dim, uint32_t act_dim, uint64_t capacity, auv_rbuf*
   r->A = act_dim;
   r->C = capacity;
   cudaGetDevice(&r->device);
+  r->sms = auv::engine_sm_count();
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t b_obs = up(capacity * obs_dim * 4), b_act = up(capacity * act_dim * 4),
                b_rew = up(capacity * 4), b_done = up(capacity);
@@ -425,13 +430,22 @@ int rbuf_insert(auv_rbuf* r, int T, int N, const float* obs, const float* act, c
   const uint64_t lost = added > r->C ? added - r->C : 0;
   const int t0 = (int)(lost / (uint64_t)N), skip = (int)(lost % (uint64_t)N), steps = T - t0;
   const size_t o = (size_t)t0 * (size_t)N;
-  auto kern = wide ? (skip ? auv::k_rb_insert<64, true> : auv::k_rb_insert<64, false>)
-                   : (skip ? auv::k_rb_insert<32, true> : auv::k_rb_insert<32, false>);
+  // Eight steps a block read each observation once, but one after the other: fewer
+  // while the blocks are under four per SM, or two rounds of those that its shared
+  // memory holds (64 envs x 200 steps of 18 + 8 floats: 16.5 us with eight, 9.5 with
+  // one; 4,096 x 16: 16.5, and 9.4).
+  const int tiles = (N + tile - 1) / tile;
+  const int64_t want = (int64_t)r->sms * std::min<int>(4, 2 * (int)(227 * 1024 / (smem + 1024)));
+  int per = auv::kSteps;
+  while (per > 1 && (int64_t)tiles * ((steps + per - 1) / per) < want) per /= 2;
+  const bool any = per != auv::kSteps || skip;
+  auto kern = wide ? (any ? auv::k_rb_insert<64, true> : auv::k_rb_insert<64, false>)
+                   : (any ? auv::k_rb_insert<32, true> : auv::k_rb_insert<32, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel attributes");
-  const dim3 grid((N + tile - 1) / tile, (steps + auv::kSteps - 1) / auv::kSteps);
+  const dim3 grid(tiles, (steps + per - 1) / per);
   kern<<<grid, auv::kInThreads, smem, static_cast<cudaStream_t>(stream)>>>(
-      steps, N, D, A, obs + o * D, act + o * A, rew + o, done + o, last_obs, skip, (r->head + o) % r->C, r->C, r->obs,
+      steps, N, D, A, obs + o * D, act + o * A, rew + o, done + o, last_obs, per, skip, (r->head + o) % r->C, r->C, r->obs,
       r->act, r->rew, r->next, r->done);
   e = cudaGetLastError();
   if (e != cudaSuccess) return rb_cuda(r, e, "insert kernel");
