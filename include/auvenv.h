@@ -507,10 +507,12 @@ int ppo_apply(auv_ppo* p, const float* grad, float* stats, void* stream);
  * the updated ones once it completes.  Each call first copies the batch into
  * a sample-major buffer (T * N rows of round8(obs_dim + act_dim + 3) floats,
  * one coalesced pass) from which every step gathers its minibatch, with 4
- * more bytes a row for the epoch's permutation; the learner allocates that buffer the first time it sees a batch of more rows
- * than the last (the one allocation after ppo_create) and frees it in
- * ppo_destroy.  If the allocation fails the steps gather from the batch's
- * own arrays.
+ * more bytes a row for the epoch's permutation; the learner allocates that
+ * buffer the first time it sees a batch of more rows than the last (the one
+ * allocation after ppo_create) and frees it in ppo_destroy.  If the
+ * allocation fails, and in epochs of fewer than four minibatches of up to
+ * 65,536 samples, which do not repay the copy, the steps gather from the
+ * batch's own arrays: the same results.
  */
 int ppo_update(auv_ppo* p, const auv_ppo_batch* batch, uint32_t epochs, uint32_t n_minibatches,
                float* stats, void* stream);

@@ -20,6 +20,13 @@ pytestmark = pytest.mark.gpu
     ("bf16", 1, 1, 32, 4, 515, 257, 8, False),      # the narrowest row
     ("bf16", 18, 8, 256, 4, 1025, 2047, 2, False),  # engine path
     ("bf16", 12, 6, 256, 4, 700, 1399, 2, True),
+    # epochs of four minibatches and more, the prepared ones: the same edges
+    ("fp32", 5, 8, 32, 3, 7, 2, 9, False),
+    ("fp32", 7, 3, 32, 8, 1237, 2049, 4, False),
+    ("fp32", 64, 8, 64, 4, 4099, 4096, 4, False),
+    ("tf32", 18, 8, 64, 9, 1012, 2277, 4, False),
+    ("bf16", 18, 8, 256, 8, 1025, 2047, 4, False),
+    ("bf16", 12, 6, 256, 8, 700, 1399, 4, True),
 ])
 def test_update_equals_minibatch_calls(precision, D, A, H, T, N, B, mb, value_only):
     torch = need_gpu()
@@ -99,12 +106,12 @@ def test_a_gradient_does_not_depend_on_its_launch(D, A, B):
 
 
 @pytest.mark.parametrize("precision,H,B,mb", [
-    ("fp32", 32, 255, 3), ("fp32", 32, 257, 2), ("tf32", 64, 2049, 2), ("bf16", 256, 4097, 2), ("bf16", 256, 700, 5)])
+    ("fp32", 32, 255, 4), ("fp32", 32, 257, 6), ("tf32", 64, 2049, 4), ("bf16", 256, 4097, 4), ("bf16", 256, 700, 5)])
 def test_prepared_advantage_sums_are_the_minibatch_calls(precision, H, B, mb):
     """Advantages far from zero: the variance is what is left of sums 10^10 times as large, so that it shows any other
     order of the fp64 additions.  The weights are the same bits as after the per-minibatch calls."""
     torch = need_gpu()
-    D, A, T, N = 18, 8, 4, 2053
+    D, A, T, N = 18, 8, 8, 2053
     pw, vw = _weights(D, H, A, seed=5)
     traj = _on_rollout_policy(_traj(6, T, N, D, A), pw, D, H, A)
     traj["adv"] = (1000.0 + 0.01 * traj["adv"]).astype(np.float32)
