@@ -345,6 +345,10 @@ int copy_batch(auv_env* env, void* const dst[4], const void* const src[4], cudaS
   }
   return AUV_OK;
 }
+auv::Fp32Nets fp32_nets(const auv_env* env) {
+  return {env->w_policy_f32, env->w_value_f32, env->w_policy_packed, env->w_value_packed};
+}
+
 }  // namespace
 
 extern "C" {
@@ -480,9 +484,7 @@ int env_set_weights(auv_env* env, const float* policy, const float* value, void*
     e = auv::launch_pack_tf32(env->model, env->w_policy_f32, env->w_policy_packed, s);
     if (e != cudaSuccess) return cuda_fail(env, e, "pack tf32 weights");
   } else {
-    e = auv::launch_pack_fp32(env->model, env->w_policy_f32, env->w_policy_packed, s);
-    if (e == cudaSuccess && value)
-      e = auv::launch_pack_fp32(env->model, env->w_value_f32, env->w_value_packed, s);
+    e = auv::launch_pack_fp32(env->model, fp32_nets(env), value != nullptr, s);
     if (e != cudaSuccess) return cuda_fail(env, e, "pack fp32 weights");
   }
   // host sources are read before return
@@ -507,10 +509,6 @@ int env_reset(auv_env* env, const uint8_t* mask, void* stream) {
 }
 
 namespace {
-
-auv::Fp32Nets fp32_nets(const auv_env* env) {
-  return {env->w_policy_f32, env->w_value_f32, env->w_policy_packed, env->w_value_packed};
-}
 
 // The kernels of T control steps from global step t_g0 (bf16 mode: the fused
 // rollout, then the value network over the observations just written).

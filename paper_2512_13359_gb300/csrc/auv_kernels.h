@@ -41,7 +41,8 @@ struct Fp32Nets {
   const void *policy_img, *value_img;
 };
 size_t fp32_image_bytes(int in_dim, int hidden);
-cudaError_t launch_pack_fp32(const Model& M, const float* w, void* img, cudaStream_t s);
+// Writes the policy's image, with `both` the value network's too.
+cudaError_t launch_pack_fp32(const Model& M, const Fp32Nets& w, bool both, cudaStream_t s);
 cudaError_t launch_rollout_fp32(const Model& M, const Buffers& B, const Fp32Nets& w, const Traj& tr,
                                 int T, uint64_t t_g0, Status* st, cudaStream_t s);
 // Networks over rows: input k of row r at obs[((r / ns) * obs_dim + k) * ns +

@@ -59,10 +59,14 @@ struct Image {
   static constexpr int kSlot = H * kWs, kW1T = H / kSlice * kSlot, kFloats = kW1T + IN * H;
 };
 
+// The images of one network or (gridDim.y = 2) both.
 template <int IN, int H>
-__global__ void k_pack_fp32(const float* __restrict__ w, float* __restrict__ img) {
+__global__ void k_pack_fp32(const float* __restrict__ w0, float* __restrict__ img0, const float* __restrict__ w1,
+                            float* __restrict__ img1) {
   using F = Flat<IN, H>;
   using I = Image<IN, H>;
+  const float* const w = blockIdx.y ? w1 : w0;
+  float* const img = blockIdx.y ? img1 : img0;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x < I::kW1T) {
     const int s = x / I::kSlot, u = x % I::kSlot / kWs, k = x % kWs;
@@ -540,8 +544,10 @@ cudaError_t rows_any(int H, const Net& p, const Net& v, const float* obs, size_t
 }
 
 template <int IN, int H>
-cudaError_t pack(const float* w, float* img, cudaStream_t s) {
-  k_pack_fp32<IN, H><<<(Image<IN, H>::kFloats + 255) / 256, 256, 0, s>>>(w, img);
+cudaError_t pack(const Fp32Nets& w, bool both, cudaStream_t s) {
+  auto img = [](const void* p) { return const_cast<float*>(static_cast<const float*>(p)); };
+  k_pack_fp32<IN, H><<<dim3((Image<IN, H>::kFloats + 255) / 256, both ? 2 : 1), 256, 0, s>>>(
+      w.policy, img(w.policy_img), w.value, img(w.value_img));
   return cudaGetLastError();
 }
 
@@ -551,11 +557,10 @@ size_t fp32_image_bytes(int in_dim, int hidden) {
   return sizeof(float) * ((size_t)hidden / kSlice * hidden * kWs + (size_t)in_dim * hidden);
 }
 
-cudaError_t launch_pack_fp32(const Model& M, const float* w, void* img, cudaStream_t s) {
-  float* f = static_cast<float*>(img);
+cudaError_t launch_pack_fp32(const Model& M, const Fp32Nets& w, bool both, cudaStream_t s) {
   if (M.model == 1)
-    return M.hidden == 64 ? pack<paper::kObs, 64>(w, f, s) : pack<paper::kObs, 256>(w, f, s);
-  return M.hidden == 64 ? pack<kObs, 64>(w, f, s) : pack<kObs, 256>(w, f, s);
+    return M.hidden == 64 ? pack<paper::kObs, 64>(w, both, s) : pack<paper::kObs, 256>(w, both, s);
+  return M.hidden == 64 ? pack<kObs, 64>(w, both, s) : pack<kObs, 256>(w, both, s);
 }
 
 cudaError_t launch_rollout_fp32(const Model& M, const Buffers& B, const Fp32Nets& w, const Traj& tr,
