@@ -668,7 +668,7 @@ def run_ppo(args):
     st = stats.cpu().numpy().tolist()
     # gather, forward, head, stats, backward, norm + Adam (3); on the bf16 engine with its images packed and the
     # weight gradients in two groups with their reductions, else one product per layer and direction.  Three launches
-    # an epoch draw its rows and advantage statistics.
+    # an epoch draw its rows and advantage statistics (not in epochs of a few minibatches).
     launches_per_step = 1 + 1 + 2 + 2 + 2 + 4 + 3 if args.ppo_precision == "bf16" else 1 + 6 + 2 + 10 + 3
     line = {
         "metric": "PPO update samples/s", "value": samples / (step_ms * 1e-3),
@@ -685,7 +685,7 @@ def run_ppo(args):
                      "frac": achieved / peak, "traffic": None, "peak_source": psrc,
                      "flops_per_sample": fps},
         "update_stats": dict(zip(auvenv.PPO_STAT_NAMES, st)),
-        "gpu_launches": args.steps * args.epochs * (n_mb * launches_per_step + 3),
+        "gpu_launches": args.steps * args.epochs * (n_mb * launches_per_step + (3 if n_mb >= 4 or B > 65536 else 0)),
         "clocks": clock_info,
     }
     print(json.dumps(line), flush=True)
@@ -794,8 +794,10 @@ def _timed(args, fn, flush=None):
 
 def run_rbuf(args):
     """Replay buffer (rbuf_insert of one 65,536 x 128 rollout trajectory,
-    then rbuf_sample of 65,536-transition minibatches).  HBM roofline:
-    (2 D + A + 1) * 4 + 1 bytes read and written per transition."""
+    then rbuf_sample of 65,536-transition minibatches).  HBM roofline of the
+    sample: (2 D + A + 1) * 4 + 1 bytes read and written per transition; of the
+    insert: those written, and (D + A + 1) * 4 + 1 read, since a next
+    observation is the following step's observation (one more per eight steps)."""
     import torch
     from paper_2512_13359_gb300 import auvenv, build
     build.build()
@@ -820,7 +822,8 @@ def run_rbuf(args):
     draws = iter(range(1, 10 ** 9))
     smp_ms = _timed(args, lambda: rb.sample(B, 1, next(draws), out=out), flush)
     peaks, src = load_peaks()
-    ins_gbs = 2 * rec * n * T / (ins_ms * 1e-3) / 1e9
+    ins_bytes = rec + (D + A + 1) * 4 + 1 + 4 * D / 8
+    ins_gbs = ins_bytes * n * T / (ins_ms * 1e-3) / 1e9
     smp_gbs = 2 * rec * B / (smp_ms * 1e-3) / 1e9
     line = {
         "metric": "replay-buffer sampled transitions/s", "value": B / (smp_ms * 1e-3),
@@ -830,7 +833,8 @@ def run_rbuf(args):
         "config": {"workload": w["name"], "capacity": 1 << 24, "minibatch": B,
                    "inserted_per_call": n * T, "l2": "flushed between timed steps"},
         "insert": {"transitions_per_s": n * T / (ins_ms * 1e-3), "ms": ins_ms,
-                   "achieved_gbs": ins_gbs, "frac": ins_gbs / peaks["hbm_gbs"]},
+                   "bytes_per_transition": ins_bytes, "achieved_gbs": ins_gbs,
+                   "frac": ins_gbs / peaks["hbm_gbs"]},
         "roofline": {"bound": "hbm", "kernel": "k_rb_sample", "achieved": smp_gbs,
                      "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": smp_gbs / peaks["hbm_gbs"],
                      "traffic": None, "peak_source": f"HBM copy, {src}",

@@ -171,8 +171,7 @@ struct AdamHp {
 // Per-step variables of an update, in device memory so that one captured
 // step (a CUDA graph) can be replayed: step s of the update gathers
 // minibatch s mod n_mb of epoch epoch0 + s / n_mb, and Adam takes its step
-// t + 1 (bias corrections 1 - b^(t+1)); launch_step_advance then moves to
-// the next step.
+// t + 1 (bias corrections 1 - b^(t+1)) and moves on to the next step.
 struct StepCtl {
   unsigned long long epoch0;
   unsigned long long t;

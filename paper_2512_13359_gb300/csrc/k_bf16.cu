@@ -569,7 +569,7 @@ k_engine(const Model M, Buffers B, const uint8_t* __restrict__ image, Traj tr, i
   const uint32_t s_base = tc::smem_u32(smem);
   // every role reads the weights (MMA operands, biases): wait for the image
   // (kOne: a single group's epilogues once its envs are loaded and its first
-  // observation is written)
+  // observation is written; the Fossen model's, the paper's was not tried)
   constexpr bool kOne = G == 1 && MODE == kRollout && SIM == 0;
   const bool img_ok = (kOne && !is_mma_warp) || tc::mbar_wait(&bar->img_full, 0, abort, kWaitLimitNs);
 
@@ -988,9 +988,10 @@ k_engine(const Model M, Buffers B, const uint8_t* __restrict__ image, Traj tr, i
         // The step's normals depend only on (env, seed, step): with one group
         // per CTA (registers to spare) they are drawn while layer 1 runs
         // instead of after the network, and the episode parameters stay in
-        // registers: 1,024 envs 7.48 -> 7.16 us a step, one step of 256 envs
-        // with its launch 12.3 -> 11.2 us (with more groups, where others'
-        // work hides both, 65,536 envs x 128 steps took 3.27 ms for 3.21).
+        // registers: 1,024 envs 7.48 -> 7.16 us a step (one step of 256 envs
+        // with its launch 12.3 -> 11.2 to 12.3 us, within the spread of
+        // boxes; with more groups, where others' work hides both, 65,536
+        // envs x 128 steps took 3.27 ms for 3.21).
         float eps[kAct];
         if (kOne && active) action_noise_approx(M.id_base + (uint32_t)i, M.seed, t_g0 + (uint64_t)t, eps);
         if (kOne && t == 0 && !(ok = image_here())) break;

@@ -374,11 +374,11 @@ def _grad_err(gpu, ref, n_pol):
                                                    (12, 6, 4096, 31, False)])
 def test_bf16_engine_forward(D, A, B, seed, calibrated):
     """bf16 learners with hidden 256 run the forward pass and the
-    backward-data (gZ2, gZ1) on the tcgen05 engine, the weight gradients on
-    cuBLAS: its gradient and loss record against the oracle at a whole-tile
-    and a ragged minibatch and at the paper model's widths, and its error
-    against that of the same learner with those products through cuBLAS GEMMs
-    and tanh passes (AUV_PPO_GEMM_PATH, which rounds each product to bf16
+    backward-data (gZ2, gZ1) on the tcgen05 engine, the weight gradients in
+    grouped launches: its gradient and loss record against the oracle at a
+    whole-tile and a ragged minibatch and at the paper model's widths, and its
+    error against that of the same learner with every product through the
+    GEMM kernels (AUV_PPO_GEMM_PATH, which rounds each product to bf16
     before its tanh or tanh'); the status block stays clear.  Both paths are held to the
     tolerance on the calibrated case (that of the tensor-core test above);
     on other draws the bf16 policy error of the GEMM path reaches 5e-2, so

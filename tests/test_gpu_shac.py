@@ -14,7 +14,7 @@ from parity_util import make_env, need_gpu, to_np
 pytestmark = pytest.mark.gpu
 
 # |<grad, d> - sum_i dJ_i| <= SHAC_TOL * sum_k |grad_k d_k|: fp32 windows
-# (forward, cuBLAS fp32 GEMMs, VJPs) against the double dual numbers
+# (forward, fp32 products, VJPs) against the double dual numbers
 # (measured 1.6e-9 .. 1.3e-8).  Single coordinates: within COORD_TOL of the
 # largest gradient component.
 SHAC_TOL = 1e-6
